@@ -63,6 +63,11 @@ struct ap_ctx {
     // block-solve work split and partial sums
     float* spart = nullptr;
     unsigned* sticket = nullptr;
+    // column-group sums of the FP32 products: one area for the solve's shapes
+    // (part of the captured graph), one that predictions grow
+    float *gscr = nullptr, *pscr = nullptr;
+    unsigned *gtick = nullptr, *ptick = nullptr;
+    int64_t gscr_alloc = 0, gtick_alloc = 0, pscr_alloc = 0, ptick_alloc = 0;
     int sol_tpc = 1, sol_maxj = 1;
     // always-present device scalars
     double *norms = nullptr, *colnorm = nullptr, *gout = nullptr, *gpart = nullptr;
@@ -131,7 +136,37 @@ int pad_d(int d) {
     return 32;
 }
 
-ap_status dalloc(ap_ctx* ctx, void** p, size_t bytes) {
+void drop_graph(ap_ctx* ctx) {
+    if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
+    ctx->graph = nullptr;
+}
+
+template <class T>
+void dfree(ap_ctx* ctx, T*& p) {
+    if (!p) return;
+    auto it = ctx->sizes.find((void*)p);
+    if (it != ctx->sizes.end()) {
+        ctx->bytes -= it->second;
+        ctx->sizes.erase(it);
+    }
+    cudaFreeAsync((void*)p, ctx->st);
+    p = nullptr;
+}
+
+// Give back the column-group sums (products run without groups then).  False when
+// there is nothing to give.
+bool release_groups(ap_ctx* ctx) {
+    if (!ctx->gscr && !ctx->gtick && !ctx->pscr && !ctx->ptick) return false;
+    drop_graph(ctx);
+    dfree(ctx, ctx->gscr);
+    dfree(ctx, ctx->gtick);
+    dfree(ctx, ctx->pscr);
+    dfree(ctx, ctx->ptick);
+    ctx->gscr_alloc = ctx->gtick_alloc = ctx->pscr_alloc = ctx->ptick_alloc = 0;
+    return true;
+}
+
+ap_status dalloc_once(ap_ctx* ctx, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     if (ctx->o.hbm_budget && ctx->bytes + bytes > ctx->o.hbm_budget) return AP_ERR_NOMEM;
@@ -147,26 +182,16 @@ ap_status dalloc(ap_ctx* ctx, void** p, size_t bytes) {
     return AP_OK;
 }
 
+// Required memory takes precedence over the optional column-group sums.
+ap_status dalloc(ap_ctx* ctx, void** p, size_t bytes) {
+    ap_status s = dalloc_once(ctx, p, bytes);
+    if (s != AP_OK && release_groups(ctx)) s = dalloc_once(ctx, p, bytes);
+    return s;
+}
+
 template <class T>
 ap_status dalloc_t(ap_ctx* ctx, T** p, size_t count) {
     return dalloc(ctx, reinterpret_cast<void**>(p), count * sizeof(T));
-}
-
-template <class T>
-void dfree(ap_ctx* ctx, T*& p) {
-    if (!p) return;
-    auto it = ctx->sizes.find((void*)p);
-    if (it != ctx->sizes.end()) {
-        ctx->bytes -= it->second;
-        ctx->sizes.erase(it);
-    }
-    cudaFreeAsync((void*)p, ctx->st);
-    p = nullptr;
-}
-
-void drop_graph(ap_ctx* ctx) {
-    if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
-    ctx->graph = nullptr;
 }
 
 // Order the context stream after the caller's stream.
@@ -195,14 +220,48 @@ struct Shape {
     int S;
 };
 
-// Row tiling of an AP-step product over the n training rows.
-Shape step_shape(const ap_ctx* ctx, int Cp, int64_t ncols) {
+Shape shape_of(const KmvSplit& sp) {
     Shape sh;
-    sh.rows = kmv_rows_per_cta(ctx->D, Cp);
-    sh.tps = (ctx->b + sh.rows - 1) / sh.rows;
-    sh.ntiles = ctx->m * sh.tps;
-    sh.S = choose_split(sh.ntiles, ncols);
+    sh.rows = sp.rows;
+    sh.tps = sp.tps;
+    sh.ntiles = sp.ntiles;
+    sh.S = sp.S;
     return sh;
+}
+
+// Split of an AP-step product over the n training rows.
+KmvSplit step_split(const ap_ctx* ctx, int Cp, int64_t ncols) {
+    return kmv_split(ctx->D, Cp, ctx->b, ctx->m, ncols);
+}
+
+// Column-group sums for split sp: an area that cannot be had (the HBM budget)
+// leaves the product without groups.  Grown areas start with zero tickets.
+ap_status grow_groups(ap_ctx* ctx, const KmvSplit& sp, float** scr, int64_t* scr_n, unsigned** tick,
+                      int64_t* tick_n) {
+    const int64_t ns = sp.scratch, nt = sp.tickets;
+    if (ns > *scr_n) {
+        dfree(ctx, *scr);
+        *scr_n = 0;
+        if (dalloc_once(ctx, (void**)scr, sizeof(float) * ns) == AP_OK) *scr_n = ns;
+    }
+    if (nt > *tick_n) {
+        dfree(ctx, *tick);
+        *tick_n = 0;
+        if (dalloc_once(ctx, (void**)tick, sizeof(unsigned) * nt) == AP_OK) {
+            AP_CK(cudaMemsetAsync(*tick, 0, sizeof(unsigned) * nt, ctx->st));
+            *tick_n = nt;
+        }
+    }
+    return AP_OK;
+}
+
+// Fill the split's part of the launch parameters from an area that grow_groups
+// sized (or could not).
+void set_split(KmvParams* kp, const KmvSplit& sp, float* scr, int64_t scr_n, unsigned* tick, int64_t tick_n) {
+    kp->rm = sp.rm;
+    kp->G = sp.scratch <= scr_n && sp.tickets <= tick_n ? sp.G : 1;
+    kp->gscr = scr;
+    kp->gtick = tick;
 }
 
 // Row tiling of the compensated recompute (one row per thread).
@@ -397,7 +456,8 @@ ap_status ensure_solve(ap_ctx* ctx, int Cp) {
         AP_TRY(dalloc_t(ctx, &ctx->spart, (size_t)ctx->nt * ctx->sol_maxj * kTile * std::max(Cp, 4)));
         AP_TRY(dalloc_t(ctx, &ctx->sticket, (size_t)ctx->nt));
         AP_CK(cudaMemsetAsync(ctx->sticket, 0, sizeof(unsigned) * ctx->nt, ctx->st));
-        const Shape a = step_shape(ctx, Cp, ctx->b), b = step_shape(ctx, Cp, ctx->n), c = norm_shape(ctx);
+        const KmvSplit a = step_split(ctx, Cp, ctx->b), b = step_split(ctx, Cp, ctx->n);
+        const Shape c = norm_shape(ctx);
         const Shape d = comp_shape(ctx, ctx->n);
         int64_t need = std::max(std::max(a.ntiles * a.S, b.ntiles * b.S), std::max(c.ntiles, d.ntiles * d.S));
         need = std::max(need, ctx->m * ctx->tps128);
@@ -409,6 +469,8 @@ ap_status ensure_solve(ap_ctx* ctx, int Cp) {
         AP_TRY(dalloc_t(ctx, &ctx->part_norm, (size_t)need));
         AP_TRY(dalloc_t(ctx, &ctx->part_col, (size_t)need * Cp));
         ctx->part_alloc = need;
+        for (const KmvSplit& sp : {a, b})
+            AP_TRY(grow_groups(ctx, sp, &ctx->gscr, &ctx->gscr_alloc, &ctx->gtick, &ctx->gtick_alloc));
         ctx->Cp = Cp;
     }
     return AP_OK;
@@ -484,8 +546,10 @@ ap_status launch_step(ap_ctx* ctx, bool colnorms, int64_t j) {
         if (prof) AP_CK(cudaEventRecordWithFlags(ctx->ev_up[2 * j + 1], ctx->st, rec_flags));
         return AP_OK;
     }
-    const Shape sh = step_shape(ctx, Cp, ctx->b);
+    const KmvSplit split = step_split(ctx, Cp, ctx->b);
+    const Shape sh = shape_of(split);
     KmvParams kp = {};
+    set_split(&kp, split, ctx->gscr, ctx->gscr_alloc, ctx->gtick, ctx->gtick_alloc);
     kp.Xa = ctx->Xs;
     kp.na = ctx->n;
     kp.Xb = ctx->Xs;
@@ -526,8 +590,10 @@ ap_status launch_full_residual(ap_ctx* ctx, const float* base, const float* V, f
     PhaseRange range("ap: residual recompute R = B - K_hat W");
     const bool comp = use_compensated(ctx);
     ctx->comp_used = comp;
-    const Shape sh = comp ? comp_shape(ctx, ctx->n) : step_shape(ctx, ctx->Cp, ctx->n);
+    const KmvSplit split = step_split(ctx, ctx->Cp, ctx->n);
+    const Shape sh = comp ? comp_shape(ctx, ctx->n) : shape_of(split);
     KmvParams kp = {};
+    if (!comp) set_split(&kp, split, ctx->gscr, ctx->gscr_alloc, ctx->gtick, ctx->gtick_alloc);
     kp.Xa = ctx->Xs;
     kp.na = ctx->n;
     kp.Xb = ctx->Xs;
@@ -1185,13 +1251,11 @@ ap_status ap_predict_mean(ap_ctx* ctx, const float* w_dev, const float* Xs_dev, 
     AP_TRY(enter(ctx));
     AP_CK(cudaMemsetAsync(ctx->nan_flag, 0, sizeof(int), ctx->st));
     AP_TRY(prep_inputs(ctx, Xs_dev, M, ctx->Xt, nullptr));
-    const int64_t rows = kmv_rows_per_cta(ctx->D, 1);
-    Shape sh;
-    sh.rows = rows;
-    sh.tps = (M + rows - 1) / rows;
-    sh.ntiles = sh.tps;
-    sh.S = choose_split(sh.ntiles, ctx->n);
+    const KmvSplit split = kmv_split(ctx->D, 1, M, 1, ctx->n);
+    AP_TRY(grow_groups(ctx, split, &ctx->pscr, &ctx->pscr_alloc, &ctx->ptick, &ctx->ptick_alloc));
+    const Shape sh = shape_of(split);
     KmvParams kp = {};
+    set_split(&kp, split, ctx->pscr, ctx->pscr_alloc, ctx->ptick, ctx->ptick_alloc);
     kp.Xa = ctx->Xt;
     kp.na = M;
     kp.Xb = ctx->Xs;

@@ -91,8 +91,23 @@ struct KmvParams {
     int64_t blk;
     const float* Xa_lo;    // compensated form only: low parts of the scaled inputs
     const float* Xb_lo;
+    int rm;                // rows per thread (KmvSplit)
+    int G;                 // column groups per row tile on top of the cluster's S splits (KmvSplit)
+    float* gscr;           // G > 1: partial sums (KmvSplit::scratch floats)
+    unsigned int* gtick;   // G > 1: arrival tickets (KmvSplit::tickets), zero between launches
     EpiParams epi;
 };
+
+// How one FP32 product is cut into CTAs: row tiles of 128 * rm rows (never across a
+// segment), S column splits per tile summed inside a cluster, G groups of S splits
+// summed through global memory by the last group to arrive.
+struct KmvSplit {
+    int rm, S, G;
+    int64_t rows, tps, ntiles;
+    int64_t scratch;  // floats of partial sums when G > 1
+    int64_t tickets;  // arrival tickets when G > 1
+};
+KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols);
 
 // FP32 SIMT kernel-matrix product with the AP epilogue (one per kernel family TU).
 cudaError_t launch_kmv_rbf(const KmvParams& p, int D, int C, cudaStream_t st);
@@ -105,9 +120,6 @@ cudaError_t launch_kmv_comp_m32(const KmvParams& p, int D, int C, cudaStream_t s
 cudaError_t launch_kmv_comp_m52(const KmvParams& p, int D, int C, cudaStream_t st);
 cudaError_t launch_kmv_comp(int kernel, const KmvParams& p, int D, int C, cudaStream_t st);
 constexpr int kCompRows = 128;  // rows per CTA of the compensated product
-
-// Rows per CTA for a (D, C) instance of the FP32 product.
-int kmv_rows_per_cta(int D, int C);
 
 // Norms of R alone (n x C) + selection: used before the first step and after refinement.
 cudaError_t launch_norms_select(const float* R, int64_t n, int C, const EpiParams& e,

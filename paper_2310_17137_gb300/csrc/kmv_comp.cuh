@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kKmvThreads) kmv_comp_kernel(const KmvParams p
         }
     }
     if (S > 1) cg::this_cluster().sync();
-    epi_ticket<C>(e, red_d, red_i, &s_last);
+    epi_ticket<C>(e, red_d, red_i, &s_last, s_col);
 }
 
 template <int KERN, int D, int C>

@@ -8,7 +8,11 @@
 //            block, so its squared norm belongs to exactly one block;
 //   grid.y = S column splits, one thread-block cluster per row tile; the S
 //            partial products are summed through distributed shared memory in
-//            a fixed rank order (deterministic, no atomics on R).
+//            a fixed rank order (deterministic, no atomics on R);
+//   grid.z = G groups of S column splits when the row tiles are too few to fill
+//            the chip or its last wave: each cluster leaves its sums in global
+//            memory, and the group that arrives last at the tile's ticket adds
+//            them in group order (kmv_split chooses rm, S and G).
 // Each thread keeps RM rows of the scaled inputs and RM x C accumulators in
 // registers; the block's columns (scaled inputs and the C right-hand sides of
 // Delta) are staged through shared memory and read as warp broadcasts.  The
@@ -80,21 +84,39 @@ __device__ __forceinline__ double cta_sum_d(double v, double* red) {
 // Executed by every thread of the CTA that finished last (ticket order):
 // reduce the per-tile partials in a fixed order, pick the next block, publish
 // the column norms, and leave the ticket at zero for the next launch.
+//
+// This runs alone on the chip at the end of every step, so it is bound by the
+// latency of its loads: the partials of a block (and of a column) are shared out
+// over as many threads as the CTA has for it.  With one thread per block and per
+// column, the last step of an epoch of a 4096-row solve spent some 20 us in the
+// column sums alone.  s_buf: 16 C doubles when the CTA has more than 128 threads,
+// 128 otherwise.
 template <int C>
-__device__ void epi_finalize(const EpiParams& e, double* red_d, int* red_i) {
+__device__ void epi_finalize(const EpiParams& e, double* red_d, int* red_i, double* s_buf) {
     const int tid = threadIdx.x, nth = blockDim.x;
     if (e.flags & kEpiBlockNorms) {
         double best = -1.0;
         int bi = 0x7fffffff;
         int bad = 0;
         const int64_t per = e.tiles_per_seg * e.S;
-        for (int J = tid; J < e.m; J += nth) {
+        // L consecutive lanes per block; whole warps go round together
+        int L = 1;
+        while (L < 32 && 2 * L * e.m <= nth) L *= 2;
+        const int lane = tid % L, stride = nth / L;
+        for (int J0 = 0; J0 < e.m; J0 += stride) {
+            const int J = J0 + tid / L;
             double acc = 0.0;
-            const double* src = e.part_norm + (int64_t)J * per;
-            for (int64_t t = 0; t < per && AP_CHK((int64_t)J * per + t < e.ntiles * e.S); ++t) acc += __ldcg(src + t);
-            e.norms_out[J] = acc;
-            if (!isfinite(acc)) bad = 1;
-            if (acc > best) { best = acc; bi = J; }
+            if (J < e.m && tid / L < stride) {
+                const double* src = e.part_norm + (int64_t)J * per;
+#pragma unroll 8
+                for (int64_t t = lane; t < per; t += L) acc += __ldcg(src + t);
+            }
+            for (int o = L / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (J < e.m && tid / L < stride && AP_CHK((int64_t)(J + 1) * per <= e.ntiles * e.S)) {
+                if (lane == 0) e.norms_out[J] = acc;
+                if (!isfinite(acc)) bad = 1;
+                if (acc > best) { best = acc; bi = J; }
+            }
         }
         // argmax over the CTA, ties to the smallest block index
         for (int o = 16; o > 0; o >>= 1) {
@@ -123,11 +145,22 @@ __device__ void epi_finalize(const EpiParams& e, double* red_d, int* red_i) {
         __syncthreads();
     }
     if (e.flags & kEpiColNorms) {
+        // thread t sums column t % C over the tiles t / C, t / C + groups, ...
         const int64_t tot = e.ntiles * e.S;
-        for (int c = tid; c < C; c += nth) {
-            double acc = 0.0;
-            for (int64_t t = 0; t < tot; ++t) acc += __ldcg(e.part_col + t * C + c);
-            e.colnorm_out[c] = acc;
+        const int nwu = min(nth >> 5, 16), nthu = 32 * nwu;
+        double acc = 0.0;
+        if (tid < nthu) {
+#pragma unroll 8
+            for (int64_t t = tid / C; t < tot; t += nthu / C) acc += __ldcg(e.part_col + t * C + tid % C);
+        }
+        for (int o = 16; o >= C; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        __syncthreads();
+        if (tid < nthu && (tid & 31) < C) s_buf[(tid >> 5) * C + (tid & 31)] = acc;
+        __syncthreads();
+        if (tid < C) {
+            acc = 0.0;
+            for (int w = 0; w < nwu; ++w) acc += s_buf[w * C + tid];
+            e.colnorm_out[tid] = acc;
             if (!isfinite(acc)) *e.nan_flag = 1;
         }
     }
@@ -136,26 +169,51 @@ __device__ void epi_finalize(const EpiParams& e, double* red_d, int* red_i) {
 
 // Phase 2 of every product: reduce the S rank partials of this CTA's share of
 // rows (fixed rank order), add the base, store, and write the norm partials.
+// With G > 1 column groups the sums go to the tile's slots first, and only the
+// group that arrives last (returns true) goes on with the slots' sums, added in
+// group order.
 template <int C, int ROWS>
-__device__ __forceinline__ void epi_store(const KmvParams& p, float* s_part, int S, int rank,
+__device__ __forceinline__ bool epi_store(const KmvParams& p, float* s_part, int S, int rank,
                                           int64_t r0, int64_t r1, int64_t part_idx, double* red_d,
-                                          double* s_col) {
+                                          double* s_col, int* s_last) {
     const int tid = threadIdx.x;
     const int rpr = ROWS / S;  // rows reduced by this rank
+    const int G = gridDim.z;
     double sq = 0.0, colacc = 0.0;
+    auto cluster_sum = [&](int t) {
+        const int lc = (rank * rpr + t / C) * C + t % C;
+        if (S == 1) return s_part[lc];
+        cg::cluster_group cluster = cg::this_cluster();
+        float sum = 0.0f;
+        for (int src = 0; src < S; ++src) sum += cluster.map_shared_rank(s_part, src)[lc];
+        return sum;
+    };
+    // slot of group g: this rank's rpr x C sums of the tile
+    float* slots = G > 1 ? p.gscr + (int64_t)blockIdx.x * G * ROWS * C + (int64_t)rank * rpr * C : nullptr;
+    if (G > 1) {
+        for (int t = tid; t < rpr * C; t += kKmvThreads)
+            __stcg(slots + (int64_t)blockIdx.z * ROWS * C + t, cluster_sum(t));
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            unsigned int* tick = p.gtick + (int64_t)blockIdx.x * S + rank;
+            *s_last = atomicAdd(tick, 1u) == (unsigned)(G - 1) ? 1 : 0;
+            if (*s_last) *tick = 0u;
+        }
+        __syncthreads();
+        if (!*s_last) return false;
+        __threadfence();
+    }
     for (int t = tid; t < rpr * C; t += kKmvThreads) {
         const int lr = rank * rpr + t / C;
         const int c = t % C;  // == tid % C since kKmvThreads % C == 0
         const int64_t i = r0 + lr;
         float sum = 0.0f;
-        if (S == 1) {
-            sum = s_part[lr * C + c];
+        if (G > 1) {
+#pragma unroll 8
+            for (int g = 0; g < G; ++g) sum += __ldcg(slots + (int64_t)g * ROWS * C + t);
         } else {
-            cg::cluster_group cluster = cg::this_cluster();
-            for (int src = 0; src < S; ++src) {
-                const float* peer = cluster.map_shared_rank(s_part, src);
-                sum += peer[lr * C + c];
-            }
+            sum = cluster_sum(t);
         }
         if (i < r1 && AP_CHK(i < p.na)) {
             const float bv = p.base ? p.base[i * C + c] : p.base_const;
@@ -181,11 +239,12 @@ __device__ __forceinline__ void epi_store(const KmvParams& p, float* s_part, int
             if (AP_CHK(part_idx < e.ntiles * e.S)) e.part_col[part_idx * C + tid] = acc;
         }
     }
+    return true;
 }
 
 template <int C>
 __device__ __forceinline__ void epi_ticket(const EpiParams& e, double* red_d, int* red_i,
-                                           int* s_last) {
+                                           int* s_last, double* s_buf) {
     if (e.flags == 0) return;
     __threadfence();
     __syncthreads();
@@ -196,20 +255,16 @@ __device__ __forceinline__ void epi_ticket(const EpiParams& e, double* red_d, in
     __syncthreads();
     if (*s_last) {
         __threadfence();
-        epi_finalize<C>(e, red_d, red_i);
+        epi_finalize<C>(e, red_d, red_i, s_buf);
     }
 }
 
-// With C a multiple of 4 the distance and the contraction run as packed FP32
-// pairs (fma.rn.f32x2: one instruction for two lanes, each rounded as the scalar
+// The distance and (for C > 1) the contraction run as packed FP32 pairs
+// (fma.rn.f32x2: one instruction for two lanes, each rounded as the scalar
 // operation): the squared distance over pairs of coordinates (two partial sums,
-// added at the end), the contraction over pairs of right-hand sides.  Shared
-// memory holds the operands exactly as in the scalar form.
-template <int C>
-struct KmvPaired {
-    static constexpr bool value = C % 4 == 0;
-};
-
+// added at the end), the contraction over pairs of right-hand sides.  The FMA pipe
+// does the same work either way; the issue slots saved are what the SFU and
+// shared-memory instructions need.
 template <int D, int C, int RM>
 constexpr size_t kmv_smem_floats() {
     return (size_t)kKmvTN * (D + C) + (size_t)kKmvThreads * RM * C;
@@ -218,7 +273,6 @@ constexpr size_t kmv_smem_floats() {
 template <int KERN, int D, int C, int RM>
 __global__ void __launch_bounds__(kKmvThreads, 4) kmv_fp32_kernel(const KmvParams p) {
     constexpr int ROWS = kKmvThreads * RM;
-    constexpr bool kPaired = KmvPaired<C>::value;
     extern __shared__ float4 kmv_smem4[];
     float* s_xb = reinterpret_cast<float*>(kmv_smem4);  // kKmvTN * D
     float* s_v = s_xb + kKmvTN * D;                     // kKmvTN * C
@@ -244,8 +298,9 @@ __global__ void __launch_bounds__(kKmvThreads, 4) kmv_fp32_kernel(const KmvParam
         col0 = (int64_t)(*p.sel) * p.blk;
         ncols = min(p.blk, p.nb - col0);
     }
-    const int64_t cs = ((ncols + S - 1) / S + kKmvTN - 1) / kKmvTN * kKmvTN;
-    const int64_t c_lo = col0 + rank * cs;
+    const int nsplit = S * gridDim.z, split = (int)blockIdx.z * S + rank;
+    const int64_t cs = ((ncols + nsplit - 1) / nsplit + 15) / 16 * 16;
+    const int64_t c_lo = col0 + split * cs;
     const int64_t c_hi = min(col0 + ncols, c_lo + cs);
 
     float xa[RM][D];
@@ -262,74 +317,15 @@ __global__ void __launch_bounds__(kKmvThreads, 4) kmv_fp32_kernel(const KmvParam
             xa[q][4 * k4 + 3] = v.w;
         }
     }
-    float acc[RM][C];
+    float2 xa2[RM][D / 2], acc2[RM][(C + 1) / 2];
 #pragma unroll
-    for (int q = 0; q < RM; ++q)
+    for (int q = 0; q < RM; ++q) {
 #pragma unroll
-        for (int c = 0; c < C; ++c) acc[q][c] = 0.0f;
-
-    if constexpr (kPaired) {
-        float2 xa2[RM][D / 2], acc2[RM][C / 2];
+        for (int k = 0; k < D / 2; ++k) xa2[q][k] = make_float2(xa[q][2 * k], xa[q][2 * k + 1]);
 #pragma unroll
-        for (int q = 0; q < RM; ++q) {
-#pragma unroll
-            for (int k = 0; k < D / 2; ++k) xa2[q][k] = make_float2(xa[q][2 * k], xa[q][2 * k + 1]);
-#pragma unroll
-            for (int c = 0; c < C / 2; ++c) acc2[q][c] = make_float2(0.0f, 0.0f);
-        }
-        const float2 m1 = make_float2(-1.0f, -1.0f);
-        for (int64_t cb = c_lo; cb < c_hi; cb += kKmvTN) {
-            const int cnt = (int)min((int64_t)kKmvTN, c_hi - cb);
-            __syncthreads();
-            if (AP_CHK(cb >= 0 && cb + cnt <= p.nb) && AP_CHK(cb - col0 >= 0 && cb - col0 + cnt <= ncols)) {
-                const float4* gx = reinterpret_cast<const float4*>(p.Xb + cb * D);
-                float4* sx = reinterpret_cast<float4*>(s_xb);
-                for (int t = tid; t < cnt * D / 4; t += kKmvThreads) sx[t] = __ldg(gx + t);
-                const float4* gv4 = reinterpret_cast<const float4*>(p.V + (cb - col0) * C);
-                float4* sv4 = reinterpret_cast<float4*>(s_v);
-                for (int t = tid; t < cnt * C / 4; t += kKmvThreads) sv4[t] = __ldg(gv4 + t);
-            }
-            __syncthreads();
-#pragma unroll 2
-            for (int jj = 0; jj < cnt; ++jj) {
-                float2 xb2[D / 2];
-#pragma unroll
-                for (int k4 = 0; k4 < D / 4; ++k4) {
-                    const float4 v = reinterpret_cast<const float4*>(s_xb + jj * D)[k4];
-                    xb2[2 * k4] = make_float2(v.x, v.y);
-                    xb2[2 * k4 + 1] = make_float2(v.z, v.w);
-                }
-                float kv[RM];
-#pragma unroll
-                for (int q = 0; q < RM; ++q) {
-                    float2 tp = make_float2(0.0f, 0.0f);
-#pragma unroll
-                    for (int k = 0; k < D / 2; ++k) {
-                        const float2 df = __ffma2_rn(xb2[k], m1, xa2[q][k]);  // xa - xb, exact negation
-                        tp = __ffma2_rn(df, df, tp);
-                    }
-                    kv[q] = phi_fp32<KERN>(tp.x + tp.y);
-                }
-#pragma unroll
-                for (int c4 = 0; c4 < C / 4; ++c4) {
-                    const float4 v = reinterpret_cast<const float4*>(s_v + jj * C)[c4];
-#pragma unroll
-                    for (int q = 0; q < RM; ++q) {
-                        const float2 kd = make_float2(kv[q], kv[q]);
-                        acc2[q][2 * c4] = __ffma2_rn(kd, make_float2(v.x, v.y), acc2[q][2 * c4]);
-                        acc2[q][2 * c4 + 1] = __ffma2_rn(kd, make_float2(v.z, v.w), acc2[q][2 * c4 + 1]);
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < RM; ++q)
-#pragma unroll
-            for (int c = 0; c < C / 2; ++c) {
-                acc[q][2 * c] = acc2[q][c].x;
-                acc[q][2 * c + 1] = acc2[q][c].y;
-            }
-    } else
+        for (int c = 0; c < (C + 1) / 2; ++c) acc2[q][c] = make_float2(0.0f, 0.0f);
+    }
+    const float2 m1 = make_float2(-1.0f, -1.0f);
     for (int64_t cb = c_lo; cb < c_hi; cb += kKmvTN) {
         const int cnt = (int)min((int64_t)kKmvTN, c_hi - cb);
         __syncthreads();
@@ -349,25 +345,23 @@ __global__ void __launch_bounds__(kKmvThreads, 4) kmv_fp32_kernel(const KmvParam
         __syncthreads();
 #pragma unroll 2
         for (int jj = 0; jj < cnt; ++jj) {
-            float xb[D];
+            float2 xb2[D / 2];
 #pragma unroll
             for (int k4 = 0; k4 < D / 4; ++k4) {
-                float4 v = reinterpret_cast<const float4*>(s_xb + jj * D)[k4];
-                xb[4 * k4 + 0] = v.x;
-                xb[4 * k4 + 1] = v.y;
-                xb[4 * k4 + 2] = v.z;
-                xb[4 * k4 + 3] = v.w;
+                const float4 v = reinterpret_cast<const float4*>(s_xb + jj * D)[k4];
+                xb2[2 * k4] = make_float2(v.x, v.y);
+                xb2[2 * k4 + 1] = make_float2(v.z, v.w);
             }
             float kv[RM];
 #pragma unroll
             for (int q = 0; q < RM; ++q) {
-                float t2 = 0.0f;
+                float2 tp = make_float2(0.0f, 0.0f);
 #pragma unroll
-                for (int k = 0; k < D; ++k) {
-                    const float df = xa[q][k] - xb[k];
-                    t2 = fmaf(df, df, t2);
+                for (int k = 0; k < D / 2; ++k) {
+                    const float2 df = __ffma2_rn(xb2[k], m1, xa2[q][k]);  // xa - xb, exact negation
+                    tp = __ffma2_rn(df, df, tp);
                 }
-                kv[q] = phi_fp32<KERN>(t2);
+                kv[q] = phi_fp32<KERN>(tp.x + tp.y);
             }
             if constexpr (C % 4 == 0) {
 #pragma unroll
@@ -375,22 +369,24 @@ __global__ void __launch_bounds__(kKmvThreads, 4) kmv_fp32_kernel(const KmvParam
                     const float4 v = reinterpret_cast<const float4*>(s_v + jj * C)[c4];
 #pragma unroll
                     for (int q = 0; q < RM; ++q) {
-                        acc[q][4 * c4 + 0] = fmaf(kv[q], v.x, acc[q][4 * c4 + 0]);
-                        acc[q][4 * c4 + 1] = fmaf(kv[q], v.y, acc[q][4 * c4 + 1]);
-                        acc[q][4 * c4 + 2] = fmaf(kv[q], v.z, acc[q][4 * c4 + 2]);
-                        acc[q][4 * c4 + 3] = fmaf(kv[q], v.w, acc[q][4 * c4 + 3]);
+                        const float2 kd = make_float2(kv[q], kv[q]);
+                        acc2[q][2 * c4] = __ffma2_rn(kd, make_float2(v.x, v.y), acc2[q][2 * c4]);
+                        acc2[q][2 * c4 + 1] = __ffma2_rn(kd, make_float2(v.z, v.w), acc2[q][2 * c4 + 1]);
                     }
                 }
             } else {
+                static_assert(C % 4 == 0 || C == 1, "one right-hand side, or quads of them");
+                const float v = s_v[jj];
 #pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    const float v = s_v[jj * C + c];
-#pragma unroll
-                    for (int q = 0; q < RM; ++q) acc[q][c] = fmaf(kv[q], v, acc[q][c]);
-                }
+                for (int q = 0; q < RM; ++q) acc2[q][0].x = fmaf(kv[q], v, acc2[q][0].x);
             }
         }
     }
+    float acc[RM][C];
+#pragma unroll
+    for (int q = 0; q < RM; ++q)
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[q][c] = c % 2 ? acc2[q][c / 2].y : acc2[q][c / 2].x;
     // scale by s, add sigma^2 V_i on the index diagonal, park in shared memory
     __syncthreads();
 #pragma unroll
@@ -407,9 +403,9 @@ __global__ void __launch_bounds__(kKmvThreads, 4) kmv_fp32_kernel(const KmvParam
     }
     if (S > 1) cg::this_cluster().sync();
     else __syncthreads();
-    epi_store<C, ROWS>(p, s_part, S, rank, r0, r1, tile * S + rank, red_d, s_col);
+    const bool done = epi_store<C, ROWS>(p, s_part, S, rank, r0, r1, tile * S + rank, red_d, s_col, &s_last);
     if (S > 1) cg::this_cluster().sync();
-    epi_ticket<C>(e, red_d, red_i, &s_last);
+    if (done) epi_ticket<C>(e, red_d, red_i, &s_last, s_col);
 }
 
 // Norms + selection of R alone (before the first step, after a refinement).
@@ -447,7 +443,7 @@ __global__ void __launch_bounds__(kKmvThreads) norms_select_kernel(const float* 
             if (AP_CHK(tile < e.ntiles)) e.part_col[tile * C + tid] = acc;
         }
     }
-    epi_ticket<C>(e, red_d, red_i, &s_last);
+    epi_ticket<C>(e, red_d, red_i, &s_last, s_col);
 }
 
 inline int rows_per_thread(int D, int C) {
@@ -455,16 +451,15 @@ inline int rows_per_thread(int D, int C) {
     return w <= 20 ? 4 : (w <= 36 ? 2 : 1);
 }
 
-template <int KERN, int D, int C>
-cudaError_t launch_kmv_inst(const KmvParams& p, cudaStream_t st) {
-    constexpr int RM = (D + C <= 20) ? 4 : ((D + C <= 36) ? 2 : 1);
+template <int KERN, int D, int C, int RM>
+cudaError_t launch_kmv_rm(const KmvParams& p, cudaStream_t st) {
     const size_t smem = sizeof(float) * kmv_smem_floats<D, C, RM>();
     auto fn = kmv_fp32_kernel<KERN, D, C, RM>;
     cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const int S = p.epi.S;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)p.epi.ntiles, (unsigned)S, 1);
+    cfg.gridDim = dim3((unsigned)p.epi.ntiles, (unsigned)S, (unsigned)p.G);
     cfg.blockDim = dim3(kKmvThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -478,6 +473,17 @@ cudaError_t launch_kmv_inst(const KmvParams& p, cudaStream_t st) {
         cfg.numAttrs = 1;
     }
     return cudaLaunchKernelEx(&cfg, fn, p);
+}
+
+// rows per thread as kmv_split chose them, at most what (D, C) leaves registers for
+template <int KERN, int D, int C>
+cudaError_t launch_kmv_inst(const KmvParams& p, cudaStream_t st) {
+    constexpr int kMaxRm = (D + C <= 20) ? 4 : ((D + C <= 36) ? 2 : 1);
+    if constexpr (kMaxRm >= 4)
+        if (p.rm == 4) return launch_kmv_rm<KERN, D, C, 4>(p, st);
+    if constexpr (kMaxRm >= 2)
+        if (p.rm == 2) return launch_kmv_rm<KERN, D, C, 2>(p, st);
+    return p.rm == 1 ? launch_kmv_rm<KERN, D, C, 1>(p, st) : cudaErrorInvalidValue;
 }
 
 // (D, C) dispatch for one kernel family.

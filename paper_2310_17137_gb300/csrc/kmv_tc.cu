@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(tc::kThreads, 1) kmv_tc_kernel(const TcParams 
     __syncthreads();
     if (s_last) {
         __threadfence();
-        epi_finalize<C>(e, red_d, red_i);
+        epi_finalize<C>(e, red_d, red_i, &s_colred[0][0][0]);
     }
 }
 

@@ -2,6 +2,8 @@
 // the kernel-family dispatch of the FP32 product.
 #include <math.h>
 
+#include <algorithm>
+
 #include "kmv_fp32.cuh"
 
 namespace ap {
@@ -12,7 +14,54 @@ double kernel_input_scale(int kernel) {
     return sqrt(5.0);
 }
 
-int kmv_rows_per_cta(int D, int C) { return kKmvThreads * rows_per_thread(D, C); }
+// The split of one product of `nseg` segments of `seg` rows with `ncols` columns.
+//
+// Rows per thread: more rows share each staged column (the shared-memory reads per
+// entry fall as 1 / rm), but a tile of 128 rm rows may be mostly padding (a segment of
+// 600 rows is 60 % of two 512-row tiles) and leaves fewer tiles.  The modelled issue
+// slots per useful entry, times the shortfall of CTAs when the whole product cannot
+// give two per SM, decide.
+//
+// Columns: S splits inside a cluster until 4 CTAs per SM exist, then G groups through
+// global memory: enough of them for about 8 waves of CTAs while every CTA keeps at
+// least 512 columns and 64 per right-hand side (a last wave that is nearly empty costs
+// at most an eighth; shorter ranges measured slower, 11.9 -> 12.3 ms on 16 steps of
+// n = 65,536, b = 4096, c = 32), and for 8 CTAs per SM with at least 64 columns when the
+// clusters alone leave places free.  Measured on GB300: n = 100,003, d = 11, 1024 test
+// points, 16 CTAs (cluster only) 1102 us per ap_predict_mean call, with the groups
+// 135 us; n = 20,600, d = 8, one column, ap_residual 500 -> 377 us.
+KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
+    constexpr int64_t kSms = 152, kMaxScratch = (int64_t)8 << 20;
+    KmvSplit best = {};
+    double best_cost = 0.0;
+    for (int rm = rows_per_thread(D, C); rm >= 1; rm /= 2) {
+        KmvSplit sp = {};
+        sp.rm = rm;
+        sp.rows = (int64_t)kKmvThreads * rm;
+        sp.tps = (seg + sp.rows - 1) / sp.rows;
+        sp.ntiles = nseg * sp.tps;
+        const double pad = (double)(sp.tps * sp.rows) / (double)seg;
+        const double ctas = (double)sp.ntiles * (double)((ncols + kKmvTN - 1) / kKmvTN);
+        const double idle = ctas < 2.0 * kSms ? 2.0 * kSms / ctas : 1.0;
+        const double cost = pad * idle * ((D + C + 8) + (D + C) / (4.0 * rm));
+        if (!best.rm || cost < best_cost) best = sp, best_cost = cost;
+    }
+    best.S = 1;
+    while (best.S < kMaxSplit && best.ntiles * best.S < 4 * kSms && ncols / (2 * best.S) >= kKmvTN) best.S *= 2;
+    const int64_t ctas = best.ntiles * best.S;
+    auto groups = [&](int64_t want, int64_t min_cols) {
+        return std::min<int64_t>((want + ctas - 1) / ctas, ncols / (best.S * min_cols));
+    };
+    int64_t G = groups(64 * kSms, std::max(512, 64 * C));
+    if (ctas < 4 * kSms) G = std::max(G, groups(8 * kSms, kKmvTN));
+    G = std::min<int64_t>(G, kMaxScratch / (best.ntiles * best.rows * C));
+    best.G = (int)std::max<int64_t>(1, std::min<int64_t>(G, 1024));
+    if (best.G > 1) {
+        best.scratch = best.ntiles * best.G * best.rows * C;
+        best.tickets = best.ntiles * best.S;
+    }
+    return best;
+}
 
 cudaError_t launch_kmv(int kernel, const KmvParams& p, int D, int C, cudaStream_t st) {
     switch (kernel) {
