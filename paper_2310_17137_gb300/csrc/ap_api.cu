@@ -260,6 +260,7 @@ ap_status grow_groups(ap_ctx* ctx, const KmvSplit& sp, float** scr, int64_t* scr
 void set_split(KmvParams* kp, const KmvSplit& sp, float* scr, int64_t scr_n, unsigned* tick, int64_t tick_n) {
     kp->rm = sp.rm;
     kp->G = sp.scratch <= scr_n && sp.tickets <= tick_n ? sp.G : 1;
+    kp->ctas = kp->G > 1 ? sp.ctas : (int)std::min<int64_t>(sp.ctas, sp.ntiles);
     kp->gscr = scr;
     kp->gtick = tick;
 }
@@ -457,10 +458,11 @@ ap_status ensure_solve(ap_ctx* ctx, int Cp) {
         AP_TRY(dalloc_t(ctx, &ctx->sticket, (size_t)ctx->nt));
         AP_CK(cudaMemsetAsync(ctx->sticket, 0, sizeof(unsigned) * ctx->nt, ctx->st));
         const KmvSplit a = step_split(ctx, Cp, ctx->b), b = step_split(ctx, Cp, ctx->n);
+        const KmvSplit whole = kmv_split(ctx->D, Cp, ctx->n, 1, ctx->n);
         const Shape c = norm_shape(ctx);
         const Shape d = comp_shape(ctx, ctx->n);
         int64_t need = std::max(std::max(a.ntiles * a.S, b.ntiles * b.S), std::max(c.ntiles, d.ntiles * d.S));
-        need = std::max(need, ctx->m * ctx->tps128);
+        need = std::max(std::max(need, whole.ntiles * whole.S), ctx->m * ctx->tps128);
         if (ctx->tc) {
             dfree(ctx, ctx->DT);
             AP_TRY(dalloc_t(ctx, &ctx->DT, tc_delta_bytes(ctx->cpb, Cp)));
@@ -469,7 +471,7 @@ ap_status ensure_solve(ap_ctx* ctx, int Cp) {
         AP_TRY(dalloc_t(ctx, &ctx->part_norm, (size_t)need));
         AP_TRY(dalloc_t(ctx, &ctx->part_col, (size_t)need * Cp));
         ctx->part_alloc = need;
-        for (const KmvSplit& sp : {a, b})
+        for (const KmvSplit& sp : {a, b, whole})
             AP_TRY(grow_groups(ctx, sp, &ctx->gscr, &ctx->gscr_alloc, &ctx->gtick, &ctx->gtick_alloc));
         ctx->Cp = Cp;
     }
@@ -563,6 +565,7 @@ ap_status launch_step(ap_ctx* ctx, bool colnorms, int64_t j) {
     kp.noise_diag = 1;
     kp.sel = ctx->sel;
     kp.blk = ctx->b;
+    kp.err = ctx->tc_err;
     kp.epi = make_epi(ctx, kEpiBlockNorms | (colnorms ? kEpiColNorms : 0), 1, sh);
     AP_CK(launch_kmv(ctx->kernel, kp, ctx->D, Cp, ctx->st));
     ++ctx->launches;
@@ -585,12 +588,24 @@ void collect_profile(ap_ctx* ctx, int64_t steps) {
     cudaGetLastError();
 }
 
+// Clear the timeout flag and the arrival tickets (a launch that gave up on a wait
+// leaves them partial).
+ap_status reset_waits(ap_ctx* ctx) {
+    AP_CK(cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->st));
+    AP_CK(cudaMemsetAsync(ctx->ticket, 0, 4 * sizeof(unsigned), ctx->st));
+    if (ctx->gtick) AP_CK(cudaMemsetAsync(ctx->gtick, 0, sizeof(unsigned) * ctx->gtick_alloc, ctx->st));
+    if (ctx->tc_tick) AP_CK(cudaMemsetAsync(ctx->tc_tick, 0, sizeof(int) * ctx->num_sms, ctx->st));
+    return AP_OK;
+}
+
 // out = base - K_hat V over all n columns (the FP32 residual recompute).
 ap_status launch_full_residual(ap_ctx* ctx, const float* base, const float* V, float* out, int flags) {
     PhaseRange range("ap: residual recompute R = B - K_hat W");
     const bool comp = use_compensated(ctx);
     ctx->comp_used = comp;
-    const KmvSplit split = step_split(ctx, ctx->Cp, ctx->n);
+    // without block norms the row tiles need not respect the blocks
+    const bool blocks = comp || (flags & kEpiBlockNorms);
+    const KmvSplit split = blocks ? step_split(ctx, ctx->Cp, ctx->n) : kmv_split(ctx->D, ctx->Cp, ctx->n, 1, ctx->n);
     const Shape sh = comp ? comp_shape(ctx, ctx->n) : shape_of(split);
     KmvParams kp = {};
     if (!comp) set_split(&kp, split, ctx->gscr, ctx->gscr_alloc, ctx->gtick, ctx->gtick_alloc);
@@ -609,7 +624,9 @@ ap_status launch_full_residual(ap_ctx* ctx, const float* base, const float* V, f
     kp.ncols = ctx->n;
     kp.Xa_lo = ctx->Xs_lo;
     kp.Xb_lo = ctx->Xs_lo;
+    kp.err = ctx->tc_err;
     kp.epi = make_epi(ctx, flags, 0, sh);
+    if (!blocks) kp.epi.seg = ctx->n;
     if (comp) AP_CK(launch_kmv_comp(ctx->kernel, kp, ctx->D, ctx->Cp, ctx->st));
     else AP_CK(launch_kmv(ctx->kernel, kp, ctx->D, ctx->Cp, ctx->st));
     ++ctx->launches;
@@ -746,10 +763,7 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
     ++ctx->launches;
     AP_CK(cudaMemsetAsync(ctx->step, 0, sizeof(int64_t), ctx->st));
     AP_CK(cudaMemsetAsync(ctx->nan_flag, 0, sizeof(int), ctx->st));
-    AP_CK(cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->st));
-    // arrival tickets start at zero (a launch that gave up on a wait leaves them partial)
-    AP_CK(cudaMemsetAsync(ctx->ticket, 0, 4 * sizeof(unsigned), ctx->st));
-    if (ctx->tc_tick) AP_CK(cudaMemsetAsync(ctx->tc_tick, 0, sizeof(int) * ctx->num_sms, ctx->st));
+    AP_TRY(reset_waits(ctx));
     // ||b_c|| for the relative residuals
     AP_TRY(launch_norms(ctx, ctx->Bp, kEpiColNorms));
     double bn[AP_MAX_RHS] = {}, rn[AP_MAX_RHS] = {};
@@ -828,7 +842,12 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
             AP_CK(cudaEventRecord(ctx->ev_r1, ctx->st));
             AP_CK(cudaMemcpyAsync(rn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
             AP_CK(cudaMemcpyAsync(&nanf, ctx->nan_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+            AP_CK(cudaMemcpyAsync(&tcerr, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
             AP_CK(cudaStreamSynchronize(ctx->st));
+            if (tcerr) {
+                status = AP_ERR_TIMEOUT;
+                break;
+            }
             float rms = 0.f;
             cudaEventElapsedTime(&rms, ctx->ev_r0, ctx->ev_r1);
             t_refine += rms * 1e-3;
@@ -854,7 +873,12 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
             AP_CK(cudaEventRecord(ctx->ev_r1, ctx->st));
             AP_CK(cudaMemcpyAsync(rn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
             AP_CK(cudaMemcpyAsync(&nanf, ctx->nan_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+            AP_CK(cudaMemcpyAsync(&tcerr, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
             AP_CK(cudaStreamSynchronize(ctx->st));
+            if (tcerr) {
+                status = AP_ERR_TIMEOUT;
+                break;
+            }
             float rms = 0.f;
             cudaEventElapsedTime(&rms, ctx->ev_r0, ctx->ev_r1);
             t_refine += rms * 1e-3;
@@ -907,8 +931,11 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
         AP_CK(cudaEventRecord(ctx->ev_r0, ctx->st));
         AP_TRY(launch_full_residual(ctx, ctx->Bp, ctx->W, ctx->R, kEpiColNorms));
         AP_CK(cudaEventRecord(ctx->ev_r1, ctx->st));
+        int tcerr = 0;
         AP_CK(cudaMemcpyAsync(rn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
+        AP_CK(cudaMemcpyAsync(&tcerr, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
         AP_CK(cudaStreamSynchronize(ctx->st));
+        if (tcerr) status = AP_ERR_TIMEOUT;
         float rms = 0.f;
         cudaEventElapsedTime(&rms, ctx->ev_r0, ctx->ev_r1);
         t_refine += rms * 1e-3;
@@ -1229,13 +1256,18 @@ ap_status ap_residual(ap_ctx* ctx, const float* B_dev, int32_t c, const float* W
     AP_TRY(ensure_solve(ctx, Cp));
     ctx->r_tracked_c = 0;
     AP_TRY(enter(ctx));
+    const bool waits = Cp >= kX3MinC && !use_compensated(ctx);  // the tensor-core form runs
+    if (waits) AP_TRY(reset_waits(ctx));
     AP_CK(launch_pad_copy(B_dev, ctx->n, c, ctx->Bp, Cp, ctx->st));
     AP_CK(launch_pad_copy(W_dev, ctx->n, c, ctx->Tmp, Cp, ctx->st));
     ctx->launches += 2;
     AP_TRY(launch_full_residual(ctx, ctx->Bp, ctx->Tmp, ctx->R, 0));
     AP_CK(launch_unpad_copy(ctx->R, ctx->n, Cp, R_dev, c, ctx->st));
     ++ctx->launches;
-    return leave(ctx);
+    int tmo = 0;
+    if (waits) AP_CK(cudaMemcpyAsync(&tmo, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+    AP_TRY(leave(ctx));
+    return tmo ? AP_ERR_TIMEOUT : AP_OK;
 }
 
 ap_status ap_predict_mean(ap_ctx* ctx, const float* w_dev, const float* Xs_dev, int64_t M, float* mean_dev) {

@@ -92,27 +92,38 @@ struct KmvParams {
     const float* Xa_lo;    // compensated form only: low parts of the scaled inputs
     const float* Xb_lo;
     int rm;                // rows per thread (KmvSplit)
-    int G;                 // column groups per row tile on top of the cluster's S splits (KmvSplit)
+    int G;                 // > 1: row tiles are shared between CTAs through gscr (KmvSplit)
+    int ctas;              // CTAs of the tensor-core form's persistent grid (KmvSplit)
     float* gscr;           // G > 1: partial sums (KmvSplit::scratch floats)
     unsigned int* gtick;   // G > 1: arrival tickets (KmvSplit::tickets), zero between launches
+    int* err;              // wait-timeout flag of the tensor-core form
     EpiParams epi;
 };
 
 // How one FP32 product is cut into CTAs: row tiles of 128 * rm rows (never across a
-// segment), S column splits per tile summed inside a cluster, G groups of S splits
-// summed through global memory by the last group to arrive.
+// segment).  SIMT form (C <= 4): S column splits per tile summed inside a cluster, G
+// groups of S splits summed through global memory by the last group to arrive.
+// Tensor-core form: a persistent grid over (tile, column chunk) units; G > 1 lets a
+// range of units end inside a tile.
 struct KmvSplit {
-    int rm, S, G;
+    int rm, S, G, ctas;
     int64_t rows, tps, ntiles;
     int64_t scratch;  // floats of partial sums when G > 1
     int64_t tickets;  // arrival tickets when G > 1
 };
 KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols);
+constexpr int kX3MinC = 16;  // right-hand sides (padded) from which the tensor-core form runs
+constexpr int kX3MaxD2 = 16; // largest D whose two rows per thread fit the registers
+constexpr int kX3Chunk = 128;
 
 // FP32 SIMT kernel-matrix product with the AP epilogue (one per kernel family TU).
 cudaError_t launch_kmv_rbf(const KmvParams& p, int D, int C, cudaStream_t st);
 cudaError_t launch_kmv_m32(const KmvParams& p, int D, int C, cudaStream_t st);
 cudaError_t launch_kmv_m52(const KmvParams& p, int D, int C, cudaStream_t st);
+// The same product for C >= kX3MinC with the contraction on the tensor cores (kmv_x3.cuh).
+cudaError_t launch_x3_rbf(const KmvParams& p, int D, int C, cudaStream_t st);
+cudaError_t launch_x3_m32(const KmvParams& p, int D, int C, cudaStream_t st);
+cudaError_t launch_x3_m52(const KmvParams& p, int D, int C, cudaStream_t st);
 cudaError_t launch_kmv(int kernel, const KmvParams& p, int D, int C, cudaStream_t st);
 // Compensated (double-float FP32) form of the same product, for refinement.
 cudaError_t launch_kmv_comp_rbf(const KmvParams& p, int D, int C, cudaStream_t st);

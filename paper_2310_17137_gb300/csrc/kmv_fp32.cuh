@@ -1,4 +1,4 @@
-// FP32 SIMT form of the fused kernel-matrix product (the AP residual update,
+// FP32 SIMT form (up to 4 right-hand sides; kmv_x3.cuh for more) of the fused kernel-matrix product (the AP residual update,
 // Eq. text_update_of_r, the residual recompute of the App. B lemma and the
 // posterior mean of Sec. 2), with the block-norm / Gauss-Southwell epilogue of
 // Eq. approximate_gauss_southwell fused in.
@@ -493,8 +493,6 @@ cudaError_t dispatch_kmv(const KmvParams& p, int D, int C, cudaStream_t st) {
     switch (C) {                                                          \
         case 1: return launch_kmv_inst<KERN, DD, 1>(p, st);               \
         case 4: return launch_kmv_inst<KERN, DD, 4>(p, st);               \
-        case 16: return launch_kmv_inst<KERN, DD, 16>(p, st);             \
-        case 32: return launch_kmv_inst<KERN, DD, 32>(p, st);             \
         default: return cudaErrorInvalidValue;                            \
     }
     switch (D) {

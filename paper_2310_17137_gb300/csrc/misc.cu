@@ -19,41 +19,52 @@ double kernel_input_scale(int kernel) {
 // Rows per thread: more rows share each staged column (the shared-memory reads per
 // entry fall as 1 / rm), but a tile of 128 rm rows may be mostly padding (a segment of
 // 600 rows is 60 % of two 512-row tiles) and leaves fewer tiles.  The modelled issue
-// slots per useful entry, times the shortfall of CTAs when the whole product cannot
-// give two per SM, decide.
+// slots per useful entry, times the shortfall of work when the whole product cannot
+// fill the chip, decide.
 //
-// Columns: S splits inside a cluster until 4 CTAs per SM exist, then G groups through
-// global memory: enough of them for about 8 waves of CTAs while every CTA keeps at
-// least 512 columns and 64 per right-hand side (a last wave that is nearly empty costs
-// at most an eighth; shorter ranges measured slower, 11.9 -> 12.3 ms on 16 steps of
-// n = 65,536, b = 4096, c = 32), and for 8 CTAs per SM with at least 64 columns when the
-// clusters alone leave places free.  Measured on GB300: n = 100,003, d = 11, 1024 test
-// points, 16 CTAs (cluster only) 1102 us per ap_predict_mean call, with the groups
-// 135 us; n = 20,600, d = 8, one column, ap_residual 500 -> 377 us.
+// Columns, SIMT form: S splits inside a cluster until 4 CTAs per SM exist, then G groups
+// through global memory: enough of them for about 8 waves of CTAs while every CTA keeps
+// at least 512 columns (a last wave that is nearly empty costs at most an eighth), and
+// for 8 CTAs per SM with at least 64 columns when the clusters alone leave places free.
+// Measured on GB300: n = 100,003, d = 11, 1024 test points, 16 CTAs (cluster only)
+// 1102 us per ap_predict_mean call, with the groups 135 us; n = 20,600, d = 8, one
+// column, ap_residual 500 -> 377 us.
+// Tensor-core form: one CTA per SM over equal ranges of (tile, 128-column chunk) units.
 KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
     constexpr int64_t kSms = 152, kMaxScratch = (int64_t)8 << 20;
+    const bool x3 = C >= kX3MinC;
+    const int64_t chunk = x3 ? kX3Chunk : kKmvTN;
+    const double places = x3 ? kSms : 2.0 * kSms;
+    const double instr = x3 ? D + 16.0 : D + C + 8.0, lds = x3 ? D / 4.0 : (D + C) / 4.0;
     KmvSplit best = {};
     double best_cost = 0.0;
-    for (int rm = rows_per_thread(D, C); rm >= 1; rm /= 2) {
+    for (int rm = x3 ? (D <= kX3MaxD2 ? 2 : 1) : rows_per_thread(D, C); rm >= 1; rm /= 2) {
         KmvSplit sp = {};
         sp.rm = rm;
         sp.rows = (int64_t)kKmvThreads * rm;
         sp.tps = (seg + sp.rows - 1) / sp.rows;
         sp.ntiles = nseg * sp.tps;
         const double pad = (double)(sp.tps * sp.rows) / (double)seg;
-        const double ctas = (double)sp.ntiles * (double)((ncols + kKmvTN - 1) / kKmvTN);
-        const double idle = ctas < 2.0 * kSms ? 2.0 * kSms / ctas : 1.0;
-        const double cost = pad * idle * ((D + C + 8) + (D + C) / (4.0 * rm));
+        const double units = (double)sp.ntiles * (double)((ncols + chunk - 1) / chunk);
+        const double idle = units < places ? places / units : 1.0;
+        const double cost = pad * idle * (instr + lds / rm);
         if (!best.rm || cost < best_cost) best = sp, best_cost = cost;
     }
     best.S = 1;
-    while (best.S < kMaxSplit && best.ntiles * best.S < 4 * kSms && ncols / (2 * best.S) >= kKmvTN) best.S *= 2;
+    if (x3) {
+        best.ctas = (int)std::min<int64_t>(kSms, best.ntiles * ((ncols + chunk - 1) / chunk));
+        best.G = 2;
+        best.scratch = 2 * (int64_t)best.ctas * best.rows * C;
+        best.tickets = best.ntiles;
+        return best;
+    }
+    while (best.S < kMaxSplit && best.ntiles * best.S < 4 * kSms && ncols / (2 * best.S) >= chunk) best.S *= 2;
     const int64_t ctas = best.ntiles * best.S;
     auto groups = [&](int64_t want, int64_t min_cols) {
         return std::min<int64_t>((want + ctas - 1) / ctas, ncols / (best.S * min_cols));
     };
-    int64_t G = groups(64 * kSms, std::max(512, 64 * C));
-    if (ctas < 4 * kSms) G = std::max(G, groups(8 * kSms, kKmvTN));
+    int64_t G = groups(64 * kSms, 512);
+    if (ctas < 4 * kSms) G = std::max(G, groups(8 * kSms, chunk));
     G = std::min<int64_t>(G, kMaxScratch / (best.ntiles * best.rows * C));
     best.G = (int)std::max<int64_t>(1, std::min<int64_t>(G, 1024));
     if (best.G > 1) {
@@ -64,10 +75,11 @@ KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
 }
 
 cudaError_t launch_kmv(int kernel, const KmvParams& p, int D, int C, cudaStream_t st) {
+    const bool x3 = C >= kX3MinC;
     switch (kernel) {
-        case AP_RBF: return launch_kmv_rbf(p, D, C, st);
-        case AP_MATERN32: return launch_kmv_m32(p, D, C, st);
-        case AP_MATERN52: return launch_kmv_m52(p, D, C, st);
+        case AP_RBF: return x3 ? launch_x3_rbf(p, D, C, st) : launch_kmv_rbf(p, D, C, st);
+        case AP_MATERN32: return x3 ? launch_x3_m32(p, D, C, st) : launch_kmv_m32(p, D, C, st);
+        case AP_MATERN52: return x3 ? launch_x3_m52(p, D, C, st) : launch_kmv_m52(p, D, C, st);
         default: return cudaErrorInvalidValue;
     }
 }
