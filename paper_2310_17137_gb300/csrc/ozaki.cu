@@ -15,13 +15,14 @@
 //   2. for every level L = p + q = 2..9 the tensor cores accumulate
 //      acc_L = sum_{p+q=L} sum_kk s_p(r, kk) s_q(c, kk) in FP32.  Every partial
 //      sum is an integer below 2^22, so the accumulation is exact;
-//   3. the levels are combined exactly in 64-bit integers,
-//      H = sum_{L<=5} acc_L 2^{7(5-L)}, Lo = sum_{L>=6} acc_L 2^{7(9-L)}, and
-//      A_rc -= 2^{e_r+e_c-35} (H + 2^-28 Lo) with two FP64 roundings.
-// The terms left out (levels above 9 and the slice remainders) are below about
-// 2^-50 K max_kk|a_r,kk| max_kk|a_c,kk| per entry, the size of FP64 rounding
-// when the entries of a panel row have similar magnitudes; the matrix itself
-// stays FP64.  On kernel blocks the factor's backward error ||L L^T - K|| / ||K||
+//   3. the levels are combined in integers,
+//      H = sum_{L<=5} acc_L 2^{7(5-L)}, Lo = sum_{L>=6} acc_L 2^{7(9-L)},
+//      T = 2^19 H + round(2^-9 Lo) (below 2^63), and A_rc -= 2^{e_r+e_c-54} T with
+//      two FP64 roundings: T's own to 53 bits, in integer arithmetic, and the sum's.
+// The terms left out (levels above 9, the slice remainders, Lo's last 9 bits) are
+// below about 2^-50 K max_kk|a_r,kk| max_kk|a_c,kk| per entry, the size of FP64
+// rounding when the entries of a panel row have similar magnitudes; the matrix
+// itself stays FP64.  On kernel blocks the factor's backward error ||L L^T - K|| / ||K||
 // matches the all-FP64 factorisation (6e-16 vs 5e-16 on a Matern-5/2 block
 // with condition number 1.6e4, in a NumPy model of these exact steps).
 //
@@ -32,6 +33,14 @@
 // columns), then an epilogue of one row per thread.  One persistent CTA per SM
 // walks the work items; the next item's slices are copied in while the
 // epilogue of the current one runs.  Every wait is bounded.
+//
+// The epilogue is what bounds the kernel: FP64 runs at 2 results per clock per SM, so
+// an FP64 operation per entry of a super-tile costs 4096 clocks, as much as all its
+// MMAs.  It therefore reads and combines the accumulators in 32-bit integers first
+// (after which the next item's MMAs start), builds each product's double with integer
+// instructions, and spends one FP64 operation per entry, the subtraction itself, under
+// those MMAs.  Measured (GB300, b = 4096, mean over the 63 panels): 5 blocks 277 -> 148 us,
+// 13 blocks 693 -> 395 us; panel solves of 5 blocks 33 -> 14 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -50,7 +59,8 @@ constexpr int kSlabRows = 2 * T;                            // rows of a super-t
 constexpr uint32_t kPlaneA = kSlabRows * T * 2;             // 16 KB of BF16
 constexpr uint32_t kPlaneB = T * T * 2;                     // 8 KB
 constexpr uint32_t kOzSmem = kSlices * (kPlaneA + kPlaneB); // 192 KB
-constexpr int kOzThreads = 256;  // 8 warps: two per tensor-memory lane quarter
+constexpr int kEpiWarps = 16;                             // four per tensor-memory lane quarter
+constexpr int kOzThreads = (kEpiWarps + 1) * 32;          // and one that issues copies and MMAs
 constexpr uint32_t kRowBytes = T * 2;                       // one slice row (64 BF16)
 constexpr int kBadExp = -(1 << 30);  // row exponent marking a non-finite panel row
 
@@ -129,6 +139,27 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const double* src0, int64
     if (grp == 0) E[(int64_t)z * rows_pad + r] = nonfinite ? kBadExp : e;
 }
 
+// 2^e0 (2^33 h1 + 2^19 h2 + 2^5 l1 + round(2^-9 l2)) rounded to a double, h1 .. l2
+// below 2^29: the sum is a 64-bit integer below 2^63, normalised and rounded (half
+// away from zero) with integer instructions.
+__device__ __noinline__ double level_sum_extreme(long long v, int e0) {  // beyond the normal doubles
+    return ldexp((double)v, max(-2000, min(2000, e0)));
+}
+
+__device__ __forceinline__ double level_sum(int h1, int h2, int l1, int l2, int e0) {
+    const long long v = (long long)h1 * (1LL << 33) + (long long)h2 * (1LL << 19) + (long long)l1 * 32 + ((l2 + 256) >> 9);
+    if (v == 0) return 0.0;
+    const long long sign = v >> 63;
+    const unsigned long long m0 = (unsigned long long)((v ^ sign) - sign);
+    const int lz = __clzll((long long)m0);
+    const int be = 1023 + 63 - lz + e0;  // biased exponent
+    if (be < 1 || be > 2045) return level_sum_extreme(v, e0);
+    const unsigned long long m = m0 << lz;
+    const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // 53 bits, the leading one included
+    const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + r;
+    return __longlong_as_double((long long)(bits | ((unsigned long long)sign & 0x8000000000000000ull)));
+}
+
 // kTrsm = false: A_ij -= A_ik A_jk^T over the trailing lower tiles (SYRK/GEMM);
 // kTrsm = true:  A_ik := A_ik L_kk^{-T} for the panel tiles i > k (TRSM as a
 // product with the inverse diagonal tile, whose slices sit in the plane rows
@@ -138,11 +169,12 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
                                                                size_t plane_bytes, const int* E, int* err,
                                                                int tiles_per_block, int nwork) {
     extern __shared__ __align__(1024) uint8_t oz_smem[];
-    __shared__ __align__(8) uint64_t bar_load, bar_mma;
+    // slices in shared memory, accumulators complete, accumulators read
+    __shared__ __align__(8) uint64_t bar_load, bar_mma, bar_read;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
-    __shared__ int s_ec[T];
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int rem = nt - k - 1;
     const int64_t ld = (int64_t)nt * T, rows_pad = ld + T;
     uint8_t* sA = oz_smem;
@@ -182,10 +214,11 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
     if (tid == 0) {
         mbar_init(&bar_load, 1);
         mbar_init(&bar_mma, 1);
+        mbar_init(&bar_read, kEpiWarps);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) {
+    if (warp == kEpiWarps) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                      "r"(512)
                      : "memory");
@@ -195,108 +228,125 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
-    if (tid == 0 && (int)blockIdx.x < nwork) issue_loads((int)blockIdx.x);
 
-    // Persistent loop: the slices of the next work item are copied in while the
-    // epilogue of the current one runs (shared memory is free once its MMAs are
-    // done; the accumulators are free after the epilogue).
-    int it = 0;
-    for (int w = (int)blockIdx.x; w < nwork; w += (int)gridDim.x, ++it) {
-        int z, i0, j;
-        decode(w, z, i0, j);
-        if (tid < T) s_ec[tid] = E[(int64_t)z * rows_pad + (int64_t)j * T + tid];
-        __syncthreads();
-        if (tid == 0) {
-            if (mbar_wait(&bar_load, (uint32_t)(it & 1), &s_abort, err)) {
-                tc_fence_after();
-                constexpr uint32_t idesc = instr_desc(1, kSlabRows, T);  // BF16 x BF16 -> F32, 128 x 64
-                const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
+    if (warp == kEpiWarps) {
+        // ------------------------------------------------- copy and MMA issuer
+        // (whole warp in the loop, warp-uniform descriptors, one elected lane issues)
+        constexpr uint32_t idesc = instr_desc(1, kSlabRows, T);  // BF16 x BF16 -> F32, 128 x 64
+        const bool leader = elect_one();
+        const uint64_t a0 = smem_desc(smem_u32(sA), 128, 1024), b0 = smem_desc(smem_u32(sB), 128, 1024);
+        if (leader && (int)blockIdx.x < nwork) issue_loads((int)blockIdx.x);
+        __syncwarp();
+        bool ok = true;
+        int it = 0;
+        for (int w = (int)blockIdx.x; w < nwork && ok; w += (int)gridDim.x, ++it) {
+            ok = mbar_wait(&bar_load, (uint32_t)(it & 1), &s_abort, err) &&
+                 (it == 0 || mbar_wait(&bar_read, (uint32_t)((it - 1) & 1), &s_abort, err));
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            if (leader) {
+#pragma unroll 1
                 for (int L = 2; L <= kSlices + 1; ++L) {
                     const uint32_t d = tmem + 64u * (uint32_t)(L - 2);
                     uint32_t acc = 0;
-                    for (int p = max(1, L - kSlices); p <= min(kSlices, L - 1); ++p) {
-                        const int q = L - p;
-                        const uint32_t ap = a0 + (uint32_t)(p - 1) * kPlaneA, bq = b0 + (uint32_t)(q - 1) * kPlaneB;
+#pragma unroll 1
+                    for (int p = 1; p < L; ++p) {  // level L <= 9: slices p and L - p, both <= 8
+                        const uint64_t ap = a0 + (uint64_t)(((p - 1) * kPlaneA) >> 4);
+                        const uint64_t bq = b0 + (uint64_t)(((L - p - 1) * kPlaneB) >> 4);
 #pragma unroll
                         for (int ks = 0; ks < T / 16; ++ks) {
-                            mma_ss(d, smem_desc(ap + ks * 256, 128, 1024), smem_desc(bq + ks * 256, 128, 1024),
-                                   idesc, acc);
+                            mma_ss(d, ap + (uint64_t)(ks * 16), bq + (uint64_t)(ks * 16), idesc, acc);
                             acc = 1;
                         }
                     }
                 }
                 tc_commit(&bar_mma);
             }
+            __syncwarp();
+            if (w + (int)gridDim.x < nwork) {
+                // the MMAs have consumed the slices: fetch the next item's
+                ok = __all_sync(0xffffffffu, mbar_wait(&bar_mma, (uint32_t)(it & 1), &s_abort, err));
+                if (ok && leader) issue_loads(w + (int)gridDim.x);
+                __syncwarp();
+            }
         }
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(&bar_mma, (uint32_t)(it & 1), &s_abort, err));
-        if (ok) tc_fence_after();
-        // the shared slices are consumed: fetch the next work item's
-        if (tid == 0 && ok && w + (int)gridDim.x < nwork) issue_loads(w + (int)gridDim.x);
-
-        // epilogue: warp v owns tensor-memory lanes (rows) 32 (v % 4) .. + 31 and
-        // columns 32 (v / 4) .. + 31 of the super-tile
-        const int rl = 32 * (warp & 3) + (tid & 31);
-        const int64_t r = (int64_t)i0 * T + rl;
-        const int rtile = i0 + rl / T;
-        const bool live = ok && rtile < nt && (kTrsm || j <= rtile);
-        const int er = live ? E[(int64_t)z * rows_pad + r] : 0;
-        double* Crow = A + (int64_t)z * ld * ld + r * ld + (int64_t)j * T;
+    } else {
+        // ------------------------------------------------------------ epilogue
+        // warp v owns tensor-memory lanes (rows) 32 (v % 4) .. + 31 and columns
+        // 16 (v / 4) .. + 15 of the super-tile
+        const int rl = 32 * (warp & 3) + lane, c0 = 16 * (warp >> 2);
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        // exact conversions: an FP32 integer below 2^22 through the FP32 mantissa,
-        // a 64-bit integer below 2^51 through the FP64 mantissa
-        constexpr float kMagicF = 12582912.0f;                  // 1.5 * 2^23
-        constexpr long long kMagicDBits = 0x4338000000000000LL;  // 1.5 * 2^52
-        constexpr double kMagicD = 6755399441055744.0;
-#pragma unroll 1
-        for (int c0 = 32 * (warp >> 2); c0 < 32 * (warp >> 2) + 32; c0 += 16) {
-            long long H[16], Lo[16];
+        int it = 0;
+        for (int w = (int)blockIdx.x; w < nwork; w += (int)gridDim.x, ++it) {
+            int z, i0, j;
+            decode(w, z, i0, j);
+            const int64_t r = (int64_t)i0 * T + rl;
+            const int rtile = i0 + rl / T;
+            const bool mine = rtile < nt && (kTrsm || j <= rtile);
+            const int er = mine ? E[(int64_t)z * rows_pad + r] : 0;
+            const int ecl = E[(int64_t)z * rows_pad + (int64_t)j * T + c0 + (lane & 15)];
+            double2* Crow = reinterpret_cast<double2*>(A + (int64_t)z * ld * ld + r * ld + (int64_t)j * T + c0);
+            if (!kTrsm && mine) asm volatile("prefetch.global.L2 [%0];" ::"l"(Crow));
+            if (!__all_sync(0xffffffffu, mbar_wait(&bar_mma, (uint32_t)(it & 1), &s_abort, err))) break;
+            tc_fence_after();
+            // pairs of levels as exact 32-bit integers, acc_L 2^7 + acc_{L+1} (below 2^29)
+            int q[4][16];
 #pragma unroll
-            for (int c = 0; c < 16; ++c) H[c] = Lo[c] = 0;
+            for (int half = 0; half < 2; ++half) {
 #pragma unroll
-            for (int L = 2; L <= kSlices + 1; ++L) {
-                uint32_t v[16];
-                if (ok) {
-                    tmem_ld16(tmem + lane_base + 64u * (uint32_t)(L - 2) + (uint32_t)c0, v);
+                for (int pr = 0; pr < 4; ++pr) {
+                    uint32_t va[8], vb[8];
+                    const uint32_t at = tmem + lane_base + 128u * (uint32_t)pr + (uint32_t)(c0 + 8 * half);
+                    tmem_ld8(at, va);
+                    tmem_ld8(at + 64u, vb);
                     tmem_wait_ld();
-                } else {
+                    // exact conversion of an FP32 integer below 2^22: its bits after adding
+                    // 1.5 * 2^23 are the integer plus those of the constant
+                    constexpr float kMagicF = 12582912.0f;
+                    constexpr unsigned kMagicBits = 0x4b400000u;
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) v[c] = 0u;
-                }
-#pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const long long iv =
-                        (long long)(__float_as_int(__uint_as_float(v[c]) + kMagicF) - __float_as_int(kMagicF));
-                    if (L <= 5) H[c] = H[c] * 128 + iv;
-                    else Lo[c] = Lo[c] * 128 + iv;
+                    for (int c = 0; c < 8; ++c) {
+                        const unsigned ba = __float_as_uint(__uint_as_float(va[c]) + kMagicF);
+                        const unsigned bb = __float_as_uint(__uint_as_float(vb[c]) + kMagicF);
+                        q[pr][8 * half + c] = (int)(ba * 128u + bb - 129u * kMagicBits);
+                    }
                 }
             }
-            if (live) {
+            // every accumulator has been read: the next item's MMAs may overwrite them
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_read);
+            if (!mine) continue;  // (warp-uniform: a warp's 32 rows lie in one tile)
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const double hd = __longlong_as_double(kMagicDBits + H[c]) - kMagicD;
-                    const double ld_ = __longlong_as_double(kMagicDBits + Lo[c]) - kMagicD;
-                    const double t = fma(ld_, 0x1p-28, hd);
-                    const int ec = s_ec[c0 + c];
-                    const int e = er + ec - 35;
-                    double scale;
-                    if (e >= -1022 && e <= 1023) scale = __longlong_as_double((long long)(e + 1023) << 52);
-                    else scale = ldexp(1.0, max(-1074, min(1023, e)));
-                    const double nv = kTrsm ? t * scale : fma(-t, scale, Crow[c0 + c]);
-                    Crow[c0 + c] = (er == kBadExp || ec == kBadExp) ? __longlong_as_double(0x7ff8000000000000LL) : nv;
+            for (int half = 0; half < 2; ++half) {
+                double2 cv[4];
+                if constexpr (!kTrsm) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) cv[c] = Crow[4 * half + c];
                 }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const int cc = 8 * half + c;
+                    const int ec = __shfl_sync(0xffffffffu, ecl, cc);
+                    double t = level_sum(q[0][cc], q[1][cc], q[2][cc], q[3][cc], er + ec - 54);
+                    // a NaN or infinity in the panel must reach the next pivot test as NaN
+                    if (er == kBadExp || ec == kBadExp) t = __longlong_as_double(0x7ff8000000000000LL);
+                    double& dst = c & 1 ? cv[c / 2].y : cv[c / 2].x;
+                    if constexpr (kTrsm) dst = t;
+                    else dst -= t;
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) Crow[4 * half + c] = cv[c];
             }
         }
-        // every accumulator has been read before the next MMAs overwrite them
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        if (s_abort) break;
     }
 
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) {
+    if (warp == kEpiWarps) {
         if (s_abort) {
             // a wait gave up: let copies and MMAs still in flight land first
             const long long t0 = clock64();
