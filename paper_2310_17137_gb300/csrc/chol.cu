@@ -155,17 +155,82 @@ __global__ void __launch_bounds__(256) phi_fp64_eval_kernel(int kernel, const do
         out[i] = phi_fp64(kernel, r2[i], s_tab);
 }
 
-// Factor the diagonal tile (k, k) in place and write its inverse to Dinv.
-// 1/sqrt(p) for a pivot: the FP32 reciprocal square root refined by two
-// Newton steps in FP64 (relative error 2^-22 -> 2^-44 -> below the last bit);
-// outside the FP32 range the library square root and division.
+// 1/sqrt(p) for a pivot: the reciprocal square root approximation (relative error
+// below 2^-21) refined by one third-order step, y + y e (1/2 + 3/8 e) with
+// e = 1 - p y^2 (error 5/16 e^3 < 2^-60, below the last bit); outside the FP32 range
+// the library square root and division.
 __device__ __forceinline__ double rsqrt_pivot(double p) {
     if (!(p > 1e-30 && p < 1e30)) return 1.0 / sqrt(p);
-    float yf;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"((float)p));
-    double y = (double)yf;
-    y = fma(0.5 * y, fma(-p * y, y, 1.0), y);
-    return fma(0.5 * y, fma(-p * y, y, 1.0), y);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(p));
+    const double e = fma(-p * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// Factor the diagonal tile (k, k) in place and write its inverse to Dinv.
+//
+// One CTA per block, on the critical path of every panel.  FP64 runs at 2 results per
+// clock per SM, whoever asks: a warp instruction holds the pipe for 16 clocks, so the
+// 2 x 64^3 / 6 multiply-adds of the factor and the inverse cost 21 us however they are
+// arranged, and work done for all threads (or by threads with nothing to do) counts in
+// full.  The tile is factored in 16-column panels: the diagonal 16 x 16 in one warp's
+// registers (the pivot chain: shuffles and about six dependent FP64 operations per
+// column, no CTA barrier), the rows below by one thread each, the rest as a rank-16
+// update on all warps.  While warp 0 is on a diagonal block, the other warps form the
+// inverse's block row above it, X_ik = -X_ii sum_j L_ij X_jk.
+// Measured (GB300, 5 blocks): 206 us per launch with a barrier round per column and
+// every thread deriving every pivot, 101 us now (FP64 pipe 46 % busy).
+constexpr int NB = 16;
+
+__device__ __forceinline__ void bar_sync_n(int id, int n) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+// Block row bi of the inverse by threads t = 0 .. nthr - 1 (whole warps, named barrier id).
+__device__ __forceinline__ void inverse_block_row(const double* a, double* x, const double* s_rd, int bi, int t,
+                                                  int nthr, int bar) {
+    const int r0 = NB * bi;
+    if (t < 32) {
+        // X_ii: lane c forward-substitutes the unit vector c (lanes 16 .. 31 repeat 0 .. 15)
+        const int c = t & (NB - 1);
+        double v[NB];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) v[i] = i == c ? 1.0 : 0.0;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            v[i] *= s_rd[r0 + i];
+#pragma unroll
+            for (int l = i + 1; l < NB; ++l) v[l] = fma(-a[(r0 + l) * TP + r0 + i], v[i], v[l]);
+        }
+        if (t < NB) {
+#pragma unroll
+            for (int i = 0; i < NB; ++i) x[(r0 + i) * TP + r0 + c] = v[i];
+        }
+    } else {
+        // E_ik = sum_j L_ij X_jk (j = k .. i - 1) into the place of X_ik
+        for (int o = t - 32; o < bi * NB * NB; o += nthr - 32) {
+            const int c = o % (bi * NB), r = r0 + o / (bi * NB);
+            double s0 = 0.0, s1 = 0.0;
+            for (int q = c & ~(NB - 1); q < r0; q += 2) {
+                s0 = fma(a[r * TP + q], x[q * TP + c], s0);
+                s1 = fma(a[r * TP + q + 1], x[(q + 1) * TP + c], s1);
+            }
+            x[r * TP + c] = s0 + s1;
+        }
+    }
+    bar_sync_n(bar, nthr);
+    double out[4];
+    int n = 0;
+    for (int o = t; o < bi * NB * NB; o += nthr, ++n) {
+        const int c = o % (bi * NB), rl = o / (bi * NB);
+        double s = 0.0;
+        for (int q = 0; q <= rl; ++q) s = fma(x[(r0 + rl) * TP + r0 + q], x[(r0 + q) * TP + c], s);
+        out[n & 3] = -s;
+    }
+    bar_sync_n(bar, nthr);
+    n = 0;
+    for (int o = t; o < bi * NB * NB; o += nthr, ++n) x[(r0 + o / (bi * NB)) * TP + o % (bi * NB)] = out[n & 3];
+    bar_sync_n(bar, nthr);
 }
 
 __global__ void __launch_bounds__(256) potrf_diag_kernel(double* A, int nt, int k, double* Dinv, int* bad) {
@@ -175,57 +240,85 @@ __global__ void __launch_bounds__(256) potrf_diag_kernel(double* A, int nt, int 
     __shared__ double s_rd[T];  // 1 / L_jj
     __shared__ int s_bad;
     const int z = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
-    const int ty = tid / 16, tx = tid % 16;
+    const int warp = tid >> 5, lane = tid & 31;
     const int64_t ld = (int64_t)nt * T;
     double* Ab = A + (int64_t)z * ld * ld + (int64_t)k * T * ld + (int64_t)k * T;
     for (int t = tid; t < T * T; t += nth) {
         const int r = t / T, q = t % T;
         a[r * TP + q] = (q <= r) ? Ab[r * ld + q] : 0.0;
+        x[r * TP + q] = 0.0;
     }
     if (tid == 0) s_bad = 0;
-    __syncthreads();
-    for (int j = 0; j < T; ++j) {
-        // every thread derives the pivot's reciprocal square root itself
-        double pv = a[j * TP + j];
-        const bool badp = !(pv > 0.0) || !isfinite(pv);
-        if (badp) pv = 1.0;
-        const double rj = rsqrt_pivot(pv);
-        __syncthreads();  // everyone has read the pivot
-        if (tid == 0) {
-            if (badp) s_bad = 1;
-            const double l = pv * rj;
-            a[j * TP + j] = fma(0.5 * rj, fma(-l, l, pv), l);  // sqrt(pv), Newton-corrected
-            s_rd[j] = rj;
-        }
-        for (int i = j + 1 + tid; i < T; i += nth) a[i * TP + j] *= rj;
+    for (int kb = 0; kb < T / NB; ++kb) {
+        const int c0 = NB * kb;
         __syncthreads();
-        // trailing update of the lower triangle, rows j+1+ty+16a, columns j+1+tx+16b
-        for (int i = j + 1 + ty; i < T; i += 16) {
-            const double aij = a[i * TP + j];
-            for (int l = j + 1 + tx; l <= i; l += 16) a[i * TP + l] = fma(-aij, a[l * TP + j], a[i * TP + l]);
-        }
-        __syncthreads();
-    }
-    // inverse of the lower-triangular tile, one column per thread, the inner
-    // products in four independent partial sums
-    if (tid < T) {
-        const int c = tid;
-        for (int i = 0; i < c; ++i) x[i * TP + c] = 0.0;
-        x[c * TP + c] = s_rd[c];
-        for (int i = c + 1; i < T; ++i) {
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            int q = c;
-            for (; q + 3 < i; q += 4) {
-                s0 = fma(a[i * TP + q], x[q * TP + c], s0);
-                s1 = fma(a[i * TP + q + 1], x[(q + 1) * TP + c], s1);
-                s2 = fma(a[i * TP + q + 2], x[(q + 2) * TP + c], s2);
-                s3 = fma(a[i * TP + q + 3], x[(q + 3) * TP + c], s3);
+        if (warp == 0) {
+            // the diagonal block: lane i holds row c0 + i (lanes 16 .. 31 repeat 0 .. 15)
+            const int i = lane & (NB - 1);
+            double p[NB];
+#pragma unroll
+            for (int j = 0; j < NB; ++j) p[j] = a[(c0 + i) * TP + c0 + j];
+            bool anybad = false;
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                double pv = __shfl_sync(0xffffffffu, p[j], j);
+                const bool badp = !(pv > 0.0) || !isfinite(pv);
+                if (badp) pv = 1.0;
+                anybad |= badp;
+                const double rj = rsqrt_pivot(pv);
+                if (lane == j) s_rd[c0 + j] = rj;
+                p[j] *= rj;
+                if (i == j) {
+                    const double l = pv * rj;
+                    p[j] = fma(0.5 * rj, fma(-l, l, pv), l);  // sqrt(pv), Newton-corrected
+                }
+#pragma unroll
+                for (int l = j + 1; l < NB; ++l) p[l] = fma(-p[j], __shfl_sync(0xffffffffu, p[j], l), p[l]);
             }
-            for (; q < i; ++q) s0 = fma(a[i * TP + q], x[q * TP + c], s0);
-            x[i * TP + c] = -((s0 + s1) + (s2 + s3)) * s_rd[i];
+            if (lane < NB) {
+#pragma unroll
+                for (int j = 0; j < NB; ++j)
+                    if (j <= i) a[(c0 + i) * TP + c0 + j] = p[j];
+            }
+            if (lane == 0 && anybad) s_bad = 1;
+        } else if (kb > 0) {
+            inverse_block_row(a, x, s_rd, kb - 1, tid - 32, nth - 32, 1);
+        }
+        __syncthreads();
+        const int M = T - NB - c0;  // rows below
+        if (tid < M) {
+            const int r = c0 + NB + tid;
+            double p[NB];
+#pragma unroll
+            for (int j = 0; j < NB; ++j) p[j] = a[r * TP + c0 + j];
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                p[j] *= s_rd[c0 + j];
+#pragma unroll
+                for (int l = j + 1; l < NB; ++l) p[l] = fma(-p[j], a[(c0 + l) * TP + c0 + j], p[l]);
+            }
+#pragma unroll
+            for (int j = 0; j < NB; ++j) a[r * TP + c0 + j] = p[j];
+        }
+        __syncthreads();
+        // rank-16 update of the lower 16 x 16 tiles below and right of the panel
+        const int ty = tid / NB, tx = tid % NB;
+        for (int ta = 0; ta < M / NB; ++ta) {
+            const int r = c0 + NB + ta * NB + ty;
+            double row[NB];
+#pragma unroll
+            for (int q = 0; q < NB; ++q) row[q] = a[r * TP + c0 + q];
+            for (int tb = 0; tb <= ta; ++tb) {
+                const int c = c0 + NB + tb * NB + tx;
+                double s = a[r * TP + c];
+#pragma unroll
+                for (int q = 0; q < NB; ++q) s = fma(-row[q], a[c * TP + c0 + q], s);
+                if (c <= r) a[r * TP + c] = s;
+            }
         }
     }
     __syncthreads();
+    inverse_block_row(a, x, s_rd, T / NB - 1, tid, nth, 1);
     double* Db = Dinv + ((int64_t)z * nt + k) * T * T;
     for (int t = tid; t < T * T; t += nth) {
         const int r = t / T, q = t % T;
