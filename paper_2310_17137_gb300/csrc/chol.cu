@@ -11,8 +11,8 @@
 //      tensor cores in ozaki.cu); all blocks of a group advance together, one
 //      launch per phase;
 //   3. form the inverse factor L^{-1} tile by tile (diagonal tiles from the
-//      FP64 tile inverses, off-diagonal tiles by the block recurrence
-//      X_ik = -L_ii^{-1} sum_{j=k}^{i-1} L_ij X_jk) and store it packed in FP32.
+//      FP64 tile inverses, off-diagonal blocks by halves,
+//      [A 0; B C]^{-1} = [A^{-1} 0; -C^{-1} B A^{-1} C^{-1}]) and store it packed in FP32.
 // The per-step block solve Delta = L^{-T} (L^{-1} R_I) then becomes two
 // parallel triangular products instead of two sequential substitutions.
 #include <math.h>
@@ -437,68 +437,100 @@ __global__ void __launch_bounds__(256) lower_to_f32_kernel(double* A, int nt) {
     }
 }
 
-// Row of tiles i of L^{-1}: X_ik = -X_ii * sum_{j=k}^{i-1} L_ij X_jk for k < i
-// (X_ii = L_ii^{-1} is already packed).  Thread (tr, tc) owns rows 4 tr .. + 3
-// and columns 4 tc .. + 3 of the tile; L is staged transposed and X row-major,
-// so every K step is two 16-byte shared loads for 16 FMAs.
-constexpr int TQ = T + 4;  // padded stride: rows stay 16-byte aligned, transposed stores spread over banks
+// Off-diagonal tiles of the inverse, by halves: for a lower-triangular matrix
+// [A 0; B C] with A^{-1} and C^{-1} known, the block below is -C^{-1} (B A^{-1}).  Level h
+// joins neighbouring diagonal blocks of h tiles (all pairs, all blocks of the group in
+// one launch): T = B A^{-1}, then X = -C^{-1} T, both triangular times dense.
+// log2(nt) levels of two launches replace nt row-by-row launches, whose later ones
+// were a few hundred CTAs with up to nt dependent tile products each (GB300, b = 4096:
+// 5 blocks 10.5 -> 2.4 ms in all, 13 blocks 15.6 -> 5.9 ms).  T is kept in FP32 in the place of the FP64 factor tiles, which
+// nothing reads any more (the inverse uses the FP32 copies).
+//
+// One CTA of 128 threads per 64 x 64 output tile; K in slices of 32, copied
+// asynchronously one slice ahead.  Thread (tr, tc) owns rows tr + 8 u and columns
+// 4 tc .. + 3: per four K values 8 + 4 shared 16-byte loads (the first eight are
+// broadcasts) for 128 multiply-adds, as packed pairs.
+constexpr int kTriK = 32;
+constexpr int kTriThreads = 128;
+constexpr int kTriLda = kTriK + 4;  // padded rows: 16-byte aligned
 
-__global__ void __launch_bounds__(256) tri_inv_step_kernel(double* A, int nt, int i, int64_t blk0, int64_t ntri,
-                                                           float* Linv) {
-    __shared__ __align__(16) float slt[T * TQ];  // slt[p][r] = L_ij(r, p)
-    __shared__ __align__(16) float sx[T * TQ];   // sx[p][c]  = X_jk(p, c)
-    const int z = blockIdx.y, k = blockIdx.x, tid = threadIdx.x;
+__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+
+template <bool kSecond>
+__global__ void __launch_bounds__(kTriThreads) tri_join_kernel(double* A, int nt, int h, int64_t blk0, int64_t ntri,
+                                                               float* Linv) {
+    __shared__ __align__(16) float sa[2][T * kTriLda];  // left operand, row-major 64 x 32
+    __shared__ __align__(16) float sb[2][kTriK * T];    // right operand, 32 x 64
+    const int tid = threadIdx.x;
+    // the tiles with the longest sums first
+    const int npair = (nt + 2 * h - 1) / (2 * h);
+    const int pair = (int)blockIdx.x % npair, rest = (int)blockIdx.x / npair;
+    const int mid = pair * 2 * h + h;
+    const int i = kSecond ? mid + h - 1 - rest / h : mid + rest % h;
+    const int k = mid - h + (kSecond ? rest % h : rest / h);
+    if (i >= nt) return;
     const int64_t ld = (int64_t)nt * T;
-    double* Ab = A + (int64_t)z * ld * ld;
-    float* Lb = Linv + (blk0 + z) * ntri * T * T;
-    const int tr = tid / 16, tc = tid % 16;
-    float acc[4][4] = {};
-    auto kstep_product = [&]() {
-#pragma unroll 8
-        for (int p = 0; p < T; ++p) {
-            const float4 lv = *reinterpret_cast<const float4*>(&slt[p * TQ + 4 * tr]);
-            const float4 xv = *reinterpret_cast<const float4*>(&sx[p * TQ + 4 * tc]);
-            const float l4[4] = {lv.x, lv.y, lv.z, lv.w}, x4[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(l4[u], x4[v], acc[u][v]);
+    double* Ab = A + (int64_t)blockIdx.y * ld * ld;
+    float* Lb = Linv + (blk0 + blockIdx.y) * ntri * T * T;
+    const int j0 = kSecond ? mid : k, j1 = kSecond ? i : mid - 1;  // tiles of the sum
+    const int nslice = (j1 - j0 + 1) * (T / kTriK);
+    auto fetch = [&](int sl, int buf) {
+        const int j = j0 + sl / (T / kTriK), off = (sl % (T / kTriK)) * kTriK;
+        // left: L_ij (FP32 copy) or X_ij (packed); right: X_jk (packed) or T_jk
+        const float* la = kSecond ? Lb + packed_tile(i, j) * T * T : lf32_tile(Ab, ld, i, j);
+        const int64_t lda = kSecond ? T : 2 * ld;
+        const float* rb = kSecond ? lf32_tile(Ab, ld, k, j) : Lb + packed_tile(j, k) * T * T;
+        const int64_t ldb = kSecond ? 2 * ld : T;
+        for (int t = tid; t < T * kTriK / 4; t += kTriThreads) {
+            const int r = t / (kTriK / 4), q = 4 * (t % (kTriK / 4));
+            cp_async16(&sa[buf][r * kTriLda + q], la + r * lda + off + q);
+            const int rr = t / (T / 4), qq = 4 * (t % (T / 4));
+            cp_async16(&sb[buf][rr * T + qq], rb + (int64_t)(off + rr) * ldb + qq);
         }
+        asm volatile("cp.async.commit_group;");
     };
-    for (int j = k; j < i; ++j) {
-        __syncthreads();
-        const float* Lij = lf32_tile(Ab, ld, i, j);
-        const float* Xjk = Lb + packed_tile(j, k) * T * T;
-        for (int t = tid; t < T * T; t += 256) {
-            const int r = t / T, q = t % T;
-            slt[q * TQ + r] = Lij[(int64_t)r * 2 * ld + q];
-            sx[r * TQ + q] = Xjk[t];
+    const int tr = tid / 16, tc = tid % 16;
+    float2 acc[8][2];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc[u][0] = acc[u][1] = make_float2(0.0f, 0.0f);
+    fetch(0, 0);
+    for (int sl = 0; sl < nslice; ++sl) {
+        const int buf = sl & 1;
+        if (sl + 1 < nslice) {
+            fetch(sl + 1, buf ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
-        kstep_product();
+#pragma unroll 2
+        for (int p = 0; p < kTriK; p += 4) {
+            float4 av[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) av[u] = *reinterpret_cast<const float4*>(&sa[buf][(tr + 8 * u) * kTriLda + p]);
+#pragma unroll
+            for (int pp = 0; pp < 4; ++pp) {
+                const float4 bv = *reinterpret_cast<const float4*>(&sb[buf][(p + pp) * T + 4 * tc]);
+                const float2 b0 = make_float2(bv.x, bv.y), b1 = make_float2(bv.z, bv.w);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const float a = pp == 0 ? av[u].x : pp == 1 ? av[u].y : pp == 2 ? av[u].z : av[u].w;
+                    acc[u][0] = __ffma2_rn(make_float2(a, a), b0, acc[u][0]);
+                    acc[u][1] = __ffma2_rn(make_float2(a, a), b1, acc[u][1]);
+                }
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    // out = X_ii acc: X_ii staged transposed like L, acc row-major like X
-    const float* Xii = Lb + packed_tile(i, i) * T * T;
-    for (int t = tid; t < T * T; t += 256) {
-        const int r = t / T, q = t % T;
-        slt[q * TQ + r] = Xii[t];
-    }
+    float* dst = kSecond ? Lb + packed_tile(i, k) * T * T : lf32_tile(Ab, ld, k, i);
+    const int64_t ldd = kSecond ? T : 2 * ld;
+    const float sg = kSecond ? -1.0f : 1.0f;
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-        *reinterpret_cast<float4*>(&sx[(4 * tr + u) * TQ + 4 * tc]) =
-            make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0f;
-    __syncthreads();
-    kstep_product();
-    float* dst = Lb + packed_tile(i, k) * T * T;
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        *reinterpret_cast<float4*>(&dst[(4 * tr + u) * T + 4 * tc]) =
-            make_float4(-acc[u][0], -acc[u][1], -acc[u][2], -acc[u][3]);
+    for (int u = 0; u < 8; ++u)
+        *reinterpret_cast<float4*>(dst + (int64_t)(tr + 8 * u) * ldd + 4 * tc) =
+            make_float4(sg * acc[u][0].x, sg * acc[u][0].y, sg * acc[u][1].x, sg * acc[u][1].y);
 }
 
 }  // namespace
@@ -546,9 +578,11 @@ cudaError_t cache_factor_group(const CacheParams& cp, int64_t blk0, int g, doubl
     ++nl;
     lower_to_f32_kernel<<<dim3((unsigned)ntri, g), 256, 0, st>>>(A, nt);
     ++nl;
-    for (int i = 1; i < nt; ++i) {
-        tri_inv_step_kernel<<<dim3(i, g), 256, 0, st>>>(A, nt, i, blk0, ntri, Linv);
-        ++nl;
+    for (int h = 1; h < nt; h *= 2) {
+        const dim3 grid((unsigned)((nt + 2 * h - 1) / (2 * h) * h * h), g);
+        tri_join_kernel<false><<<grid, kTriThreads, 0, st>>>(A, nt, h, blk0, ntri, Linv);
+        tri_join_kernel<true><<<grid, kTriThreads, 0, st>>>(A, nt, h, blk0, ntri, Linv);
+        nl += 2;
     }
     if (launches) *launches += nl;
     return cudaGetLastError();
