@@ -33,6 +33,15 @@ class PhaseRange {
 };
 }  // namespace
 
+// What the host reads of a solve's progress: one block, one copy per look.  (Each copy
+// to pageable memory waits for the stream; three a look cost some 20 us of a small
+// model's epoch.)
+struct SolveState {
+    double colnorm[AP_MAX_RHS];  // ||R_:,c||^2
+    int nan_flag;                // a norm (or an input) was not finite
+    int tc_err;                  // a bounded device wait ran out
+};
+
 struct ap_ctx {
     int device = 0;  // current device at ap_create; every call runs with it current
     int64_t n = 0;
@@ -70,12 +79,15 @@ struct ap_ctx {
     int64_t gscr_alloc = 0, gtick_alloc = 0, pscr_alloc = 0, ptick_alloc = 0;
     int sol_tpc = 1, sol_maxj = 1;
     // always-present device scalars
-    double *norms = nullptr, *colnorm = nullptr, *gout = nullptr, *gpart = nullptr;
+    double *norms = nullptr, *gout = nullptr, *gpart = nullptr;
+    SolveState* state = nullptr;
+    // flags and tickets of `state` and the products are known to be zero: set when a call
+    // has read clean flags, so that the next one need not clear them
+    bool clean = false;
     int64_t gpart_alloc = 0;
     unsigned* ticket = nullptr;
     int* sel = nullptr;
     int64_t* step = nullptr;
-    int* nan_flag = nullptr;
     int* bad = nullptr;
     int* trace = nullptr;
     int64_t trace_alloc = 0;
@@ -97,7 +109,6 @@ struct ap_ctx {
     uint8_t *XA = nullptr, *XB = nullptr, *DT = nullptr;
     float* tc_scr = nullptr;  // boundary slots of tiles shared by two CTAs
     int* tc_tick = nullptr;
-    int* tc_err = nullptr;
     int64_t launches = 0;
     int r_tracked_c = 0;  // c of the solve whose residual R holds (0: none)
     int divergences = 0;  // low-precision runs rolled back to a checkpoint (this solve)
@@ -209,6 +220,28 @@ ap_status leave(ap_ctx* ctx) {
     return AP_OK;
 }
 
+// Flags and arrival tickets to zero (a launch that gave up on a wait leaves tickets
+// partial) unless the last call left them so.  Until this call has read clean flags
+// itself they count as unknown.
+ap_status clear_flags(ap_ctx* ctx) {
+    if (!ctx->clean) {
+        AP_CK(cudaMemsetAsync(ctx->state, 0, sizeof(SolveState), ctx->st));
+        AP_CK(cudaMemsetAsync(ctx->ticket, 0, 4 * sizeof(unsigned), ctx->st));
+        if (ctx->gtick) AP_CK(cudaMemsetAsync(ctx->gtick, 0, sizeof(unsigned) * ctx->gtick_alloc, ctx->st));
+        if (ctx->tc_tick) AP_CK(cudaMemsetAsync(ctx->tc_tick, 0, sizeof(int) * ctx->num_sms, ctx->st));
+    }
+    ctx->clean = false;
+    return AP_OK;
+}
+
+// Copy the state to the host (waits for the stream).
+ap_status read_state(ap_ctx* ctx, SolveState* out) {
+    AP_CK(cudaMemcpyAsync(out, ctx->state, sizeof(SolveState), cudaMemcpyDeviceToHost, ctx->st));
+    AP_CK(cudaStreamSynchronize(ctx->st));
+    ctx->clean = !out->nan_flag && !out->tc_err;
+    return AP_OK;
+}
+
 int choose_split(int64_t ntiles, int64_t ncols) {
     int S = 1;
     while (S < kMaxSplit && ntiles * S < 4 * 152 && ncols / (2 * S) >= kKmvTN) S *= 2;
@@ -275,7 +308,7 @@ Shape comp_shape(const ap_ctx* ctx, int64_t ncols) {
     return sh;
 }
 
-constexpr int64_t kNormRows = 512;
+constexpr int64_t kNormRows = 128;
 
 Shape norm_shape(const ap_ctx* ctx) {
     Shape sh;
@@ -299,12 +332,12 @@ EpiParams make_epi(ap_ctx* ctx, int flags, int advance, const Shape& sh) {
     e.part_col = ctx->part_col;
     e.ticket = ctx->ticket;
     e.norms_out = ctx->norms;
-    e.colnorm_out = ctx->colnorm;
+    e.colnorm_out = ctx->state->colnorm;
     e.select = ctx->o.select;
     e.seed = ctx->o.seed;
     e.step_ctr = ctx->step;
     e.sel_out = ctx->sel;
-    e.nan_flag = ctx->nan_flag;
+    e.nan_flag = &ctx->state->nan_flag;
     return e;
 }
 
@@ -316,7 +349,7 @@ ap_status prep_inputs(ap_ctx* ctx, const float* X, int64_t n, float* out, float*
         sh[k] = (float)sc;
         sl[k] = (float)(sc - (double)sh[k]);
     }
-    AP_CK(launch_prep_inputs(X, n, ctx->d, ctx->D, sh, sl, out, out_lo, ctx->nan_flag, ctx->st));
+    AP_CK(launch_prep_inputs(X, n, ctx->d, ctx->D, sh, sl, out, out_lo, &ctx->state->nan_flag, ctx->st));
     ++ctx->launches;
     return AP_OK;
 }
@@ -330,7 +363,7 @@ bool use_compensated(const ap_ctx* ctx) {
 ap_status build_cache(ap_ctx* ctx) {
     PhaseRange range("ap: Cholesky cache (prep, K_II, FP64 factor, inverse)");
     drop_graph(ctx);
-    AP_CK(cudaMemsetAsync(ctx->nan_flag, 0, sizeof(int), ctx->st));
+    AP_TRY(clear_flags(ctx));
     AP_TRY(prep_inputs(ctx, ctx->X, ctx->n, ctx->Xs, ctx->Xs_lo));
     if (ctx->tc) {
         AP_CK(launch_tc_pack_inputs(ctx->kernel, ctx->Xs, ctx->n, ctx->d, ctx->D, ctx->b, ctx->m, ctx->tps128, ctx->cpb, ctx->kd,
@@ -377,8 +410,7 @@ ap_status build_cache(ap_ctx* ctx) {
             return s;
         }
     }
-    const OzWork oz = {ozS, ozE, ctx->tc_err};
-    AP_CK(cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->st));
+    const OzWork oz = {ozS, ozE, &ctx->state->tc_err};
     AP_CK(cudaMemsetAsync(ctx->bad, 0, sizeof(int) * ctx->m, ctx->st));
     CacheParams cp = {};
     cp.X = ctx->X;
@@ -407,11 +439,10 @@ ap_status build_cache(ap_ctx* ctx) {
     dfree(ctx, Dinv);
     dfree(ctx, ozS);
     dfree(ctx, ozE);
-    int tmo = 0, nanx = 0;
-    AP_CK(cudaMemcpy(&tmo, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-    AP_CK(cudaMemcpy(&nanx, ctx->nan_flag, sizeof(int), cudaMemcpyDeviceToHost));
-    if (nanx) return AP_ERR_NAN;  // a NaN or Inf training input
-    if (tmo) return AP_ERR_TIMEOUT;
+    SolveState now = {};
+    AP_TRY(read_state(ctx, &now));
+    if (now.nan_flag) return AP_ERR_NAN;  // a NaN or Inf training input
+    if (now.tc_err) return AP_ERR_TIMEOUT;
     std::vector<int> bad((size_t)ctx->m);
     AP_CK(cudaMemcpy(bad.data(), ctx->bad, sizeof(int) * ctx->m, cudaMemcpyDeviceToHost));
     for (int64_t J = 0; J < ctx->m; ++J)
@@ -453,8 +484,8 @@ ap_status ensure_solve(ap_ctx* ctx, int Cp) {
         if (ctx->tc) AP_TRY(dalloc_t(ctx, &ctx->W_ckpt, nc));
         AP_TRY(dalloc_t(ctx, &ctx->Z, (size_t)ctx->nt * kTile * Cp));
         AP_TRY(dalloc_t(ctx, &ctx->Delta, (size_t)ctx->b * Cp));
-        block_solve_layout(ctx->nt, ctx->num_sms, &ctx->sol_tpc, &ctx->sol_maxj);
-        AP_TRY(dalloc_t(ctx, &ctx->spart, (size_t)ctx->nt * ctx->sol_maxj * kTile * std::max(Cp, 4)));
+        block_solve_layout(ctx->nt, Cp, ctx->num_sms, &ctx->sol_tpc, &ctx->sol_maxj);
+        AP_TRY(dalloc_t(ctx, &ctx->spart, (size_t)ctx->nt * ctx->sol_maxj * kTile * Cp));
         AP_TRY(dalloc_t(ctx, &ctx->sticket, (size_t)ctx->nt));
         AP_CK(cudaMemsetAsync(ctx->sticket, 0, sizeof(unsigned) * ctx->nt, ctx->st));
         const KmvSplit a = step_split(ctx, Cp, ctx->b), b = step_split(ctx, Cp, ctx->n);
@@ -466,6 +497,8 @@ ap_status ensure_solve(ap_ctx* ctx, int Cp) {
         if (ctx->tc) {
             dfree(ctx, ctx->DT);
             AP_TRY(dalloc_t(ctx, &ctx->DT, tc_delta_bytes(ctx->cpb, Cp)));
+            // (the block solve fills the rows of its tiles; a last half chunk stays zero)
+            AP_CK(cudaMemsetAsync(ctx->DT, 0, tc_delta_bytes(ctx->cpb, Cp), ctx->st));
         }
         dfree(ctx, ctx->part_norm);
         AP_TRY(dalloc_t(ctx, &ctx->part_norm, (size_t)need));
@@ -510,11 +543,10 @@ ap_status launch_step(ap_ctx* ctx, bool colnorms, int64_t j) {
     sp.maxj = ctx->sol_maxj;
     sp.spart = ctx->spart;
     sp.sticket = ctx->sticket;
+    sp.DT = ctx->tc_steps ? ctx->DT : nullptr;
+    // timing events between the kernels measure them one by one
+    sp.dependent = !prof;
     AP_CK(launch_block_solve(sp, ctx->st, &ctx->launches));
-    if (ctx->tc_steps) {
-        AP_CK(launch_tc_pack_delta(ctx->Delta, ctx->b, Cp, ctx->cpb, ctx->DT, ctx->st));
-        ++ctx->launches;
-    }
     if (prof) {
         AP_CK(cudaEventRecordWithFlags(ctx->ev_bs[2 * j + 1], ctx->st, rec_flags));
         AP_CK(cudaEventRecordWithFlags(ctx->ev_up[2 * j], ctx->st, rec_flags));
@@ -537,7 +569,7 @@ ap_status launch_step(ap_ctx* ctx, bool colnorms, int64_t j) {
         tl.s = ctx->s;
         tl.noise = ctx->noise;
         tl.sel = ctx->sel;
-        tl.err = ctx->tc_err;
+        tl.err = &ctx->state->tc_err;
         tl.wait_cycles = ctx->o.wait_limit_cycles;
         tl.scr = ctx->tc_scr;
         tl.tick = ctx->tc_tick;
@@ -565,7 +597,8 @@ ap_status launch_step(ap_ctx* ctx, bool colnorms, int64_t j) {
     kp.noise_diag = 1;
     kp.sel = ctx->sel;
     kp.blk = ctx->b;
-    kp.err = ctx->tc_err;
+    kp.dependent = !prof;
+    kp.err = &ctx->state->tc_err;
     kp.epi = make_epi(ctx, kEpiBlockNorms | (colnorms ? kEpiColNorms : 0), 1, sh);
     AP_CK(launch_kmv(ctx->kernel, kp, ctx->D, Cp, ctx->st));
     ++ctx->launches;
@@ -588,19 +621,10 @@ void collect_profile(ap_ctx* ctx, int64_t steps) {
     cudaGetLastError();
 }
 
-// Clear the timeout flag and the arrival tickets (a launch that gave up on a wait
-// leaves them partial).
-ap_status reset_waits(ap_ctx* ctx) {
-    AP_CK(cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->st));
-    AP_CK(cudaMemsetAsync(ctx->ticket, 0, 4 * sizeof(unsigned), ctx->st));
-    if (ctx->gtick) AP_CK(cudaMemsetAsync(ctx->gtick, 0, sizeof(unsigned) * ctx->gtick_alloc, ctx->st));
-    if (ctx->tc_tick) AP_CK(cudaMemsetAsync(ctx->tc_tick, 0, sizeof(int) * ctx->num_sms, ctx->st));
-    return AP_OK;
-}
-
 // out = base - K_hat V over all n columns (the FP32 residual recompute).
 ap_status launch_full_residual(ap_ctx* ctx, const float* base, const float* V, float* out, int flags) {
     PhaseRange range("ap: residual recompute R = B - K_hat W");
+    ctx->clean = false;
     const bool comp = use_compensated(ctx);
     ctx->comp_used = comp;
     // without block norms the row tiles need not respect the blocks
@@ -624,7 +648,7 @@ ap_status launch_full_residual(ap_ctx* ctx, const float* base, const float* V, f
     kp.ncols = ctx->n;
     kp.Xa_lo = ctx->Xs_lo;
     kp.Xb_lo = ctx->Xs_lo;
-    kp.err = ctx->tc_err;
+    kp.err = &ctx->state->tc_err;
     kp.epi = make_epi(ctx, flags, 0, sh);
     if (!blocks) kp.epi.seg = ctx->n;
     if (comp) AP_CK(launch_kmv_comp(ctx->kernel, kp, ctx->D, ctx->Cp, ctx->st));
@@ -663,7 +687,7 @@ ap_status run_epoch(ap_ctx* ctx, int64_t steps) {
         }
         if (ctx->graph) {
             AP_CK(cudaGraphLaunch(ctx->graph, ctx->st));
-            ctx->launches += (ctx->tc_steps ? 4 : 3) * steps;
+            ctx->launches += 3 * steps;
             return AP_OK;
         }
     }
@@ -759,28 +783,23 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
     if (ctx->graph && ctx->graph_tc != ctx->tc_steps) drop_graph(ctx);
     int fp32_epochs = 0;
     AP_TRY(enter(ctx));
-    AP_CK(launch_pad_copy(B_dev, ctx->n, c, ctx->Bp, Cp, ctx->st));
-    ++ctx->launches;
+    AP_TRY(clear_flags(ctx));
     AP_CK(cudaMemsetAsync(ctx->step, 0, sizeof(int64_t), ctx->st));
-    AP_CK(cudaMemsetAsync(ctx->nan_flag, 0, sizeof(int), ctx->st));
-    AP_TRY(reset_waits(ctx));
-    // ||b_c|| for the relative residuals
-    AP_TRY(launch_norms(ctx, ctx->Bp, kEpiColNorms));
-    double bn[AP_MAX_RHS] = {}, rn[AP_MAX_RHS] = {};
-    AP_CK(cudaMemcpyAsync(bn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
+    // ||b_c|| for the relative residuals, and the first block; without W0, R = B
+    SolveState now = {};
+    double bn[AP_MAX_RHS] = {};
+    const double* rn = now.colnorm;
+    AP_CK(launch_init_solve(B_dev, W0_dev, ctx->n, c, Cp, ctx->Bp, W0_dev ? nullptr : ctx->R, ctx->W,
+                            ctx->tc ? ctx->W_ckpt : nullptr, ctx->st));
+    ++ctx->launches;
+    AP_TRY(launch_norms(ctx, ctx->Bp, kEpiColNorms | (W0_dev ? 0 : kEpiBlockNorms)));
+    AP_TRY(read_state(ctx, &now));
+    for (int k = 0; k < Cp; ++k) bn[k] = now.colnorm[k];
     if (W0_dev) {
-        AP_CK(launch_pad_copy(W0_dev, ctx->n, c, ctx->W, Cp, ctx->st));
-        ++ctx->launches;
         AP_TRY(launch_full_residual(ctx, ctx->Bp, ctx->W, ctx->R, 0));
-    } else {
-        AP_CK(cudaMemsetAsync(ctx->W, 0, sizeof(float) * ctx->n * Cp, ctx->st));
-        AP_CK(cudaMemcpyAsync(ctx->R, ctx->Bp, sizeof(float) * ctx->n * Cp, cudaMemcpyDeviceToDevice, ctx->st));
+        AP_TRY(launch_norms(ctx, ctx->R, kEpiBlockNorms | kEpiColNorms));
+        AP_TRY(read_state(ctx, &now));
     }
-    AP_TRY(launch_norms(ctx, ctx->R, kEpiBlockNorms | kEpiColNorms));
-    AP_CK(cudaMemcpyAsync(rn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
-    if (ctx->tc)
-        AP_CK(cudaMemcpyAsync(ctx->W_ckpt, ctx->W, sizeof(float) * ctx->n * Cp, cudaMemcpyDeviceToDevice, ctx->st));
-    AP_CK(cudaStreamSynchronize(ctx->st));
 
     double rel[AP_MAX_RHS] = {}, rel_true[AP_MAX_RHS] = {};
     bool have_true = false;
@@ -812,17 +831,14 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
         if (ctx->o.max_steps > 0) ns = std::min<int64_t>(ns, ctx->o.max_steps - steps);
         if (ns <= 0) break;
         PhaseRange epoch_range(ctx->tc_steps ? "ap: epoch (tensor-core update)" : "ap: epoch (FP32 update)");
+        ctx->clean = false;
         AP_TRY(run_epoch(ctx, ns));
         steps += ns;
         ++epoch;
         if (ctx->tc && !ctx->tc_steps) ++fp32_epochs;
-        int nanf = 0, tcerr = 0;
-        AP_CK(cudaMemcpyAsync(rn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
-        AP_CK(cudaMemcpyAsync(&nanf, ctx->nan_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-        AP_CK(cudaMemcpyAsync(&tcerr, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-        AP_CK(cudaStreamSynchronize(ctx->st));
+        AP_TRY(read_state(ctx, &now));
         collect_profile(ctx, ns);
-        if (tcerr) {
+        if (now.tc_err) {
             status = AP_ERR_TIMEOUT;
             break;
         }
@@ -832,19 +848,16 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
         // smooth kernels): a NaN, or a tracked residual above twice the last
         // certified one.  Roll W back to the last checkpoint, recompute R and
         // continue with the FP32 update.
-        if (ctx->tc_steps && ctx->o.escalate && (nanf || !(rule_measure(ctx->o.stop, c, rel, bn) <= 2.0 * true_prev))) {
+        if (ctx->tc_steps && ctx->o.escalate && (now.nan_flag || !(rule_measure(ctx->o.stop, c, rel, bn) <= 2.0 * true_prev))) {
             ctx->tc_steps = false;
             drop_graph(ctx);
             AP_CK(cudaMemcpyAsync(ctx->W, ctx->W_ckpt, sizeof(float) * ctx->n * Cp, cudaMemcpyDeviceToDevice, ctx->st));
-            AP_CK(cudaMemsetAsync(ctx->nan_flag, 0, sizeof(int), ctx->st));
+            AP_CK(cudaMemsetAsync(&ctx->state->nan_flag, 0, sizeof(int), ctx->st));
             AP_CK(cudaEventRecord(ctx->ev_r0, ctx->st));
             AP_TRY(launch_full_residual(ctx, ctx->Bp, ctx->W, ctx->R, kEpiBlockNorms | kEpiColNorms));
             AP_CK(cudaEventRecord(ctx->ev_r1, ctx->st));
-            AP_CK(cudaMemcpyAsync(rn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
-            AP_CK(cudaMemcpyAsync(&nanf, ctx->nan_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-            AP_CK(cudaMemcpyAsync(&tcerr, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-            AP_CK(cudaStreamSynchronize(ctx->st));
-            if (tcerr) {
+            AP_TRY(read_state(ctx, &now));
+            if (now.tc_err) {
                 status = AP_ERR_TIMEOUT;
                 break;
             }
@@ -859,7 +872,7 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
             for (int k = 0; k < c; ++k) rel_true[k] = rel[k];
             true_prev = rule_measure(ctx->o.stop, c, rel, bn);
         }
-        if (nanf) {
+        if (now.nan_flag) {
             status = AP_ERR_NAN;
             break;
         }
@@ -871,11 +884,8 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
             AP_CK(cudaEventRecord(ctx->ev_r0, ctx->st));
             AP_TRY(launch_full_residual(ctx, ctx->Bp, ctx->W, ctx->R, kEpiBlockNorms | kEpiColNorms));
             AP_CK(cudaEventRecord(ctx->ev_r1, ctx->st));
-            AP_CK(cudaMemcpyAsync(rn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
-            AP_CK(cudaMemcpyAsync(&nanf, ctx->nan_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-            AP_CK(cudaMemcpyAsync(&tcerr, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-            AP_CK(cudaStreamSynchronize(ctx->st));
-            if (tcerr) {
+            AP_TRY(read_state(ctx, &now));
+            if (now.tc_err) {
                 status = AP_ERR_TIMEOUT;
                 break;
             }
@@ -883,7 +893,7 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
             cudaEventElapsedTime(&rms, ctx->ev_r0, ctx->ev_r1);
             t_refine += rms * 1e-3;
             ++refinements;
-            if (nanf) {
+            if (now.nan_flag) {
                 status = AP_ERR_NAN;
                 break;
             }
@@ -931,11 +941,8 @@ ap_status solve_impl(ap_ctx* ctx, const float* B_dev, int c, const float* W0_dev
         AP_CK(cudaEventRecord(ctx->ev_r0, ctx->st));
         AP_TRY(launch_full_residual(ctx, ctx->Bp, ctx->W, ctx->R, kEpiColNorms));
         AP_CK(cudaEventRecord(ctx->ev_r1, ctx->st));
-        int tcerr = 0;
-        AP_CK(cudaMemcpyAsync(rn, ctx->colnorm, sizeof(double) * Cp, cudaMemcpyDeviceToHost, ctx->st));
-        AP_CK(cudaMemcpyAsync(&tcerr, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-        AP_CK(cudaStreamSynchronize(ctx->st));
-        if (tcerr) status = AP_ERR_TIMEOUT;
+        AP_TRY(read_state(ctx, &now));
+        if (now.tc_err) status = AP_ERR_TIMEOUT;
         float rms = 0.f;
         cudaEventElapsedTime(&rms, ctx->ev_r0, ctx->ev_r1);
         t_refine += rms * 1e-3;
@@ -1150,28 +1157,20 @@ ap_status ap_create(ap_ctx** out, const float* X_dev, int64_t n, int32_t d, cons
     if ((s = dalloc_t(ctx, &ctx->Xs, (size_t)(n * ctx->D))) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->Xs_lo, (size_t)(n * ctx->D))) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->norms, (size_t)ctx->m)) != AP_OK) return fail(s);
-    if ((s = dalloc_t(ctx, &ctx->colnorm, AP_MAX_RHS)) != AP_OK) return fail(s);
+    if ((s = dalloc_t(ctx, &ctx->state, 1)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->gout, AP_MAX_DIM + 4)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->ticket, 4)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->sel, 1)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->step, 1)) != AP_OK) return fail(s);
-    if ((s = dalloc_t(ctx, &ctx->nan_flag, 1)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->bad, (size_t)ctx->m)) != AP_OK) return fail(s);
-    if ((s = dalloc_t(ctx, &ctx->tc_err, 1)) != AP_OK) return fail(s);
     if (ctx->tc) {
         if ((s = dalloc_t(ctx, &ctx->XA, tc_rows_bytes(ctx->m * ctx->tps128, ctx->kd))) != AP_OK) return fail(s);
         if ((s = dalloc_t(ctx, &ctx->XB, tc_cols_bytes(ctx->m, ctx->cpb, ctx->kd))) != AP_OK) return fail(s);
         if ((s = dalloc_t(ctx, &ctx->tc_scr, tc_share_bytes(ctx->num_sms, AP_MAX_RHS) / sizeof(float))) != AP_OK)
             return fail(s);
         if ((s = dalloc_t(ctx, &ctx->tc_tick, (size_t)ctx->num_sms)) != AP_OK) return fail(s);
-        if (cudaMemsetAsync(ctx->tc_tick, 0, sizeof(int) * ctx->num_sms, ctx->st) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(AP_ERR_CUDA);
-        }
     }
-    if (cudaMemsetAsync(ctx->ticket, 0, 4 * sizeof(unsigned), ctx->st) != cudaSuccess ||
-        cudaMemsetAsync(ctx->tc_err, 0, sizeof(int), ctx->st) != cudaSuccess ||
-        cudaMemsetAsync(ctx->sel, 0, sizeof(int), ctx->st) != cudaSuccess) {
+    if (cudaMemsetAsync(ctx->sel, 0, sizeof(int), ctx->st) != cudaSuccess) {
         cudaGetLastError();
         return fail(AP_ERR_CUDA);
     }
@@ -1257,17 +1256,17 @@ ap_status ap_residual(ap_ctx* ctx, const float* B_dev, int32_t c, const float* W
     ctx->r_tracked_c = 0;
     AP_TRY(enter(ctx));
     const bool waits = Cp >= kX3MinC && !use_compensated(ctx);  // the tensor-core form runs
-    if (waits) AP_TRY(reset_waits(ctx));
+    if (waits) AP_TRY(clear_flags(ctx));
     AP_CK(launch_pad_copy(B_dev, ctx->n, c, ctx->Bp, Cp, ctx->st));
     AP_CK(launch_pad_copy(W_dev, ctx->n, c, ctx->Tmp, Cp, ctx->st));
     ctx->launches += 2;
     AP_TRY(launch_full_residual(ctx, ctx->Bp, ctx->Tmp, ctx->R, 0));
     AP_CK(launch_unpad_copy(ctx->R, ctx->n, Cp, R_dev, c, ctx->st));
     ++ctx->launches;
-    int tmo = 0;
-    if (waits) AP_CK(cudaMemcpyAsync(&tmo, ctx->tc_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+    SolveState now = {};
+    if (waits) AP_TRY(read_state(ctx, &now));
     AP_TRY(leave(ctx));
-    return tmo ? AP_ERR_TIMEOUT : AP_OK;
+    return now.tc_err ? AP_ERR_TIMEOUT : AP_OK;
 }
 
 ap_status ap_predict_mean(ap_ctx* ctx, const float* w_dev, const float* Xs_dev, int64_t M, float* mean_dev) {
@@ -1281,7 +1280,7 @@ ap_status ap_predict_mean(ap_ctx* ctx, const float* w_dev, const float* Xs_dev, 
         ctx->Xt_alloc = M;
     }
     AP_TRY(enter(ctx));
-    AP_CK(cudaMemsetAsync(ctx->nan_flag, 0, sizeof(int), ctx->st));
+    AP_TRY(clear_flags(ctx));
     AP_TRY(prep_inputs(ctx, Xs_dev, M, ctx->Xt, nullptr));
     const KmvSplit split = kmv_split(ctx->D, 1, M, 1, ctx->n);
     AP_TRY(grow_groups(ctx, split, &ctx->pscr, &ctx->pscr_alloc, &ctx->ptick, &ctx->ptick_alloc));
@@ -1306,10 +1305,10 @@ ap_status ap_predict_mean(ap_ctx* ctx, const float* w_dev, const float* Xs_dev, 
     kp.epi.seg = M;
     AP_CK(launch_kmv(ctx->kernel, kp, ctx->D, 1, ctx->st));
     ++ctx->launches;
-    int nanx = 0;
-    AP_CK(cudaMemcpyAsync(&nanx, ctx->nan_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+    SolveState now = {};
+    AP_TRY(read_state(ctx, &now));
     AP_TRY(leave(ctx));
-    return nanx ? AP_ERR_NAN : AP_OK;
+    return now.nan_flag ? AP_ERR_NAN : AP_OK;
 }
 
 static ap_status grad_quadforms_impl(ap_ctx* ctx, const float* U, const float* V, int Cp, const double* alpha,

@@ -2,6 +2,7 @@
 // Nothing here is part of the public ABI (include/ap.h is).
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -39,6 +40,39 @@ constexpr int kTile = 64;           // tile edge of the block-Cholesky cache
 constexpr int kKmvThreads = 128;    // threads per CTA of the kernel-matrix products
 constexpr int kKmvTN = 64;          // columns staged per shared-memory chunk
 constexpr int kMaxSplit = 8;        // portable thread-block-cluster size
+
+// Programmatic dependent launch between the kernels of an AP step: a kernel launched
+// with launch_dependent may start once every CTA of the kernel before has passed its
+// pdl_launch (or ended); what that kernel writes is read after pdl_wait.  Every kernel
+// of the chain waits before it lets its successor go, so that anything a kernel two
+// places back wrote is complete and visible from the start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename P>
+cudaError_t launch_dependent(void (*fn)(P), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, bool dependent,
+                             const P& p, unsigned cluster_y = 1) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    unsigned n = 0;
+    if (dependent) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster_y > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = 1;
+        attr[n].val.clusterDim.y = cluster_y;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, fn, p);
+}
 
 // flags of the kernel-matrix product epilogue
 constexpr int kEpiBlockNorms = 1;   // per-block ||R_J||_F^2 partials + block selection
@@ -97,6 +131,7 @@ struct KmvParams {
     float* gscr;           // G > 1: partial sums (KmvSplit::scratch floats)
     unsigned int* gtick;   // G > 1: arrival tickets (KmvSplit::tickets), zero between launches
     int* err;              // wait-timeout flag of the tensor-core form
+    bool dependent;        // launch without waiting for the kernel before (launch_dependent)
     EpiParams epi;
 };
 
@@ -187,11 +222,13 @@ struct SolveParams {
     int64_t trace_cap;
     int tpc;               // tiles per CTA (block_solve_layout)
     int maxj;              // partial slots per output row of tiles
-    float* spart;          // nt * maxj * 64 * max(C, 4) floats of partial sums
+    float* spart;          // nt * maxj * 64 * C floats of partial sums
     unsigned* sticket;     // nt tickets, zero between launches
+    uint8_t* DT;           // tensor-core form: operand layout of Delta to fill too, or nullptr
+    bool dependent;        // launch without waiting for the kernel before (launch_dependent)
 };
-// Work split of the block solve for nt tiles per block edge on num_sms SMs.
-void block_solve_layout(int nt, int num_sms, int* tpc, int* maxj);
+// Work split of the block solve for nt tiles per block edge and C right-hand sides.
+void block_solve_layout(int nt, int C, int num_sms, int* tpc, int* maxj);
 cudaError_t launch_block_solve(const SolveParams& p, cudaStream_t st, int64_t* launches);
 
 // ---- small helpers ----------------------------------------------------------
@@ -199,6 +236,8 @@ cudaError_t launch_block_solve(const SolveParams& p, cudaStream_t st, int64_t* l
 // gets the remainder X * sc - Xs to FP32 precision.
 cudaError_t launch_prep_inputs(const float* X, int64_t n, int d, int D, const float* sc_hi, const float* sc_lo,
                                float* Xs, float* Xs_lo, int* bad, cudaStream_t st);
+cudaError_t launch_init_solve(const float* B, const float* W0, int64_t n, int c, int C, float* Bp, float* R, float* W,
+                              float* W_ckpt, cudaStream_t st);
 cudaError_t launch_pad_copy(const float* src, int64_t n, int c, float* dst, int C, cudaStream_t st);
 cudaError_t launch_unpad_copy(const float* src, int64_t n, int C, float* dst, int c, cudaStream_t st);
 
@@ -238,6 +277,19 @@ cudaError_t launch_dot0(const float* W, int C, const float* Y, int cy, int64_t n
                        double* out, cudaStream_t st);
 
 // ---- tensor-core form of the residual update (kmv_tc.cu) -------------------
+constexpr int kTcChunk = 128;  // columns of the block per chunk
+// One value of Delta^T in the contraction's operand layout: per 128-column chunk C rows
+// (right-hand sides) x 128 columns (block-local points) as BF16 hi, then lo, K-major core
+// matrices of 8 rows x 8 halves (16 K-cores per row group).
+__device__ __forceinline__ void tc_store_delta(uint8_t* DT, int C, int64_t li, int c, float v) {
+    const int k = (int)(li % kTcChunk);
+    const size_t half_bytes = (size_t)C * kTcChunk * 2;
+    uint8_t* dst = DT + (size_t)(li / kTcChunk) * 2 * half_bytes +
+                   ((size_t)((c >> 3) * (kTcChunk / 8) + (k >> 3)) * 8 + (c & 7)) * 16 + (size_t)(k & 7) * 2;
+    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+    *reinterpret_cast<__nv_bfloat16*>(dst) = hi;
+    *reinterpret_cast<__nv_bfloat16*>(dst + half_bytes) = __float2bfloat16_rn(v - __bfloat162float(hi));
+}
 struct TcParams;
 int tc_kd(int d);
 int tc_chunks_per_block(int64_t b);
@@ -246,7 +298,6 @@ size_t tc_cols_bytes(int64_t m, int cpb, int kd);
 size_t tc_delta_bytes(int cpb, int C);
 cudaError_t launch_tc_pack_inputs(int kernel, const float* Xs, int64_t n, int d, int D, int64_t b, int64_t m,
                                   int64_t tps, int cpb, int kd, uint8_t* XA, uint8_t* XB, cudaStream_t st);
-cudaError_t launch_tc_pack_delta(const float* Delta, int64_t b, int C, int cpb, uint8_t* DT, cudaStream_t st);
 struct TcLaunch {
     const uint8_t* XA;
     const uint8_t* XB;

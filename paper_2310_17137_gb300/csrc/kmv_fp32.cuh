@@ -317,6 +317,8 @@ __global__ void __launch_bounds__(kKmvThreads, 4) kmv_fp32_kernel(const KmvParam
             xa[q][4 * k4 + 3] = v.w;
         }
     }
+    pdl_wait();  // V and base (the block index was complete before the block solve began)
+    pdl_launch();
     float2 xa2[RM][D / 2], acc2[RM][(C + 1) / 2];
 #pragma unroll
     for (int q = 0; q < RM; ++q) {
@@ -457,22 +459,8 @@ cudaError_t launch_kmv_rm(const KmvParams& p, cudaStream_t st) {
     auto fn = kmv_fp32_kernel<KERN, D, C, RM>;
     cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    const int S = p.epi.S;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)p.epi.ntiles, (unsigned)S, (unsigned)p.G);
-    cfg.blockDim = dim3(kKmvThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    if (S > 1) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 1;
-        attr[0].val.clusterDim.y = (unsigned)S;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
-    return cudaLaunchKernelEx(&cfg, fn, p);
+    return launch_dependent(fn, dim3((unsigned)p.epi.ntiles, (unsigned)p.epi.S, (unsigned)p.G), kKmvThreads, smem, st,
+                            p.dependent, p, (unsigned)p.epi.S);
 }
 
 // rows per thread as kmv_split chose them, at most what (D, C) leaves registers for

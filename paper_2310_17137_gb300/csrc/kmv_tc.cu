@@ -51,7 +51,7 @@ namespace ap {
 namespace tc {
 
 constexpr int kRows = 128;
-constexpr int kChunk = 128;  // columns of the block per chunk
+constexpr int kChunk = kTcChunk;  // columns of the block per chunk
 constexpr int kStages = 4;
 constexpr int kBufs = 3;     // S/P tensor-memory buffers
 constexpr int kColsPerWarp = 32;                   // columns of a chunk per work item (two 16-column units)
@@ -427,6 +427,9 @@ __global__ void __launch_bounds__(tc::kThreads, 1) kmv_tc_kernel(const TcParams 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    // (launched in stream order: as a dependent launch the persistent CTAs started before the
+    // block solve's and a step took 22 us longer)
+    pdl_launch();
 
     if (warp == kCopyWarp) {
         // ------------------------------------------------ bulk-copy issuer
@@ -813,26 +816,6 @@ __global__ void pack_cols_kernel(const float* __restrict__ Xs, int64_t n, int d,
     }
 }
 
-// Delta^T chunks of the current step: C rows (right-hand sides) x 128 columns
-// (block-local points) as BF16 hi/lo, K-major core matrices of 8 rows x 8
-// halves (16 K-cores per row group).
-__global__ void pack_delta_kernel(const float* __restrict__ Delta, int64_t b, int C, int cpb, uint8_t* __restrict__ DT) {
-    const int q = blockIdx.x;
-    const size_t half_bytes = (size_t)C * tc::kChunk * 2;
-    uint8_t* dst = DT + (size_t)q * 2 * half_bytes;
-    for (int t = threadIdx.x; t < C * tc::kChunk; t += blockDim.x) {
-        const int c = t / tc::kChunk, k = t % tc::kChunk;  // row c, K index k
-        const int64_t li = (int64_t)q * tc::kChunk + k;
-        const float v = li < b ? Delta[li * C + c] : 0.0f;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-        const size_t off =
-            ((size_t)((c >> 3) * (tc::kChunk / 8) + (k >> 3)) * 8 + (c & 7)) * 16 + (size_t)(k & 7) * 2;
-        *reinterpret_cast<__nv_bfloat16*>(dst + off) = hi;
-        *reinterpret_cast<__nv_bfloat16*>(dst + half_bytes + off) = lo;
-    }
-}
-
 template <int KERN, int C>
 cudaError_t launch_tc_inst(const TcParams& p, int grid, cudaStream_t st) {
     const size_t xa = (size_t)tc::kRows * p.kdp * 2, xb = (size_t)tc::kChunk * p.kdp * 2;
@@ -863,11 +846,6 @@ cudaError_t launch_tc_pack_inputs(int kernel, const float* Xs, int64_t n, int d,
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     pack_cols_kernel<<<(unsigned)(m * cpb), 256, 0, st>>>(Xs, n, d, D, b, cpb, kd, fold, XB);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_tc_pack_delta(const float* Delta, int64_t b, int C, int cpb, uint8_t* DT, cudaStream_t st) {
-    pack_delta_kernel<<<cpb, 256, 0, st>>>(Delta, b, C, cpb, DT);
     return cudaGetLastError();
 }
 

@@ -168,6 +168,8 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     const uint32_t tmem_p = tmem + K::kAccCols;
+    pdl_wait();  // V and base (the block index was complete before the block solve began)
+    pdl_launch();
 
     if (warp < kXformWarps) {
         // ------------------------------------------------------- transform warps
@@ -654,8 +656,7 @@ cudaError_t launch_inst(const KmvParams& p, cudaStream_t st) {
     auto fn = kmv_x3_kernel<KERN, D, C, R>;
     cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::kSmem);
     if (err != cudaSuccess) return err;
-    fn<<<(unsigned)p.ctas, K::kThreads, K::kSmem, st>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(fn, dim3((unsigned)p.ctas), K::kThreads, K::kSmem, st, p.dependent, p);
 }
 
 // (D, C, R) dispatch for one kernel family; rows per thread as kmv_split chose them.

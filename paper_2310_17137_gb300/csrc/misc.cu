@@ -133,6 +133,24 @@ __global__ void unpad_copy_kernel(const float* __restrict__ src, int64_t n, int 
     }
 }
 
+// Start of a solve in one pass over n x C: Bp = B padded, R = Bp (when the start is
+// zero), W = W0 padded or 0, W_ckpt = W.
+__global__ void init_solve_kernel(const float* __restrict__ B, const float* __restrict__ W0, int64_t n, int c, int C,
+                                  float* __restrict__ Bp, float* __restrict__ R, float* __restrict__ W,
+                                  float* __restrict__ W_ckpt) {
+    const int64_t total = n * C;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = t / C;
+        const int k = (int)(t % C);
+        const float b = k < c ? B[i * c + k] : 0.0f, w = W0 && k < c ? W0[i * c + k] : 0.0f;
+        Bp[t] = b;
+        if (R) R[t] = b;
+        W[t] = w;
+        if (W_ckpt) W_ckpt[t] = w;
+    }
+}
+
 unsigned grid_for(int64_t total) {
     int64_t g = (total + 255) / 256;
     if (g > 152 * 32) g = 152 * 32;
@@ -150,6 +168,12 @@ cudaError_t launch_prep_inputs(const float* X, int64_t n, int d, int D, const fl
         sl.v[k] = sc_lo ? sc_lo[k] : 0.0f;
     }
     prep_inputs_kernel<<<grid_for(n * D), 256, 0, st>>>(X, n, d, D, sh, sl, Xs, Xs_lo, bad);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_init_solve(const float* B, const float* W0, int64_t n, int c, int C, float* Bp, float* R, float* W,
+                              float* W_ckpt, cudaStream_t st) {
+    init_solve_kernel<<<grid_for(n * C), 256, 0, st>>>(B, W0, n, c, C, Bp, R, W, W_ckpt);
     return cudaGetLastError();
 }
 
