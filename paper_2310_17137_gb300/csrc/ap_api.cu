@@ -1313,33 +1313,32 @@ ap_status ap_predict_mean(ap_ctx* ctx, const float* w_dev, const float* Xs_dev, 
 
 static ap_status grad_quadforms_impl(ap_ctx* ctx, const float* U, const float* V, int Cp, const double* alpha,
                                      int c, double* out_host) {
-    const int64_t rows = grad_rows_per_cta(ctx->D, Cp);
-    const int64_t ntiles = (ctx->n + rows - 1) / rows;
-    const int S = choose_split(ntiles, ctx->n);
     const int NA = ctx->D + 2;
-    const int64_t need = std::max<int64_t>(ntiles * S * NA, 256);
+    const int64_t need = std::max<int64_t>((int64_t)kGradCtas * NA, 256);
     if (need > ctx->gpart_alloc) {
         dfree(ctx, ctx->gpart);
         ctx->gpart_alloc = 0;
         AP_TRY(dalloc_t(ctx, &ctx->gpart, (size_t)need));
         ctx->gpart_alloc = need;
     }
+    AP_TRY(clear_flags(ctx));
     GradParams gp = {};
     gp.Xs = ctx->Xs;
     gp.n = ctx->n;
     gp.U = U;
     gp.V = V;
     for (int k = 0; k < c; ++k) gp.alpha[k] = (float)alpha[k];
-    gp.ntiles = ntiles;
-    gp.S = S;
     gp.part = ctx->gpart;
+    gp.err = &ctx->state->tc_err;
     gp.ticket = ctx->ticket + 1;
     gp.out = ctx->gout;
     AP_CK(launch_grad(ctx->kernel, gp, ctx->D, Cp, ctx->st));
     ++ctx->launches;
     double raw[AP_MAX_DIM + 2] = {};
     AP_CK(cudaMemcpyAsync(raw, ctx->gout, sizeof(double) * NA, cudaMemcpyDeviceToHost, ctx->st));
-    AP_CK(cudaStreamSynchronize(ctx->st));
+    SolveState now = {};
+    AP_TRY(read_state(ctx, &now));
+    if (now.tc_err) return AP_ERR_TIMEOUT;
     const double fac = ctx->kernel == AP_RBF ? 2.0 / 1.4426950408889634 : (ctx->kernel == AP_MATERN32 ? 1.0 : 1.0 / 3.0);
     for (int k = 0; k < ctx->d; ++k) out_host[k] = (double)ctx->s * fac * raw[k] / (double)ctx->ell[k];
     out_host[ctx->d] = raw[ctx->D];

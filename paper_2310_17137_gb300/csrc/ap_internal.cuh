@@ -254,17 +254,16 @@ struct GradParams {
     const float* U;        // n x C
     const float* V;        // n x C
     float alpha[AP_MAX_RHS];
-    int64_t ntiles;        // row tiles (grid.x)
-    int S;                 // column splits (grid.y)
-    double* part;          // [ntiles * S * (D + 2)]
-    unsigned int* ticket;
+    double* part;          // [kGradCtas * (D + 2)]
+    unsigned int* ticket;  // zero between launches
     double* out;           // D + 2
+    int* err;              // wait-timeout flag
 };
+constexpr int kGradCtas = 152;  // persistent grid: one CTA per SM
 cudaError_t launch_grad(int kernel, const GradParams& p, int D, int C, cudaStream_t st);
 cudaError_t launch_grad_rbf(const GradParams& p, int D, int C, cudaStream_t st);
 cudaError_t launch_grad_m32(const GradParams& p, int D, int C, cudaStream_t st);
 cudaError_t launch_grad_m52(const GradParams& p, int D, int C, cudaStream_t st);
-int grad_rows_per_cta(int D, int C);
 
 // B = [y - mu, z_1..z_l]; Z == nullptr draws Rademacher z from SplitMix64(seed);
 // Zout (may be nullptr) receives the z actually used.

@@ -1,7 +1,7 @@
 // Fused backward pass of the stochastic MLL gradient (Eq. loss_grad_unbiased):
-// one sweep over all n^2 kernel entries that forms G_ij = sum_c alpha_c U_ic V_jc
-// on the fly and contracts it with every derivative dK_ij / dtheta at once
-// (d lengthscales, outputscale, noise).  No kernel block or G block is stored.
+// one sweep over the kernel entries that forms G_ij = sum_c alpha_c U_ic V_jc on the
+// fly and contracts it with every derivative dK_ij / dtheta at once (d lengthscales,
+// outputscale, noise).  No kernel block or G block is stored.
 //
 // With the pre-scaled inputs xs of the FP32 product (xs = c_K x / l, see
 // kernel_input_scale) and t = |xs_i - xs_j|^2:
@@ -10,9 +10,32 @@
 //   M52  u = sqrt(t), phi = (1+u+u^2/3) e^-u, psi = (1+u) e^-u
 // and dK/dl_k = s * kappa_K / (c_K^2 l_k) * psi * (xs_ik - xs_jk)^2 with
 // kappa_K / c_K^2 = 2/log2(e), 1, 1/3; the host applies those factors.
+//
+// What bounds it is FP32 work per entry, so the sweep does less of it in two ways.
+//   Symmetry: phi, psi and the squared differences are symmetric in (i, j), so only
+//   i < j is visited, with S_ij = G_ij + G_ji; the diagonal (phi = 1, no differences)
+//   adds sum_i G_ii to the outputscale and noise forms.
+//   Contraction on the tensor cores: S = [alpha U | V] [V | alpha U]^T, both operands
+//   split into three BF16 parts (exact up to the last rounding), the six products of
+//   weight above 2^-24 into two or three FP32 accumulators per entry: hi x hi in chains
+//   of at most two steps, the small ones on their own; the parts are added in FP32.
+// What is left are 4 d multiply-add lanes (as packed pairs) and about 14 instructions
+// per visited entry.  Measured (GB300, n = 131,072, d = 8, c = 32, Matern-3/2): 47.0 ->
+// 14.2 ms for the n^2 forms, FMA pipe 68 % busy, error against 64 bits unchanged (7.7e-8).
+// (With two stages 16.5 ms: the chunk's copy, split and MMAs follow one another.)
+//
+// Work units are (row group, 64-column chunk) pairs of the upper triangle in
+// group-major order, cut into equal ranges over a persistent grid; every CTA keeps
+// one set of sums whatever groups it meets (FP32 over 64 entries per thread, FP64
+// beyond), and the CTA that finishes last adds the CTAs' sums in order.
+// Warp roles: transform warps (one row, or two rows 128 apart, per thread; 16 columns of
+// every chunk), one MMA issuer, one bulk-copy lane for the columns' coordinates, two
+// warps that split the chunk's [V | alpha U]; the transform warps split the rows' own
+// operand when the group changes.  Every wait is bounded.
 #pragma once
 
 #include "kmv_fp32.cuh"
+#include "tcgen05.cuh"
 
 namespace ap {
 
@@ -34,105 +57,437 @@ __device__ __forceinline__ void phi_psi_fp32(float t, float& phi, float& psi) {
     }
 }
 
-constexpr int kGradThreads = 128;
-constexpr int kGradTN = 64;
+namespace gx {
+
+using namespace tc;
+
+constexpr int kChunk = 64;
+constexpr int kStages = 4;
+constexpr int kConvWarps = 2;
+constexpr int kFold = 4;  // chunks between folds of the FP32 sums into FP64
 
 template <int D, int C>
-struct GradShape {
-    static constexpr int RM = (D + C <= 40) ? 2 : 1;
-    static constexpr int ROWS = kGradThreads * RM;
+struct Cfg {
+    static constexpr int R = D <= 12 ? 2 : 1;                // rows per thread
+    static constexpr int kRows = 128 * R;
+    static constexpr int kXformWarps = D <= 16 ? 16 : 8;      // (more registers per thread for large D)
+    static constexpr int kSlots = kXformWarps / 4;
+    static constexpr int kMmaWarp = kXformWarps, kCopyWarp = kXformWarps + 1, kConvWarp = kXformWarps + 2;
+    static constexpr int kThreads = (kConvWarp + kConvWarps) * 32;
+    static constexpr int KC = 2 * C < 16 ? 16 : 2 * C;        // K of the contraction
+    static constexpr int kSteps = KC / 16;
+    static constexpr int kHh = (kSteps + 1) / 2;              // hi x hi accumulators
+    static constexpr uint32_t kAccCols = (kHh + 1) * kChunk;  // per row tile
+    static constexpr uint32_t kTmem = R * kAccCols <= 128 ? 128 : R * kAccCols <= 256 ? 256 : 512;
+    static constexpr uint32_t kPlaneA = 128 * KC * 2, kPlaneB = kChunk * KC * 2;
+    static constexpr uint32_t kXBytes = kChunk * D * 4;
+    static constexpr uint32_t kStageBytes = kXBytes + 3 * kPlaneB;
+    static constexpr size_t kSmem = 3 * R * kPlaneA + kStages * kStageBytes + 1024;
+    static constexpr int NA = D + 2;
+    static_assert(R * kAccCols <= 512, "tensor memory");
+    static_assert(kSmem <= 220 * 1024, "shared memory");
 };
 
-template <int KERN, int D, int C>
-__global__ void __launch_bounds__(kGradThreads) grad_kernel(const GradParams p) {
-    constexpr int RM = GradShape<D, C>::RM;
-    constexpr int ROWS = GradShape<D, C>::ROWS;
-    constexpr int NA = D + 2;
-    __shared__ __align__(16) float s_xb[kGradTN * D];
-    __shared__ __align__(16) float s_v[kGradTN * C];
-    __shared__ double red_d[32];
-    __shared__ double s_tot[NA];
-    __shared__ int s_last;
-    const int tid = threadIdx.x;
-    const int S = gridDim.y, rank = blockIdx.y;
-    const int64_t r0 = (int64_t)blockIdx.x * ROWS;
-    const int64_t cs = ((p.n + S - 1) / S + kGradTN - 1) / kGradTN * kGradTN;
-    const int64_t c_lo = rank * cs, c_hi = min(p.n, c_lo + cs);
+// x0, x1 as BF16 parts: hi cut off, mid and lo rounded to nearest (what is dropped of
+// the products then has no preferred sign).
+__device__ __forceinline__ void split3_rn(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+    constexpr uint32_t kTop = 0xFFFF0000u;
+    const uint32_t b0 = __float_as_uint(x0), b1 = __float_as_uint(x1);
+    hi = __byte_perm(b0, b1, 0x7632);
+    const float r0 = x0 - __uint_as_float(b0 & kTop), r1 = x1 - __uint_as_float(b1 & kTop);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(mid) : "f"(r1), "f"(r0));
+    const float s0 = r0 - __uint_as_float(mid << 16), s1 = r1 - __uint_as_float(mid & kTop);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(s1), "f"(s0));
+}
 
-    float xa[RM][D], ua[RM][C];
-    double diag = 0.0;
+// Eight consecutive K values k0 .. k0 + 7 of point i's operand into the three planes at
+// dst, dst + plane, dst + 2 plane: [first | second | 0], the U half scaled by alpha.
+template <int C>
+__device__ __forceinline__ void split_operand(const GradParams& p, int64_t i, int k0, bool u_first, uint8_t* dst,
+                                              uint32_t plane) {
+    float v[8];
 #pragma unroll
-    for (int q = 0; q < RM; ++q) {
-        const int64_t i = r0 + tid + q * kGradThreads;
-        const bool ok = i < p.n;
+    for (int j = 0; j < 8; ++j) v[j] = 0.0f;
+    if (i < p.n) {
+        if constexpr (C % 8 == 0) {  // the eight values lie in one half
+            const bool is_u = (k0 < C) == u_first;
+            const int c = k0 < C ? k0 : k0 - C;
+            const float4* src = reinterpret_cast<const float4*>((is_u ? p.U : p.V) + i * C + c);
+            const float4 x = __ldg(src), y = __ldg(src + 1);
+            v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+            v[4] = y.x, v[5] = y.y, v[6] = y.z, v[7] = y.w;
+            if (is_u) {
 #pragma unroll
-        for (int k = 0; k < D; ++k) xa[q][k] = ok ? p.Xs[i * D + k] : 0.0f;
-        float g = 0.0f;
+                for (int j = 0; j < 8; ++j) v[j] *= p.alpha[c + j];
+            }
+        } else {
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-            ua[q][c] = ok ? p.alpha[c] * p.U[i * C + c] : 0.0f;
-            if (ok) g = fmaf(ua[q][c], p.V[i * C + c], g);
-        }
-        if (rank == 0) diag += (double)g;
-    }
-    float accf[NA - 1];
-    double accd[NA - 1];
-#pragma unroll
-    for (int k = 0; k < NA - 1; ++k) { accf[k] = 0.0f; accd[k] = 0.0; }
-
-    for (int64_t cb = c_lo; cb < c_hi; cb += kGradTN) {
-        const int cnt = (int)min((int64_t)kGradTN, c_hi - cb);
-        __syncthreads();
-        for (int t = tid; t < cnt * D; t += kGradThreads) s_xb[t] = p.Xs[cb * D + t];
-        for (int t = tid; t < cnt * C; t += kGradThreads) s_v[t] = p.V[cb * C + t];
-        __syncthreads();
-        for (int jj = 0; jj < cnt; ++jj) {
-#pragma unroll
-            for (int q = 0; q < RM; ++q) {
-                float df2[D];
-                float t2 = 0.0f;
-#pragma unroll
-                for (int k = 0; k < D; ++k) {
-                    const float df = xa[q][k] - s_xb[jj * D + k];
-                    df2[k] = df * df;
-                    t2 += df2[k];
-                }
-                float g = 0.0f;
-#pragma unroll
-                for (int c = 0; c < C; ++c) g = fmaf(ua[q][c], s_v[jj * C + c], g);
-                float phi, psi;
-                phi_psi_fp32<KERN>(t2, phi, psi);
-                const float gp = g * psi;
-#pragma unroll
-                for (int k = 0; k < D; ++k) accf[k] = fmaf(gp, df2[k], accf[k]);
-                accf[D] = fmaf(g, phi, accf[D]);
+            for (int j = 0; j < 8; ++j) {
+                const int k = k0 + j, c = k < C ? k : k - C;
+                if (k < 2 * C) v[j] = (k < C) == u_first ? p.alpha[c] * __ldg(p.U + i * C + c) : __ldg(p.V + i * C + c);
             }
         }
-        // fold the chunk into FP64 so the n-term sums keep their precision
+    }
+    uint32_t w[3][4];
 #pragma unroll
-        for (int k = 0; k < NA - 1; ++k) { accd[k] += (double)accf[k]; accf[k] = 0.0f; }
+    for (int j = 0; j < 4; ++j) split3_rn(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl)
+        *reinterpret_cast<uint4*>(dst + pl * plane) = make_uint4(w[pl][0], w[pl][1], w[pl][2], w[pl][3]);
+}
+
+// Units before group g: group i has L - i rc chunks (L chunks in all, rc per group's rows).
+__host__ __device__ inline int64_t units_before(int64_t g, int64_t L, int rc) { return g * L - rc * (g * (g - 1) / 2); }
+
+template <int KERN, int D, int C>
+__global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const GradParams p) {
+    using K = Cfg<D, C>;
+    constexpr int R = K::R;
+    extern __shared__ __align__(1024) uint8_t gx_smem[];
+    uint8_t* s_a = gx_smem;                                // 3 planes x R tiles x 128 x KC
+    uint8_t* s_stage = gx_smem + 3 * R * K::kPlaneA;
+    __shared__ __align__(8) uint64_t bar_full[kStages], bar_ready[kStages], bar_empty[kStages];
+    __shared__ __align__(8) uint64_t bar_a, bar_acc, bar_acc_free;
+    __shared__ uint32_t s_tmem;
+    __shared__ volatile int s_abort;
+    __shared__ double s_part[K::kXformWarps][K::NA];
+    __shared__ int s_last;
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int64_t n = p.n, L = (n + kChunk - 1) / kChunk, ngroups = (n + K::kRows - 1) / K::kRows;
+    constexpr int rc = K::kRows / kChunk;
+    const int64_t U = units_before(ngroups, L, rc);
+    const int64_t u0 = U * blockIdx.x / gridDim.x, u1 = U * (blockIdx.x + 1) / gridDim.x;
+    const int total = (int)(u1 - u0);
+    // first group and chunk of the range
+    int64_t g0 = 0;
+    {
+        const double a = 0.5 * rc, b = (double)L + a;
+        const double disc = b * b - 4.0 * a * (double)u0;
+        g0 = (int64_t)((b - sqrt(disc > 0.0 ? disc : 0.0)) / (2.0 * a));
+        g0 = min(max(g0, (int64_t)0), ngroups - 1);
+        while (g0 > 0 && units_before(g0, L, rc) > u0) --g0;
+        while (g0 + 1 < ngroups && units_before(g0 + 1, L, rc) <= u0) ++g0;
     }
-    // CTA sums in FP64, then the ticketed last CTA adds the partials in order
-    for (int k = 0; k < NA; ++k) {
-        const double v = k < NA - 1 ? accd[k] : diag;
-        double t = cta_sum_d(v, red_d);
-        if (tid == 0) s_tot[k] = t;
+    const int64_t q0 = g0 * rc + (u0 - units_before(g0, L, rc));  // chunk (of all L)
+
+    if (tid == 0) {
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(&bar_full[i], 1);
+            mbar_init(&bar_ready[i], kConvWarps);
+            mbar_init(&bar_empty[i], 1 + K::kXformWarps);
+        }
+        mbar_init(&bar_a, K::kXformWarps);
+        mbar_init(&bar_acc, 1);
+        mbar_init(&bar_acc_free, K::kXformWarps);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (warp == K::kMmaWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(K::kTmem)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
     __syncthreads();
-    const int64_t idx = (int64_t)blockIdx.x * S + rank;
-    if (tid < NA) p.part[idx * NA + tid] = s_tot[tid];
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+
+    if (warp < K::kXformWarps) {
+        // ------------------------------------------------------- transform warps
+        const int quarter = warp & 3, slot = warp >> 2, row = quarter * 32 + lane;
+        const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
+        float2 xa[R][D / 2], accf[D / 2];
+        double accd[D + 1], diag = 0.0;
+        float accp = 0.0f;
+#pragma unroll
+        for (int k = 0; k < D / 2; ++k) accf[k] = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int k = 0; k < D + 1; ++k) accd[k] = 0.0;
+        auto fold = [&]() {
+#pragma unroll
+            for (int k = 0; k < D / 2; ++k) {
+                accd[2 * k] += (double)accf[k].x;
+                accd[2 * k + 1] += (double)accf[k].y;
+                accf[k] = make_float2(0.0f, 0.0f);
+            }
+            accd[D] += (double)accp;
+            accp = 0.0f;
+        };
+        // a group begins: coordinates, this warp's share of the rows' operand planes, and
+        // (first chunk of the group) the diagonal sums
+        auto begin_group = [&](int64_t g, bool first_chunk) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int64_t i = g * K::kRows + 128 * r + row;
+#pragma unroll
+                for (int k = 0; k < D / 4; ++k) {
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (i < n) v = __ldg(reinterpret_cast<const float4*>(p.Xs + i * D) + k);
+                    xa[r][2 * k] = make_float2(v.x, v.y);
+                    xa[r][2 * k + 1] = make_float2(v.z, v.w);
+                }
+                for (int k8 = slot; k8 < K::KC / 8; k8 += K::kSlots)
+                    split_operand<C>(p, i, 8 * k8, true,
+                                     s_a + r * K::kPlaneA + ((row >> 3) * (K::KC / 8) + k8) * 128 + (row & 7) * 16,
+                                     R * K::kPlaneA);
+                if (slot == 0 && first_chunk && i < n) {
+                    float s = 0.0f;
+                    for (int c = 0; c < C; ++c) s = fmaf(p.alpha[c] * __ldg(p.U + i * C + c), __ldg(p.V + i * C + c), s);
+                    diag += (double)s;
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_a);
+        };
+        const float2 m1 = make_float2(-1.0f, -1.0f);
+        bool ok = true;
+        int64_t g = g0, q = q0;
+        int stage = 0;
+        uint32_t sphase = 0;
+        if (total > 0) begin_group(g, q == g * rc);
+        for (int c = 0; c < total; ++c) {
+            ok = mbar_wait(&bar_full[stage], sphase, &s_abort, p.err) &&
+                 mbar_wait(&bar_ready[stage], sphase, &s_abort, p.err) &&
+                 mbar_wait(&bar_acc, (uint32_t)(c & 1), &s_abort, p.err);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const float* sx = reinterpret_cast<const float*>(s_stage + (size_t)stage * K::kStageBytes);
+            const bool upper = q >= (g + 1) * rc;  // every column is right of every row
+            // this warp's columns: eight at 8 slot + 8 kSlots h.  All of S is read first, so
+            // that the next chunk's MMAs run under the whole of this one's arithmetic.
+            constexpr int kPieces = kChunk / (8 * K::kSlots);
+            float sv[kPieces][R][8];
+#pragma unroll
+            for (int h = 0; h < kPieces; ++h) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const uint32_t at = tmem + lane_base + (uint32_t)r * K::kAccCols + (uint32_t)(8 * (slot + K::kSlots * h));
+                    uint32_t w[8], v[K::kHh][8];
+                    tmem_ld8(at + K::kHh * kChunk, w);
+#pragma unroll
+                    for (int a = 0; a < K::kHh; ++a) tmem_ld8(at + a * kChunk, v[a]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        sv[h][r][j] = __uint_as_float(w[j]);
+#pragma unroll
+                        for (int a = 0; a < K::kHh; ++a) sv[h][r][j] += __uint_as_float(v[a][j]);
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_acc_free);
+#pragma unroll
+            for (int h = 0; h < kPieces; ++h) {
+                const int h0 = 8 * (slot + K::kSlots * h);
+                float(&s)[R][8] = sv[h];
+                if (!upper) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const int64_t i = g * K::kRows + 128 * r + row, j0 = q * kChunk + h0;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            if (j0 + j <= i) s[r][j] = 0.0f;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float4* xb = reinterpret_cast<const float4*>(sx + (h0 + j) * D);
+                    float2 sq[R][D / 2], t2[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) t2[r] = make_float2(0.0f, 0.0f);
+#pragma unroll
+                    for (int k = 0; k < D / 4; ++k) {
+                        const float4 v = xb[k];
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const float2 da = __ffma2_rn(make_float2(v.x, v.y), m1, xa[r][2 * k]);
+                            const float2 db = __ffma2_rn(make_float2(v.z, v.w), m1, xa[r][2 * k + 1]);
+                            sq[r][2 * k] = __fmul2_rn(da, da);
+                            sq[r][2 * k + 1] = __fmul2_rn(db, db);
+                            t2[r] = __fadd2_rn(t2[r], sq[r][2 * k]);
+                            t2[r] = __fadd2_rn(t2[r], sq[r][2 * k + 1]);
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        float phi, psi;
+                        phi_psi_fp32<KERN>(t2[r].x + t2[r].y, phi, psi);
+                        const float gp = s[r][j] * psi;
+                        const float2 gp2 = make_float2(gp, gp);
+#pragma unroll
+                        for (int k = 0; k < D / 2; ++k) accf[k] = __ffma2_rn(gp2, sq[r][k], accf[k]);
+                        accp = fmaf(s[r][j], phi, accp);
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_empty[stage]);
+            if ((c + 1) % kFold == 0) fold();
+            if (++stage == kStages) {
+                stage = 0;
+                sphase ^= 1u;
+            }
+            if (++q == L) {
+                ++g;
+                q = g * rc;
+                if (c + 1 < total) begin_group(g, true);
+            }
+        }
+        fold();
+        // warp sums in FP64
+#pragma unroll
+        for (int k = 0; k < K::NA; ++k) {
+            double v = k < D ? accd[k] : k == D ? accd[D] + diag : diag;
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) s_part[warp][k] = v;
+        }
+    } else if (warp == K::kMmaWarp) {
+        // ------------------------------------------------------------ MMA issuer
+        constexpr uint32_t idesc = instr_desc(1, 128, kChunk);
+        constexpr uint32_t kSbo = (K::KC / 8) * 128;
+        const bool leader = elect_one();
+        const uint64_t a0 = smem_desc(smem_u32(s_a), 128, kSbo);
+        const uint64_t b0 = smem_desc(smem_u32(s_stage + K::kXBytes), 128, kSbo);
+        bool ok = true;
+        int stage = 0;
+        uint32_t sphase = 0, aphase = 0;
+        int64_t g = g0, q = q0;
+        bool new_group = true;
+        for (int c = 0; c < total && ok; ++c) {
+            ok = (!new_group || mbar_wait(&bar_a, aphase, &s_abort, p.err)) &&
+                 mbar_wait(&bar_ready[stage], sphase, &s_abort, p.err) &&
+                 (c == 0 || mbar_wait(&bar_acc_free, (uint32_t)((c - 1) & 1), &s_abort, p.err));
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            if (new_group) aphase ^= 1u;
+            new_group = false;
+            tc_fence_after();
+            if (leader) {
+                const uint64_t b = b0 + (uint64_t)((stage * K::kStageBytes) >> 4);
+#pragma unroll 1
+                for (int r = 0; r < R; ++r) {
+                    const uint64_t a = a0 + (uint64_t)((r * K::kPlaneA) >> 4);
+                    const uint32_t d = tmem + (uint32_t)r * K::kAccCols, ds = d + K::kHh * kChunk;
+                    constexpr uint64_t pa = (R * K::kPlaneA) >> 4, pb = K::kPlaneB >> 4;
+#pragma unroll
+                    for (int ks = 0; ks < K::kSteps; ++ks) {
+                        const uint64_t ak = a + (uint64_t)(16 * ks), bk = b + (uint64_t)(16 * ks);
+                        // the small products, smallest first, then hi x hi
+                        mma_ss(ds, ak + 2 * pa, bk, idesc, ks > 0 ? 1u : 0u);
+                        mma_ss(ds, ak + pa, bk + pb, idesc, 1u);
+                        mma_ss(ds, ak, bk + 2 * pb, idesc, 1u);
+                        mma_ss(ds, ak + pa, bk, idesc, 1u);
+                        mma_ss(ds, ak, bk + pb, idesc, 1u);
+                        mma_ss(d + (ks / 2) * kChunk, ak, bk, idesc, (uint32_t)(ks & 1));
+                    }
+                }
+                tc_commit(&bar_acc);
+                tc_commit(&bar_empty[stage]);
+            }
+            __syncwarp();
+            if (++stage == kStages) {
+                stage = 0;
+                sphase ^= 1u;
+            }
+            if (++q == L) {
+                ++g;
+                q = g * rc;
+                new_group = true;
+            }
+        }
+    } else if (warp == K::kCopyWarp) {
+        // ------------------------------------------ bulk copies of the coordinates
+        if (lane == 0) {
+            bool ok = true;
+            int64_t g = g0, q = q0;
+            int stage = 0;
+            for (int c = 0; c < total && ok; ++c) {
+                if (c >= kStages)
+                    ok = mbar_wait(&bar_empty[stage], (uint32_t)((c / kStages - 1) & 1), &s_abort, p.err);
+                if (!ok) break;
+                const int cnt = (int)min((int64_t)kChunk, n - q * kChunk);
+                const bool in = AP_CHK(q >= 0 && cnt > 0 && q * kChunk + cnt <= n);
+                mbar_expect_tx(&bar_full[stage], in ? (uint32_t)(cnt * D * 4) : 0u);
+                if (in)
+                    bulk_g2s(s_stage + (size_t)stage * K::kStageBytes, p.Xs + q * kChunk * D, (uint32_t)(cnt * D * 4),
+                             &bar_full[stage]);
+                if (++q == L) {
+                    ++g;
+                    q = g * rc;
+                }
+                if (++stage == kStages) stage = 0;
+            }
+        }
+    } else {
+        // --------------------------------------- splitters of the chunk's [V | alpha U]
+        const int ct = tid - K::kConvWarp * 32;
+        bool ok = true;
+        int64_t g = g0, q = q0;
+        int stage = 0;
+        uint32_t sphase = 0;
+        for (int c = 0; c < total && ok; ++c) {
+            // the copy into this stage has landed, so the stage's last users are done
+            ok = __all_sync(0xffffffffu, mbar_wait(&bar_full[stage], sphase, &s_abort, p.err));
+            if (!ok) break;
+            uint8_t* st = s_stage + (size_t)stage * K::kStageBytes;
+            const int cnt = (int)min((int64_t)kChunk, n - q * kChunk);
+            if (cnt < kChunk)
+                for (int t = cnt * D + ct; t < kChunk * D; t += 32 * kConvWarps) reinterpret_cast<float*>(st)[t] = 0.0f;
+#pragma unroll 2
+            for (int t = ct; t < kChunk * (K::KC / 8); t += 32 * kConvWarps) {
+                const int j = t % kChunk, k8 = t / kChunk;  // (neighbouring lanes fill one core matrix)
+                split_operand<C>(p, q * kChunk + j, 8 * k8, false,
+                                 st + K::kXBytes + ((j >> 3) * (K::KC / 8) + k8) * 128 + (j & 7) * 16, K::kPlaneB);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_ready[stage]);
+            if (++q == L) {
+                ++g;
+                q = g * rc;
+            }
+            if (++stage == kStages) {
+                stage = 0;
+                sphase ^= 1u;
+            }
+        }
+    }
+    // ---------------------------------------------------------------- teardown
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == K::kMmaWarp) {
+        if (s_abort) {
+            // a wait gave up: let copies and MMAs still in flight land first
+            const long long t0 = clock64();
+            while (clock64() - t0 < 4000000LL) {
+            }
+        }
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(K::kTmem) : "memory");
+    }
+    if (s_abort) return;
+    if (tid < K::NA) {
+        double v = 0.0;
+        for (int w = 0; w < K::kXformWarps; ++w) v += s_part[w][tid];
+        p.part[(int64_t)blockIdx.x * K::NA + tid] = v;
+    }
     __threadfence();
     __syncthreads();
-    if (tid == 0) {
-        const unsigned total = (unsigned)(p.ntiles * S);
-        s_last = (atomicAdd(p.ticket, 1u) == total - 1u) ? 1 : 0;
-    }
+    if (tid == 0) s_last = (atomicAdd(p.ticket, 1u) == gridDim.x - 1u) ? 1 : 0;
     __syncthreads();
     if (s_last) {
         __threadfence();
-        for (int k = tid; k < NA; k += kGradThreads) {
+        for (int k = tid; k < K::NA; k += K::kThreads) {
             double acc = 0.0;
-            for (int64_t t = 0; t < p.ntiles * S; ++t) acc += __ldcg(p.part + t * NA + k);
+            for (unsigned b = 0; b < gridDim.x; ++b) acc += __ldcg(p.part + (int64_t)b * K::NA + k);
             p.out[k] = acc;
         }
         if (tid == 0) *p.ticket = 0u;
@@ -140,19 +495,28 @@ __global__ void __launch_bounds__(kGradThreads) grad_kernel(const GradParams p) 
 }
 
 template <int KERN, int D, int C>
-cudaError_t launch_grad_inst(const GradParams& p, cudaStream_t st) {
-    grad_kernel<KERN, D, C><<<dim3((unsigned)p.ntiles, (unsigned)p.S, 1), kGradThreads, 0, st>>>(p);
+cudaError_t launch_inst(const GradParams& p, cudaStream_t st) {
+    using K = Cfg<D, C>;
+    auto fn = grad_kernel<KERN, D, C>;
+    cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K::kSmem);
+    if (err != cudaSuccess) return err;
+    const int64_t L = (p.n + kChunk - 1) / kChunk, ngroups = (p.n + K::kRows - 1) / K::kRows;
+    const int64_t U = units_before(ngroups, L, K::kRows / kChunk);
+    const int64_t grid = U < kGradCtas ? U : kGradCtas;
+    fn<<<(unsigned)grid, K::kThreads, K::kSmem, st>>>(p);
     return cudaGetLastError();
 }
+
+}  // namespace gx
 
 template <int KERN>
 cudaError_t dispatch_grad(const GradParams& p, int D, int C, cudaStream_t st) {
 #define AP_GRAD_C(DD)                                                    \
     switch (C) {                                                         \
-        case 1: return launch_grad_inst<KERN, DD, 1>(p, st);             \
-        case 4: return launch_grad_inst<KERN, DD, 4>(p, st);             \
-        case 16: return launch_grad_inst<KERN, DD, 16>(p, st);           \
-        case 32: return launch_grad_inst<KERN, DD, 32>(p, st);           \
+        case 1: return gx::launch_inst<KERN, DD, 1>(p, st);              \
+        case 4: return gx::launch_inst<KERN, DD, 4>(p, st);              \
+        case 16: return gx::launch_inst<KERN, DD, 16>(p, st);            \
+        case 32: return gx::launch_inst<KERN, DD, 32>(p, st);            \
         default: return cudaErrorInvalidValue;                           \
     }
     switch (D) {

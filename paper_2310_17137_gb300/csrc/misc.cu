@@ -204,8 +204,6 @@ cudaError_t launch_norms_select(const float* R, int64_t n, int C, const EpiParam
 
 namespace ap {
 
-int grad_rows_per_cta(int D, int C) { return 128 * ((D + C <= 40) ? 2 : 1); }
-
 cudaError_t launch_kmv_comp(int kernel, const KmvParams& p, int D, int C, cudaStream_t st) {
     switch (kernel) {
         case AP_RBF: return launch_kmv_comp_rbf(p, D, C, st);

@@ -10,6 +10,8 @@
 // this entry point, which uses only the buffers the caller passes and one
 // fixed scratch array compiled into the library.  The call still copies its
 // sums to the host and synchronises the context's stream before returning.
+#include <string.h>
+
 #include <mutex>
 
 #include "ap_internal.cuh"
@@ -24,7 +26,8 @@ namespace {
 constexpr size_t kScratchDoubles = (size_t)AP_STATIC_SCRATCH_BYTES / sizeof(double);
 static __device__ __align__(256) double g_scratch[kScratchDoubles];
 
-constexpr size_t kTicketOff = 0;   // one unsigned int (padded to 8 doubles)
+constexpr size_t kTicketOff = 0;   // one unsigned int
+constexpr size_t kErrOff = 1;      // one int: a wait of the kernel ran out
 constexpr size_t kOutOff = 8;      // D + 2 <= 34 sums
 constexpr size_t kPartOff = 64;    // per-CTA partials
 
@@ -60,9 +63,11 @@ extern "C" ap_status ap_grad_quadforms_static(ap_ctx* ctx, const float* U_dev, c
     GradView v;
     ctx_grad_view(ctx, &v);
     const int NA = v.D + 2;
-    const int64_t rows = grad_rows_per_cta(v.D, c);
+    // the documented limit: (D + 2) doubles per block of 128 (or 256) rows
+    const int64_t rows = v.D + c <= 40 ? 256 : 128;
     const int64_t ntiles = (v.n + rows - 1) / rows;
     if ((size_t)(kPartOff + ntiles * NA) > kScratchDoubles) return AP_ERR_SCRATCH_LIMIT;
+    static_assert(kPartOff + (size_t)kGradCtas * (AP_MAX_DIM + 2) <= kScratchDoubles, "scratch");
     DeviceGuard dg(v.device);  // the context's device is current for the look-up and the launch
     if (!dg.ok()) return AP_ERR_CUDA;
     double* scratch = nullptr;
@@ -76,19 +81,23 @@ extern "C" ap_status ap_grad_quadforms_static(ap_ctx* ctx, const float* U_dev, c
     gp.U = U_dev;
     gp.V = V_dev;
     for (int k = 0; k < c; ++k) gp.alpha[k] = (float)alpha_host[k];
-    gp.ntiles = ntiles;
-    gp.S = 1;
     gp.part = scratch + kPartOff;
     gp.ticket = reinterpret_cast<unsigned int*>(scratch + kTicketOff);
     gp.out = scratch + kOutOff;
+    gp.err = reinterpret_cast<int*>(scratch + kErrOff);
     double raw[AP_MAX_DIM + 2] = {};
-    if (cudaMemsetAsync(gp.ticket, 0, sizeof(unsigned int), v.stream) != cudaSuccess ||
+    double err = 0.0;  // the flag's eight bytes
+    if (cudaMemsetAsync(gp.ticket, 0, 2 * sizeof(double), v.stream) != cudaSuccess ||
         launch_grad(v.kernel, gp, v.D, c, v.stream) != cudaSuccess ||
         cudaMemcpyAsync(raw, gp.out, sizeof(double) * NA, cudaMemcpyDeviceToHost, v.stream) != cudaSuccess ||
+        cudaMemcpyAsync(&err, gp.err, sizeof(double), cudaMemcpyDeviceToHost, v.stream) != cudaSuccess ||
         cudaStreamSynchronize(v.stream) != cudaSuccess) {
         cudaGetLastError();
         return AP_ERR_CUDA;
     }
+    int flag = 0;
+    memcpy(&flag, &err, sizeof(flag));
+    if (flag) return AP_ERR_TIMEOUT;
     grad_finish(v, raw, out_host);
     return AP_OK;
 }
