@@ -53,6 +53,8 @@ struct ap_ctx {
     ap_opts o = {};
     cudaStream_t ust = nullptr;  // caller's stream
     cudaStream_t st = nullptr;   // context stream (work is ordered after ust on entry)
+    cudaStream_t st_side = nullptr;  // diagonal tiles of the factorisation's look-ahead
+    cudaEvent_t ev_col = nullptr, ev_diag = nullptr;
     cudaEvent_t ev_a = nullptr, ev_b = nullptr, ev_sync = nullptr;
     int64_t b = 0, m = 0;
     int nt = 0;
@@ -410,7 +412,7 @@ ap_status build_cache(ap_ctx* ctx) {
             return s;
         }
     }
-    const OzWork oz = {ozS, ozE, &ctx->state->tc_err};
+    const OzWork oz = {ozS, ozE, &ctx->state->tc_err, ctx->st_side, ctx->ev_col, ctx->ev_diag};
     AP_CK(cudaMemsetAsync(ctx->bad, 0, sizeof(int) * ctx->m, ctx->st));
     CacheParams cp = {};
     cp.X = ctx->X;
@@ -742,6 +744,8 @@ void copy_hyper(ap_ctx* ctx, const ap_hyper* h) {
 
 void free_all(ap_ctx* ctx) {
     drop_graph(ctx);
+    // (the side stream's work uses the context stream's memory)
+    if (ctx->st_side) cudaStreamSynchronize(ctx->st_side);
     std::vector<void*> ptrs;
     for (auto& kv : ctx->sizes) ptrs.push_back(kv.first);
     for (void* p : ptrs) cudaFreeAsync(p, ctx->st);
@@ -757,6 +761,9 @@ void free_all(ap_ctx* ctx) {
     for (cudaEvent_t e : ctx->ev_up) cudaEventDestroy(e);
     ctx->ev_bs.clear();
     ctx->ev_up.clear();
+    if (ctx->ev_col) cudaEventDestroy(ctx->ev_col);
+    if (ctx->ev_diag) cudaEventDestroy(ctx->ev_diag);
+    if (ctx->st_side) cudaStreamDestroy(ctx->st_side);
     if (ctx->st) cudaStreamDestroy(ctx->st);
     cudaGetLastError();
 }
@@ -1148,6 +1155,9 @@ ap_status ap_create(ap_ctx** out, const float* X_dev, int64_t n, int32_t d, cons
         return e;
     };
     if (cudaStreamCreateWithFlags(&ctx->st, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&ctx->st_side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_col, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_diag, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreate(&ctx->ev_a) != cudaSuccess || cudaEventCreate(&ctx->ev_b) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_sync, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreate(&ctx->ev_r0) != cudaSuccess || cudaEventCreate(&ctx->ev_r1) != cudaSuccess) {

@@ -190,8 +190,12 @@ struct CacheParams {
 // oz_slice_bytes(nt) bytes and oz_expo_ints(nt) row exponents per block.
 size_t oz_slice_bytes(int nt);
 size_t oz_expo_ints(int nt);
-cudaError_t launch_oz_update(double* A, int nt, int k, int g, uint8_t* S, int* E, int* err, cudaStream_t st,
-                             int64_t* launches);
+// The trailing update of panel k in two parts: the panel's slices and the first trailing
+// column of tiles, then the remaining columns on `ctas` CTAs (0: one per SM).
+cudaError_t launch_oz_update_first(double* A, int nt, int k, int g, uint8_t* S, int* E, int* err, cudaStream_t st,
+                                   int64_t* launches);
+cudaError_t launch_oz_update_rest(double* A, int nt, int k, int g, uint8_t* S, int* E, int* err, int ctas,
+                                  cudaStream_t st, int64_t* launches);
 // The panel solve A_ik := A_ik L_kk^{-T} (i > k) the same way, L_kk^{-1} from Dinv.
 cudaError_t launch_oz_trsm(double* A, const double* Dinv, int nt, int k, int g, uint8_t* S, int* E, int* err,
                            cudaStream_t st, int64_t* launches);
@@ -200,6 +204,8 @@ struct OzWork {
     uint8_t* S;  // g * oz_slice_bytes(nt)
     int* E;      // g * oz_expo_ints(nt)
     int* err;    // wait-timeout flag
+    cudaStream_t side;           // the next diagonal tiles are factored here meanwhile
+    cudaEvent_t ev_col, ev_diag; // first trailing column updated; next diagonal tiles factored
 };
 // FP64 phi of the cache build at count squared distances (device arrays).
 cudaError_t launch_phi_fp64_eval(int kernel, const double* r2, int64_t count, double* out, cudaStream_t st);

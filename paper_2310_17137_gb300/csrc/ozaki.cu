@@ -163,14 +163,19 @@ __device__ __forceinline__ double level_sum(int h1, int h2, int l1, int l2, int 
     return __longlong_as_double((long long)(bits | ((unsigned long long)sign & 0x8000000000000000ull)));
 }
 
-// kTrsm = false: A_ij -= A_ik A_jk^T over the trailing lower tiles (SYRK/GEMM);
-// kTrsm = true:  A_ik := A_ik L_kk^{-T} for the panel tiles i > k (TRSM as a
+// kFirst, kRest: A_ij -= A_ik A_jk^T over the trailing lower tiles (SYRK/GEMM);
+// kPanel: A_ik := A_ik L_kk^{-T} for the panel tiles i > k (TRSM as a
 // product with the inverse diagonal tile, whose slices sit in the plane rows
 // of tile k), written instead of subtracted.
-template <bool kTrsm>
+// The SYRK form runs in two launches: column tile j = k + 1 (kFirst), which the next
+// panel's factorisation waits for, and the columns beyond.
+enum OzPart { kFirst, kRest, kPanel };
+
+template <OzPart kPart>
 __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int nt, int k, const uint8_t* S,
                                                                size_t plane_bytes, const int* E, int* err,
                                                                int tiles_per_block, int nwork) {
+    constexpr bool kTrsm = kPart == kPanel;
     extern __shared__ __align__(1024) uint8_t oz_smem[];
     // slices in shared memory, accumulators complete, accumulators read
     __shared__ __align__(8) uint64_t bar_load, bar_mma, bar_read;
@@ -187,16 +192,17 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
     auto decode = [&](int w, int& z, int& i0, int& j) {
         z = w / tiles_per_block;
         int u = 0, jj = w - z * tiles_per_block;
-        if constexpr (kTrsm) {
-            u = jj;
-            jj = -1;
-        } else {
+        if constexpr (kPart == kRest) {
             while (true) {
-                const int nc = min(2 * u + 2, rem);
+                const int nc = min(2 * u + 2, rem) - 1;
                 if (jj < nc) break;
                 jj -= nc;
                 ++u;
             }
+            ++jj;
+        } else {
+            u = jj;
+            jj = kTrsm ? -1 : 0;
         }
         i0 = k + 1 + 2 * u;
         j = k + 1 + jj;
@@ -394,13 +400,13 @@ size_t oz_plane_bytes(int nt) { return (size_t)((int64_t)nt * T + T) * kRowBytes
 size_t oz_slice_bytes(int nt) { return kSlices * oz_plane_bytes(nt); }
 size_t oz_expo_ints(int nt) { return (size_t)((int64_t)nt * T + T); }
 
-cudaError_t launch_oz_update(double* A, int nt, int k, int g, uint8_t* S, int* E, int* err, cudaStream_t st,
-                             int64_t* launches) {
+cudaError_t launch_oz_update_first(double* A, int nt, int k, int g, uint8_t* S, int* E, int* err, cudaStream_t st,
+                                   int64_t* launches) {
     const int rem = nt - k - 1;
     if (rem <= 0) return cudaSuccess;
     static_assert(kOzSmem + 1024 <= 227 * 1024, "shared memory");
     cudaError_t e =
-        cudaFuncSetAttribute(oz_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
+        cudaFuncSetAttribute(oz_gemm_kernel<kFirst>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
     if (e != cudaSuccess) return e;
     const size_t pb = oz_plane_bytes(nt);
     const int64_t ld = (int64_t)nt * T;
@@ -408,12 +414,26 @@ cudaError_t launch_oz_update(double* A, int nt, int k, int g, uint8_t* S, int* E
     oz_slice_kernel<<<dim3((unsigned)((rows + 31) / 32), (unsigned)g), 256, 0, st>>>(
         A + (int64_t)(k + 1) * T * ld + (int64_t)k * T, ld * ld, ld, rows, (int64_t)(k + 1) * T, ld + T, pb, S, E);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    int tiles = 0;
-    for (int u = 0; 2 * u < rem; ++u) tiles += std::min(2 * u + 2, rem);
-    const int nwork = tiles * g;
-    oz_gemm_kernel<false><<<(unsigned)std::min(nwork, sm_count()), kOzThreads, kOzSmem, st>>>(A, nt, k, S, pb, E, err,
-                                                                                            tiles, nwork);
+    const int tiles = (rem + 1) / 2, nwork = tiles * g;
+    oz_gemm_kernel<kFirst><<<(unsigned)std::min(nwork, sm_count()), kOzThreads, kOzSmem, st>>>(A, nt, k, S, pb, E, err,
+                                                                                             tiles, nwork);
     if (launches) *launches += 2;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_oz_update_rest(double* A, int nt, int k, int g, uint8_t* S, int* E, int* err, int ctas,
+                                  cudaStream_t st, int64_t* launches) {
+    const int rem = nt - k - 1;
+    int tiles = 0;
+    for (int u = 0; 2 * u < rem; ++u) tiles += std::min(2 * u + 2, rem) - 1;
+    if (tiles <= 0) return cudaSuccess;
+    cudaError_t e =
+        cudaFuncSetAttribute(oz_gemm_kernel<kRest>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
+    if (e != cudaSuccess) return e;
+    const int nwork = tiles * g;
+    oz_gemm_kernel<kRest><<<(unsigned)std::min(nwork, ctas > 0 ? ctas : sm_count()), kOzThreads, kOzSmem, st>>>(
+        A, nt, k, S, oz_plane_bytes(nt), E, err, tiles, nwork);
+    if (launches) *launches += 1;
     return cudaGetLastError();
 }
 
@@ -422,7 +442,7 @@ cudaError_t launch_oz_trsm(double* A, const double* Dinv, int nt, int k, int g, 
     const int rem = nt - k - 1;
     if (rem <= 0) return cudaSuccess;
     cudaError_t e =
-        cudaFuncSetAttribute(oz_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
+        cudaFuncSetAttribute(oz_gemm_kernel<kPanel>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem);
     if (e != cudaSuccess) return e;
     const size_t pb = oz_plane_bytes(nt);
     const int64_t ld = (int64_t)nt * T;
@@ -435,7 +455,7 @@ cudaError_t launch_oz_trsm(double* A, const double* Dinv, int nt, int k, int g, 
                                                                 T, (int64_t)k * T, ld + T, pb, S, E);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int tiles = (rem + 1) / 2, nwork = tiles * g;
-    oz_gemm_kernel<true><<<(unsigned)std::min(nwork, sm_count()), kOzThreads, kOzSmem, st>>>(A, nt, k, S, pb, E, err,
+    oz_gemm_kernel<kPanel><<<(unsigned)std::min(nwork, sm_count()), kOzThreads, kOzSmem, st>>>(A, nt, k, S, pb, E, err,
                                                                                            tiles, nwork);
     if (launches) *launches += 3;
     return cudaGetLastError();
