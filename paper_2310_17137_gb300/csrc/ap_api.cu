@@ -419,7 +419,7 @@ ap_status build_cache(ap_ctx* ctx) {
     cp.n = ctx->n;
     cp.d = ctx->d;
     cp.kernel = ctx->kernel;
-    for (int k = 0; k < ctx->d; ++k) cp.ell[k] = (double)ctx->ell[k];
+    for (int k = 0; k < ctx->d; ++k) cp.unit[k] = cache_unit(ctx->kernel, (double)ctx->ell[k]);
     cp.s = ctx->s;
     cp.noise = ctx->noise;
     cp.b = ctx->b;

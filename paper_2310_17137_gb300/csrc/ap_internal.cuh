@@ -177,7 +177,7 @@ struct CacheParams {
     int64_t n;
     int d;
     int kernel;
-    double ell[AP_MAX_DIM];
+    double unit[AP_MAX_DIM];  // cache_unit per dimension
     double s, noise;
     int64_t b;             // block size
     int nt;                // tiles per block edge = ceil(b / kTile)
@@ -209,6 +209,8 @@ struct OzWork {
 };
 // FP64 phi of the cache build at count squared distances (device arrays).
 cudaError_t launch_phi_fp64_eval(int kernel, const double* r2, int64_t count, double* out, cudaStream_t st);
+// Scale of a coordinate such that the squared distance is phi's argument in the cache.
+double cache_unit(int kernel, double ell);
 cudaError_t cache_factor_group(const CacheParams& cp, int64_t blk0, int g, double* A, double* Dinv,
                                float* Linv, int* bad, const OzWork* oz, cudaStream_t st, int64_t* launches);
 

@@ -30,8 +30,10 @@ constexpr int kSms = 152;
 
 // ---------------------------------------------------------------- FP64 phi
 // The kernel profile phi(r^2) in FP64 for K_II, built from a handful of FP64
-// FMAs instead of the library exp and sqrt (FP64 arithmetic is scarce on this
-// part; the library calls cost ~90 FP64 operations per entry).
+// FMAs instead of the library exp and sqrt.  FP64 arithmetic (2 results per clock per
+// SM) is all that bounds the K_II build, and comparisons, conversions and rounding count
+// as much as a multiply-add, so ranges are tested and integers taken on the bits
+// (GB300, 5 blocks of 4096, d = 8: 4.28 -> 3.23 ms).
 //
 // exp(x), x <= 0: Tang's table-driven method (P. T. P. Tang, "Table-driven
 // implementation of the exponential function in IEEE floating-point
@@ -39,20 +41,24 @@ constexpr int kSms = 152;
 // |r| <= ln2/128, e^x = 2^k 2^(j/64) e^r.  ln2/64 is split into the double
 // nearest to it and the double nearest to the remainder, so r is exact to a
 // rounding; e^r - 1 is its Taylor polynomial to degree 6 (truncation below
-// r^7/7! < 2^-62 relative).  2^k is assembled from its exponent bits.  Below
-// x = -708 the result is 0 (e^-708 ~ 3e-308, far below any kernel value
-// that matters next to sigma^2).
-// sqrt(x): the FP32 reciprocal square root (relative error < 2^-22), one
-// Newton step for 1/sqrt(x) in FP64 (error ~1.5 e^2 < 2^-44), then one
-// Newton correction of s = x y (error ~e^2, below the last bit).
+// r^7/7! < 2^-62 relative).  The integer 64 k + j is the low word of the product plus
+// 1.5 * 2^52, and k is added to the exponent bits.  Below x = -708 the result is 0
+// (e^-708 ~ 3e-308, far below any kernel value that matters next to sigma^2; above it
+// 2^k 2^(j/64) stays normal).
+// sqrt(x): from the hardware's approximate reciprocal square root (relative error
+// below 2^-20) one coupled Newton step for sqrt(x) and 1/(2 sqrt(x)) (Goldschmidt's
+// form; error 3/2 e^2 < 2^-39), then one Newton correction with the exact residual
+// (error ~e^2, below the last bit).
 constexpr double kLn2By64Hi = 0x1.62e42fefa39efp-7;   // double nearest to ln2 / 64
 constexpr double kLn2By64Lo = 0x1.abc9e3b39803fp-62;  // ln2 / 64 - kLn2By64Hi, rounded
 constexpr double k64ByLn2 = 92.33248261689366;        // 64 / ln2
+constexpr double kRound = 6755399441055744.0;         // 1.5 * 2^52
 
 __device__ __forceinline__ double exp_nonpos(double x, const double* tab2) {
-    if (!(x >= -708.0)) return 0.0;  // also maps NaN to 0; callers pass finite x
-    const double nf = rint(x * k64ByLn2);
-    const int n = (int)nf;
+    if ((__double2hiint(x) & 0x7fffffff) > __double2hiint(708.0)) return 0.0;  // (also a NaN; callers pass finite x)
+    const double nb = fma(x, k64ByLn2, kRound);
+    const int n = __double2loint(nb);
+    const double nf = nb - kRound;
     const double r = fma(-nf, kLn2By64Lo, fma(-nf, kLn2By64Hi, x));
     double q = 1.0 / 720.0;
     q = fma(q, r, 1.0 / 120.0);
@@ -62,29 +68,33 @@ __device__ __forceinline__ double exp_nonpos(double x, const double* tab2) {
     q = fma(q, r, 1.0);
     const double t = tab2[n & 63];
     const double y = fma(t, q * r, t);
-    const int k = n >> 6;  // floor(n / 64), in [-1022, 0]
-    return y * __longlong_as_double((long long)(k + 1023) << 52);
+    // k = floor(n / 64) in [-1022, 0]
+    return __hiloint2double(__double2hiint(y) + ((n >> 6) << 20), __double2loint(y));
 }
 
 __device__ __forceinline__ double sqrt_nonneg(double x) {
-    if (x < 1e-36) return 0.0;  // phi is flat at 0: the error is below the last bit
-    if (x > 1e12) return 1e6;   // e^-sqrt(x) underflows either way
-    float yf;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"((float)x));
-    double y = (double)yf;
-    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
-    const double s = x * y;
-    return fma(0.5 * y, fma(-s, s, x), s);
+    const int hi = __double2hiint(x);
+    if (hi < __double2hiint(1e-36)) return 0.0;  // phi is flat at 0: the error is below the last bit
+    if (hi > __double2hiint(1e12)) return 1e6;   // e^-sqrt(x) underflows either way
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double g = x * y, h = 0.5 * y;
+    const double e = fma(-g, h, 0.5);
+    g = fma(g, e, g);
+    h = fma(h, e, h);
+    return fma(fma(-g, g, x), h, g);
 }
 
-__device__ __forceinline__ double phi_fp64(int kernel, double r2, const double* tab2) {
-    if (kernel == AP_RBF) return exp_nonpos(-0.5 * r2, tab2);
-    if (kernel == AP_MATERN32) {
-        const double u = sqrt_nonneg(3.0 * r2);
-        return (1.0 + u) * exp_nonpos(-u, tab2);
-    }
-    const double u = sqrt_nonneg(5.0 * r2);
-    return fma(u, fma(u, 1.0 / 3.0, 1.0), 1.0) * exp_nonpos(-u, tab2);
+// phi from t = r^2 / 2 (RBF), 3 r^2 (Matern-3/2) or 5 r^2 (Matern-5/2)
+__device__ __forceinline__ double phi_of(int kernel, double t, const double* tab2) {
+    if (kernel == AP_RBF) return exp_nonpos(-t, tab2);
+    const double u = sqrt_nonneg(t);
+    const double poly = kernel == AP_MATERN32 ? 1.0 + u : fma(u, fma(u, 1.0 / 3.0, 1.0), 1.0);
+    return poly * exp_nonpos(-u, tab2);
+}
+
+__host__ __device__ inline double phi_scale(int kernel) {
+    return kernel == AP_RBF ? 0.5 : (kernel == AP_MATERN32 ? 3.0 : 5.0);
 }
 
 // 2^(j/64), j = 0..63, into shared memory (first 64 threads; caller syncs)
@@ -105,7 +115,6 @@ __device__ __forceinline__ int64_t packed_tile(int i, int k) { return (int64_t)i
 
 __global__ void __launch_bounds__(256) build_kii_kernel(const CacheParams cp, int64_t blk0, double* A) {
     __shared__ double s_tab[64];
-    __shared__ double s_inv_ell[AP_MAX_DIM];
     __shared__ double s_xi[AP_MAX_DIM * T], s_xj[AP_MAX_DIM * T];  // dimension-major
     const int z = blockIdx.y;
     const int64_t blk = blk0 + z;
@@ -117,13 +126,15 @@ __global__ void __launch_bounds__(256) build_kii_kernel(const CacheParams cp, in
     const int64_t bJ = min(cp.b, cp.n - lo);
     double* Ab = A + (int64_t)z * ld * ld;
     fill_exp2_table(s_tab);
-    if (threadIdx.x < d) s_inv_ell[threadIdx.x] = 1.0 / cp.ell[threadIdx.x];
-    // the tile's row and column points (rows past the block are never read)
+    // the tile's row and column points relative to the block's first one (differences of
+    // FP32 values, exact in FP64 unless 29 binades apart), in units that make the squared
+    // distance phi's argument: two FP64 operations per entry and dimension are left
     for (int t = threadIdx.x; t < T * d; t += blockDim.x) {
         const int r = t / d, k = t % d;
         const int64_t li = (int64_t)ti * T + r, lj = (int64_t)tj * T + r;
-        s_xi[k * T + r] = li < bJ ? (double)cp.X[(lo + li) * d + k] : 0.0;
-        s_xj[k * T + r] = lj < bJ ? (double)cp.X[(lo + lj) * d + k] : 0.0;
+        const double x0 = (double)cp.X[lo * d + k];
+        s_xi[k * T + r] = li < bJ ? ((double)cp.X[(lo + li) * d + k] - x0) * cp.unit[k] : 0.0;
+        s_xj[k * T + r] = lj < bJ ? ((double)cp.X[(lo + lj) * d + k] - x0) * cp.unit[k] : 0.0;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < T * T; t += blockDim.x) {
@@ -131,13 +142,12 @@ __global__ void __launch_bounds__(256) build_kii_kernel(const CacheParams cp, in
         const int64_t li = (int64_t)ti * T + r, lj = (int64_t)tj * T + q;
         double v;
         if (li < bJ && lj < bJ) {
-            // the difference of two FP32 values is exact in FP64
             double r2 = 0.0;
             for (int k = 0; k < d; ++k) {
-                const double df = (s_xi[k * T + r] - s_xj[k * T + q]) * s_inv_ell[k];
+                const double df = s_xi[k * T + r] - s_xj[k * T + q];
                 r2 = fma(df, df, r2);
             }
-            v = cp.s * phi_fp64(cp.kernel, r2, s_tab);
+            v = cp.s * phi_of(cp.kernel, r2, s_tab);
             if (li == lj) v += cp.noise;
         } else {
             v = (li == lj) ? 1.0 : 0.0;
@@ -153,7 +163,7 @@ __global__ void __launch_bounds__(256) phi_fp64_eval_kernel(int kernel, const do
     fill_exp2_table(s_tab);
     __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = phi_fp64(kernel, r2[i], s_tab);
+        out[i] = phi_of(kernel, phi_scale(kernel) * r2[i], s_tab);
 }
 
 // 1/sqrt(p) for a pivot: the reciprocal square root approximation (relative error
@@ -542,6 +552,8 @@ cudaError_t launch_phi_fp64_eval(int kernel, const double* r2, int64_t count, do
     phi_fp64_eval_kernel<<<(unsigned)blocks, 256, 0, st>>>(kernel, r2, count, out);
     return cudaGetLastError();
 }
+
+double cache_unit(int kernel, double ell) { return sqrt(phi_scale(kernel)) / ell; }
 
 cudaError_t cache_factor_group(const CacheParams& cp, int64_t blk0, int g, double* A, double* Dinv,
                                float* Linv, int* bad, const OzWork* oz, cudaStream_t st, int64_t* launches) {
