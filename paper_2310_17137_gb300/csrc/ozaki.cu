@@ -43,7 +43,7 @@
 // 13 blocks 693 -> 395 us; panel solves of 5 blocks 33 -> 14 us.  Each CTA takes a
 // contiguous range of items, whose neighbours share the 128 KB row slab in shared
 // memory, and fetches half of the entries to update before it waits for the MMAs:
-// 148 -> 120 us and 395 -> 289 us.
+// 148 -> 120 us and 395 -> 289 us; the 16 x 256 bit reads (see the epilogue) 120 -> 91 us.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -142,25 +142,37 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const double* src0, int64
     if (grp == 0) E[(int64_t)z * rows_pad + r] = nonfinite ? kBadExp : e;
 }
 
-// 2^e0 (2^33 h1 + 2^19 h2 + 2^5 l1 + round(2^-9 l2)) rounded to a double, h1 .. l2
-// below 2^29: the sum is a 64-bit integer below 2^63, normalised and rounded (half
-// away from zero) with integer instructions.
-__device__ __noinline__ double level_sum_extreme(long long v, int e0) {  // beyond the normal doubles
-    return ldexp((double)v, max(-2000, min(2000, e0)));
+// 2^33 h1 + 2^19 h2 + 2^5 l1 + round(2^-9 l2), h1 .. l2 below 2^29: below 2^63.
+__device__ __forceinline__ long long level_int(int h1, int h2, int l1, int l2) {
+    return (long long)h2 * (1LL << 19) + ((long long)l1 * 32 + ((l2 + 256) >> 9)) + ((long long)h1 << 33);
 }
 
-__device__ __forceinline__ double level_sum(int h1, int h2, int l1, int l2, int e0) {
-    const long long v = (long long)h1 * (1LL << 33) + (long long)h2 * (1LL << 19) + (long long)l1 * 32 + ((l2 + 256) >> 9);
-    if (v == 0) return 0.0;
+// 2^e0 v rounded to a double (half away from zero), for results in the normal range:
+// normalised and rounded with integer instructions and no branches, so that a thread's
+// sixteen chains run side by side.  `extreme` is set when the exponent leaves the
+// normal doubles (also for the marked row exponents): the result is then not usable.
+__device__ __forceinline__ double level_sum(long long v, int e0, bool& extreme) {
     const long long sign = v >> 63;
     const unsigned long long m0 = (unsigned long long)((v ^ sign) - sign);
-    const int lz = __clzll((long long)m0);
+    const unsigned hi = (unsigned)(m0 >> 32), lo = (unsigned)m0;
+    const int lz = hi ? __clz((int)hi) : 32 + __clz((int)lo);
+    // m = m0 << lz
+    const unsigned a = hi ? hi : lo, b = hi ? lo : 0u;
+    const unsigned mh = __funnelshift_l(b, a, lz), ml = b << (lz & 31);
     const int be = 1023 + 63 - lz + e0;  // biased exponent
-    if (be < 1 || be > 2045) return level_sum_extreme(v, e0);
-    const unsigned long long m = m0 << lz;
-    const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // 53 bits, the leading one included
-    const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + r;
-    return __longlong_as_double((long long)(bits | ((unsigned long long)sign & 0x8000000000000000ull)));
+    extreme |= m0 != 0 && (unsigned)(be - 1) > 2044u;
+    // 53 bits, the leading one included; a carry moves on into the exponent
+    const unsigned long long r = (((unsigned long long)(mh >> 11) << 32) | __funnelshift_r(ml, mh, 11)) + ((ml >> 10) & 1u);
+    const unsigned long long bits = r + ((unsigned long long)(unsigned)(be - 1) << 52);
+    const unsigned rh = (unsigned)(bits >> 32) | ((unsigned)(sign >> 32) & 0x80000000u);
+    return m0 ? __hiloint2double((int)rh, (int)(unsigned)bits) : 0.0;
+}
+
+// The same for any exponents; a NaN or infinity in the panel (marked row exponents) must
+// reach the next pivot test as NaN.
+__device__ __noinline__ double level_sum_any(long long v, int er, int ec) {
+    if (er == kBadExp || ec == kBadExp) return __longlong_as_double(0x7ff8000000000000LL);
+    return ldexp((double)v, max(-2000, min(2000, er + ec - 54)));
 }
 
 // kFirst, kRest: A_ij -= A_ik A_jk^T over the trailing lower tiles (SYRK/GEMM);
@@ -188,9 +200,16 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
     uint8_t* sA = oz_smem;
     uint8_t* sB = oz_smem + kSlices * kPlaneA;
     // work item w = (block z, super-tile): row tiles i0 = k + 1 + 2u, i0 + 1 and
-    // column tile j = k + 1 + jj <= i0 + 1 (SYRK) or j = k (TRSM)
-    auto decode = [&](int w, int& z, int& i0, int& j) {
-        z = w / tiles_per_block;
+    // column tile j = k + 1 + jj <= i0 + 1 (SYRK) or j = k (TRSM).  Contiguous items per
+    // CTA: neighbours share the row slab (SYRK) or the column tile (TRSM), which then
+    // stays in shared memory, and each follows from the one before.
+    const int w0 = (int)((int64_t)nwork * blockIdx.x / gridDim.x);
+    const int w1 = (int)((int64_t)nwork * (blockIdx.x + 1) / gridDim.x);
+    struct Item {
+        int z, i0, j;
+    };
+    auto first_item = [&](int w) {
+        const int z = w / tiles_per_block;
         int u = 0, jj = w - z * tiles_per_block;
         if constexpr (kPart == kRest) {
             while (true) {
@@ -204,27 +223,32 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
             u = jj;
             jj = kTrsm ? -1 : 0;
         }
-        i0 = k + 1 + 2 * u;
-        j = k + 1 + jj;
+        return Item{z, k + 1 + 2 * u, k + 1 + jj};
     };
-    // contiguous work items per CTA: neighbours share the row slab (SYRK) or the column
-    // tile (TRSM), which then stays in shared memory
-    const int w0 = (int)((int64_t)nwork * blockIdx.x / gridDim.x);
-    const int w1 = (int)((int64_t)nwork * (blockIdx.x + 1) / gridDim.x);
-    auto issue_loads = [&](int w) {
-        int z, i0, j, zp = -1, ip = -1, jp = -1;
-        decode(w, z, i0, j);
-        if (w > w0) decode(w - 1, zp, ip, jp);
-        const bool la = z != zp || i0 != ip, lb = z != zp || j != jp;
-        const uint8_t* Sz = S + (size_t)z * kSlices * plane_bytes;
+    auto next_item = [&](Item t) {
+        if constexpr (kPart == kRest) {
+            // columns of the row pair: up to its own diagonal (or the last tile)
+            if (t.j < min(t.i0 + 1, nt - 1)) return Item{t.z, t.i0, t.j + 1};
+            t.j = k + 2;
+        }
+        t.i0 += 2;
+        if (t.i0 >= nt) {
+            t.i0 = k + 1;
+            ++t.z;
+        }
+        return t;
+    };
+    auto issue_loads = [&](Item t, Item prev, bool first) {
+        const bool la = first || t.z != prev.z || t.i0 != prev.i0, lb = first || t.z != prev.z || t.j != prev.j;
+        const uint8_t* Sz = S + (size_t)t.z * kSlices * plane_bytes;
         mbar_expect_tx(&bar_load, kSlices * ((la ? kPlaneA : 0u) + (lb ? kPlaneB : 0u)));
         if (la)
             for (int p = 0; p < kSlices; ++p)
-                bulk_g2s(sA + p * kPlaneA, Sz + (size_t)p * plane_bytes + (size_t)i0 * T * kRowBytes, kPlaneA,
+                bulk_g2s(sA + p * kPlaneA, Sz + (size_t)p * plane_bytes + (size_t)t.i0 * T * kRowBytes, kPlaneA,
                          &bar_load);
         if (lb)
             for (int q = 0; q < kSlices; ++q)
-                bulk_g2s(sB + q * kPlaneB, Sz + (size_t)q * plane_bytes + (size_t)j * T * kRowBytes, kPlaneB,
+                bulk_g2s(sB + q * kPlaneB, Sz + (size_t)q * plane_bytes + (size_t)t.j * T * kRowBytes, kPlaneB,
                          &bar_load);
     };
 
@@ -252,7 +276,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
         constexpr uint32_t idesc = instr_desc(1, kSlabRows, T);  // BF16 x BF16 -> F32, 128 x 64
         const bool leader = elect_one();
         const uint64_t a0 = smem_desc(smem_u32(sA), 128, 1024), b0 = smem_desc(smem_u32(sB), 128, 1024);
-        if (leader && w0 < w1) issue_loads(w0);
+        Item item = {}, next = {};
+        if (w0 < w1) item = first_item(w0);
+        if (leader && w0 < w1) issue_loads(item, item, true);
         __syncwarp();
         bool ok = true;
         int it = 0;
@@ -263,76 +289,90 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
             if (!ok) break;
             tc_fence_after();
             if (leader) {
-#pragma unroll 1
-                for (int L = 2; L <= kSlices + 1; ++L) {
-                    const uint32_t d = tmem + 64u * (uint32_t)(L - 2);
-                    uint32_t acc = 0;
-#pragma unroll 1
-                    for (int p = 1; p < L; ++p) {  // level L <= 9: slices p and L - p, both <= 8
-                        const uint64_t ap = a0 + (uint64_t)(((p - 1) * kPlaneA) >> 4);
-                        const uint64_t bq = b0 + (uint64_t)(((L - p - 1) * kPlaneB) >> 4);
 #pragma unroll
-                        for (int ks = 0; ks < T / 16; ++ks) {
-                            mma_ss(d, ap + (uint64_t)(ks * 16), bq + (uint64_t)(ks * 16), idesc, acc);
-                            acc = 1;
-                        }
-                    }
-                }
+                for (int L = 2; L <= kSlices + 1; ++L)
+#pragma unroll
+                    for (int p = 1; p < L; ++p)  // level L <= 9: slices p and L - p, both <= 8
+#pragma unroll
+                        for (int ks = 0; ks < T / 16; ++ks)
+                            mma_ss(tmem + 64u * (uint32_t)(L - 2), a0 + (uint64_t)(((p - 1) * kPlaneA) / 16 + ks * 16),
+                                   b0 + (uint64_t)(((L - p - 1) * kPlaneB) / 16 + ks * 16), idesc,
+                                   p > 1 || ks > 0 ? 1u : 0u);
                 tc_commit(&bar_mma);
             }
             __syncwarp();
             if (w + 1 < w1) {
+                next = next_item(item);
                 // the MMAs have consumed the slices: fetch the next item's
                 ok = __all_sync(0xffffffffu, mbar_wait(&bar_mma, (uint32_t)(it & 1), &s_abort, err));
-                if (ok && leader) issue_loads(w + 1);
+                if (ok && leader) issue_loads(next, item, false);
+                item = next;
                 __syncwarp();
             }
         }
     } else {
         // ------------------------------------------------------------ epilogue
         // warp v owns tensor-memory lanes (rows) 32 (v % 4) .. + 31 and columns
-        // 16 (v / 4) .. + 15 of the super-tile
-        const int rl = 32 * (warp & 3) + lane, c0 = 16 * (warp >> 2);
-        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+        // 16 (v / 4) .. + 15 of the super-tile.  The accumulators are read in the 16 x 256
+        // bit form: a thread gets columns 2 (lane % 4), + 1 of two blocks of eight for rows
+        // lane / 4 + 8 rr, so that a load or store of the matrix takes 64 bytes of eight
+        // rows; with a row per lane it was 16 bytes of 32 rows, and the address path of
+        // these accesses alone took 8000 clocks per item.
+        const int rl = 32 * (warp & 3) + (lane >> 2), cl = 16 * (warp >> 2) + 2 * (lane & 3);
+        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16, col_base = 16u * (uint32_t)(warp >> 2);
         int it = 0;
+        Item item = {};
+        if (w0 < w1) item = first_item(w0);
         for (int w = w0; w < w1; ++w, ++it) {
-            int z, i0, j;
-            decode(w, z, i0, j);
+            const int z = item.z, i0 = item.i0, j = item.j;
+            item = next_item(item);
             const int64_t r = (int64_t)i0 * T + rl;
-            const int rtile = i0 + rl / T;
+            const int rtile = i0 + (warp & 3) / 2;  // of the warp's 32 rows
             const bool mine = rtile < nt && (kTrsm || j <= rtile);
-            const int er = mine ? E[(int64_t)z * rows_pad + r] : 0;
-            const int ecl = E[(int64_t)z * rows_pad + (int64_t)j * T + c0 + (lane & 15)];
-            double2* Crow = reinterpret_cast<double2*>(A + (int64_t)z * ld * ld + r * ld + (int64_t)j * T + c0);
-            // half of the entries to update are on their way before the MMAs are waited for
-            double2 cv[2][4];
-            if (!kTrsm && mine) {
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(Crow + 4));
+            int er[4], ec[4];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) cv[0][c] = Crow[c];
+            for (int rr = 0; rr < 4; ++rr) er[rr] = mine ? E[(int64_t)z * rows_pad + r + 8 * rr] : 0;
+#pragma unroll
+            for (int cb = 0; cb < 2; ++cb) {
+                const int2 e2 = *reinterpret_cast<const int2*>(E + (int64_t)z * rows_pad + (int64_t)j * T + cl + 8 * cb);
+                ec[2 * cb] = e2.x;
+                ec[2 * cb + 1] = e2.y;
+            }
+            double* C0 = A + (int64_t)z * ld * ld + r * ld + (int64_t)j * T + cl;
+            auto entry = [&](int rr, int cb) { return reinterpret_cast<double2*>(C0 + (int64_t)(8 * rr) * ld + 8 * cb); };
+            // half of the entries to update are on their way before the MMAs are waited for
+            double2 cv[4][2];
+            if (!kTrsm && mine) {
+#pragma unroll
+                for (int rr = 0; rr < 2; ++rr) {
+                    cv[rr][0] = *entry(rr, 0);
+                    cv[rr][1] = *entry(rr, 1);
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(entry(rr + 2, 0)));
+                }
             }
             if (!__all_sync(0xffffffffu, mbar_wait(&bar_mma, (uint32_t)(it & 1), &s_abort, err))) break;
             tc_fence_after();
-            // pairs of levels as exact 32-bit integers, acc_L 2^7 + acc_{L+1} (below 2^29)
-            int q[4][16];
+            // pairs of levels as exact 32-bit integers, acc_L 2^7 + acc_{L+1} (below 2^29):
+            // q[pair][rr][2 cb + e]
+            int q[4][4][4];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
+            for (int hh = 0; hh < 2; ++hh) {  // rows 16 hh .. + 15 of the warp's
 #pragma unroll
                 for (int pr = 0; pr < 4; ++pr) {
                     uint32_t va[8], vb[8];
-                    const uint32_t at = tmem + lane_base + 128u * (uint32_t)pr + (uint32_t)(c0 + 8 * half);
-                    tmem_ld8(at, va);
-                    tmem_ld8(at + 64u, vb);
+                    const uint32_t at = tmem + lane_base + ((uint32_t)(16 * hh) << 16) + 128u * (uint32_t)pr + col_base;
+                    tmem_ld_16x256b_x2(at, va);
+                    tmem_ld_16x256b_x2(at + 64u, vb);
                     tmem_wait_ld();
                     // exact conversion of an FP32 integer below 2^22: its bits after adding
                     // 1.5 * 2^23 are the integer plus those of the constant
                     constexpr float kMagicF = 12582912.0f;
                     constexpr unsigned kMagicBits = 0x4b400000u;
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
+                    for (int c = 0; c < 8; ++c) {  // register c: column block c / 4, row c / 2 % 2, column c % 2
                         const unsigned ba = __float_as_uint(__uint_as_float(va[c]) + kMagicF);
                         const unsigned bb = __float_as_uint(__uint_as_float(vb[c]) + kMagicF);
-                        q[pr][8 * half + c] = (int)(ba * 128u + bb - 129u * kMagicBits);
+                        q[pr][2 * hh + (c >> 1 & 1)][2 * (c >> 2) + (c & 1)] = (int)(ba * 128u + bb - 129u * kMagicBits);
                     }
                 }
             }
@@ -340,26 +380,33 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_read);
-            if (!mine) continue;  // (warp-uniform: a warp's 32 rows lie in one tile)
+            if (!mine) continue;  // (warp-uniform)
+            if constexpr (!kTrsm) {
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                if (!kTrsm && half == 0) {
+                for (int rr = 2; rr < 4; ++rr) {
+                    cv[rr][0] = *entry(rr, 0);
+                    cv[rr][1] = *entry(rr, 1);
+                }
+            }
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) cv[1][c] = Crow[4 + c];
+            for (int rr = 0; rr < 4; ++rr) {
+                double t[4];
+                bool extreme = false;
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    t[c] = level_sum(level_int(q[0][rr][c], q[1][rr][c], q[2][rr][c], q[3][rr][c]),
+                                     er[rr] + ec[c] - 54, extreme);
+                if (extreme) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        t[c] = level_sum_any(level_int(q[0][rr][c], q[1][rr][c], q[2][rr][c], q[3][rr][c]), er[rr], ec[c]);
                 }
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const int cc = 8 * half + c;
-                    const int ec = __shfl_sync(0xffffffffu, ecl, cc);
-                    double t = level_sum(q[0][cc], q[1][cc], q[2][cc], q[3][cc], er + ec - 54);
-                    // a NaN or infinity in the panel must reach the next pivot test as NaN
-                    if (er == kBadExp || ec == kBadExp) t = __longlong_as_double(0x7ff8000000000000LL);
-                    double& dst = c & 1 ? cv[half][c / 2].y : cv[half][c / 2].x;
-                    if constexpr (kTrsm) dst = t;
-                    else dst -= t;
+                for (int cb = 0; cb < 2; ++cb) {
+                    double2 o = make_double2(t[2 * cb], t[2 * cb + 1]);
+                    if constexpr (!kTrsm) o = make_double2(cv[rr][cb].x - o.x, cv[rr][cb].y - o.y);
+                    *entry(rr, cb) = o;
                 }
-#pragma unroll
-                for (int c = 0; c < 4; ++c) Crow[4 * half + c] = cv[half][c];
             }
         }
     }
