@@ -1273,9 +1273,9 @@ ap_status ap_residual(ap_ctx* ctx, const float* B_dev, int32_t c, const float* W
     AP_TRY(launch_full_residual(ctx, ctx->Bp, ctx->Tmp, ctx->R, 0));
     AP_CK(launch_unpad_copy(ctx->R, ctx->n, Cp, R_dev, c, ctx->st));
     ++ctx->launches;
+    if (!waits) return leave(ctx);
     SolveState now = {};
-    if (waits) AP_TRY(read_state(ctx, &now));
-    AP_TRY(leave(ctx));
+    AP_TRY(read_state(ctx, &now));  // (waits for everything: nothing is left to order)
     return now.tc_err ? AP_ERR_TIMEOUT : AP_OK;
 }
 
@@ -1316,8 +1316,7 @@ ap_status ap_predict_mean(ap_ctx* ctx, const float* w_dev, const float* Xs_dev, 
     AP_CK(launch_kmv(ctx->kernel, kp, ctx->D, 1, ctx->st));
     ++ctx->launches;
     SolveState now = {};
-    AP_TRY(read_state(ctx, &now));
-    AP_TRY(leave(ctx));
+    AP_TRY(read_state(ctx, &now));  // (waits for everything: nothing is left to order)
     return now.nan_flag ? AP_ERR_NAN : AP_OK;
 }
 
@@ -1367,8 +1366,7 @@ ap_status ap_grad_quadforms(ap_ctx* ctx, const float* U_dev, const float* V_dev,
     AP_CK(launch_pad_copy(U_dev, ctx->n, c, ctx->Tmp, Cp, ctx->st));
     AP_CK(launch_pad_copy(V_dev, ctx->n, c, ctx->Bp, Cp, ctx->st));
     ctx->launches += 2;
-    AP_TRY(grad_quadforms_impl(ctx, ctx->Tmp, ctx->Bp, Cp, alpha_host, c, out_host));
-    return leave(ctx);
+    return grad_quadforms_impl(ctx, ctx->Tmp, ctx->Bp, Cp, alpha_host, c, out_host);
 }
 
 ap_status ap_mll_grad(ap_ctx* ctx, const float* y_dev, int32_t n_probes, const float* Z_dev, float* grad_host,

@@ -457,8 +457,10 @@ template <int KERN, int D, int C, int RM>
 cudaError_t launch_kmv_rm(const KmvParams& p, cudaStream_t st) {
     const size_t smem = sizeof(float) * kmv_smem_floats<D, C, RM>();
     auto fn = kmv_fp32_kernel<KERN, D, C, RM>;
-    cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+    if constexpr (sizeof(float) * kmv_smem_floats<D, C, RM>() > 48 * 1024) {
+        cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err != cudaSuccess) return err;
+    }
     return launch_dependent(fn, dim3((unsigned)p.epi.ntiles, (unsigned)p.epi.S, (unsigned)p.G), kKmvThreads, smem, st,
                             p.dependent, p, (unsigned)p.epi.S);
 }
