@@ -88,18 +88,6 @@ struct Cfg {
     static_assert(kSmem <= 220 * 1024, "shared memory");
 };
 
-// x0, x1 as BF16 parts: hi cut off, mid and lo rounded to nearest (what is dropped of
-// the products then has no preferred sign).
-__device__ __forceinline__ void split3_rn(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-    constexpr uint32_t kTop = 0xFFFF0000u;
-    const uint32_t b0 = __float_as_uint(x0), b1 = __float_as_uint(x1);
-    hi = __byte_perm(b0, b1, 0x7632);
-    const float r0 = x0 - __uint_as_float(b0 & kTop), r1 = x1 - __uint_as_float(b1 & kTop);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(mid) : "f"(r1), "f"(r0));
-    const float s0 = r0 - __uint_as_float(mid << 16), s1 = r1 - __uint_as_float(mid & kTop);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(s1), "f"(s0));
-}
-
 // Eight consecutive K values k0 .. k0 + 7 of point i's operand into the three planes at
 // dst, dst + plane, dst + 2 plane: [first | second | 0], the U half scaled by alpha.
 template <int C>

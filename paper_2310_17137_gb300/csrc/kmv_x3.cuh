@@ -572,42 +572,29 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
             // item: column k of V and 8 consecutive rows = one 16-byte core row per plane
             for (int t = ct; t < C * (kChunk / 8); t += 64) {
                 const int k = t % C, j8 = t / C;
-                uint32_t w[3][4];
-                int flags = 0;
+                float v[8];
+                unsigned big = 0;  // largest magnitude, as bits
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int row = 8 * j8 + j;
-                    float v = row < cnt ? sv[row * C + k] : 0.0f;
-                    if (!(fabsf(v) <= 3.402823466e38f)) {
-                        flags |= v > 0.0f ? 1 : (v < 0.0f ? 2 : 4);
-                        v = 0.0f;
-                    }
-                    // hi rounds towards zero (v may be the largest float), mid and lo to nearest
-                    const uint32_t hb = __float_as_uint(v) & 0xFFFF0000u;
-                    const float r1 = v - __uint_as_float(hb);
-                    uint32_t mb;
-                    asm("{\n\t.reg .b16 h, z;\n\tmov.b16 z, 0;\n\tcvt.rn.bf16.f32 h, %1;\n\tmov.b32 %0, {z, h};\n\t}"
-                        : "=r"(mb)
-                        : "f"(r1));
-                    const float r2 = r1 - __uint_as_float(mb);
-                    uint32_t lb;
-                    asm("{\n\t.reg .b16 h, z;\n\tmov.b16 z, 0;\n\tcvt.rn.bf16.f32 h, %1;\n\tmov.b32 %0, {z, h};\n\t}"
-                        : "=r"(lb)
-                        : "f"(r2));
-                    if (j & 1) {
-                        w[0][j >> 1] |= hb;
-                        w[1][j >> 1] |= mb;
-                        w[2][j >> 1] |= lb;
-                    } else {
-                        w[0][j >> 1] = hb >> 16;
-                        w[1][j >> 1] = mb >> 16;
-                        w[2][j >> 1] = lb >> 16;
-                    }
+                    v[j] = row < cnt ? sv[row * C + k] : 0.0f;
+                    big = max(big, __float_as_uint(v[j]) << 1);
                 }
-                if (flags) {
+                if (big >= 0xFF000000u) {  // an infinity or NaN among the eight
+                    int flags = 0;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (!(fabsf(v[j]) <= 3.402823466e38f)) {
+                            flags |= v[j] > 0.0f ? 1 : (v[j] < 0.0f ? 2 : 4);
+                            v[j] = 0.0f;
+                        }
                     atomicOr(&nf[k], flags);
                     s_any[c % kFlagRing] = 1;
                 }
+                // hi rounds towards zero (v may be the largest float), mid and lo to nearest
+                uint32_t w[3][4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) split3_rn(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
 #pragma unroll
                 for (int pl = 0; pl < 3; ++pl) {
                     const int vr = pl * C + k;
