@@ -51,7 +51,8 @@ namespace ap {
 namespace tc {
 
 constexpr int kRows = 128;
-constexpr int kChunk = kTcChunk;  // columns of the block per chunk
+constexpr int kChunk = 128;  // columns of the block per chunk
+static_assert(kChunk == kTcChunk, "Delta's operand layout");
 constexpr int kStages = 4;
 constexpr int kBufs = 3;     // S/P tensor-memory buffers
 constexpr int kColsPerWarp = 32;                   // columns of a chunk per work item (two 16-column units)
