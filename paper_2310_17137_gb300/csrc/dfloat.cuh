@@ -119,10 +119,12 @@ __device__ __forceinline__ P2 add(P2 a, P2 b) {
 __device__ __forceinline__ P2 exp2_neg(P2 t) {
     // beyond 125 the result is 0 (set at the end); k by the rounding of a large sum
     const float2 th = make_float2(fminf(t.h.x, 126.0f), fminf(t.h.y, 126.0f));
+    // (a large t's low part would overflow the polynomial; a NaN stays in the low part)
+    const float2 tl = make_float2(t.h.x > 126.0f ? 0.0f : t.l.x, t.h.y > 126.0f ? 0.0f : t.l.y);
     const float2 big = dup(12582912.0f);  // 1.5 * 2^23
     const float2 kb = add(th, big);
     const float2 k = sub(kb, big);
-    const P2 r = fast_two_sum(sub(th, k), t.l);
+    const P2 r = fast_two_sum(sub(th, k), tl);
     const P2 z = mul(P2{dup(kLn2H), dup(kLn2L)}, r);
     const float2 zh = z.h, nzh = sub(make_float2(0.0f, 0.0f), z.h);
     float2 q = dup(-1.0f / 362880.0f);

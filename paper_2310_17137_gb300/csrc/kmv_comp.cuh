@@ -99,9 +99,10 @@ __global__ void __launch_bounds__(kKmvThreads) kmv_comp_kernel(const KmvParams p
         __syncthreads();
         if (AP_CHK(cb >= 0 && cb + cnt <= p.nb) && AP_CHK(cb - col0 >= 0 && cb - col0 + cnt <= ncols)) {
             for (int t = tid; t < kKmvTN * D; t += kKmvThreads) {
-                const int j = t / D, k = t % D;  // dimension-major, zero past the last column
-                s_xh[k * kKmvTN + j] = j < cnt ? p.Xb[cb * D + t] : 0.0f;
-                s_xl[k * kKmvTN + j] = j < cnt ? p.Xb_lo[cb * D + t] : 0.0f;
+                const int j = t / D, k = t % D;  // dimension-major, the last column repeated
+                const int64_t src = (cb + min(j, cnt - 1)) * D + k;
+                s_xh[k * kKmvTN + j] = p.Xb[src];
+                s_xl[k * kKmvTN + j] = p.Xb_lo[src];
             }
             for (int t = tid; t < kKmvTN * C; t += kKmvThreads) s_v[t] = t < cnt * C ? p.V[(cb - col0) * C + t] : 0.0f;
         }
