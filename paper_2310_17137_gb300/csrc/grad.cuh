@@ -90,9 +90,10 @@ struct Cfg {
 
 // Eight consecutive K values k0 .. k0 + 7 of point i's operand into the three planes at
 // dst, dst + plane, dst + 2 plane: [first | second | 0], the U half scaled by alpha.
+// vec: U and V start on 16-byte boundaries (the caller's own arrays need not).
 template <int C>
-__device__ __forceinline__ void split_operand(const GradParams& p, int64_t i, int k0, bool u_first, uint8_t* dst,
-                                              uint32_t plane) {
+__device__ __forceinline__ void split_operand(const GradParams& p, int64_t i, int k0, bool u_first, bool vec,
+                                              uint8_t* dst, uint32_t plane) {
     float v[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = 0.0f;
@@ -100,10 +101,16 @@ __device__ __forceinline__ void split_operand(const GradParams& p, int64_t i, in
         if constexpr (C % 8 == 0) {  // the eight values lie in one half
             const bool is_u = (k0 < C) == u_first;
             const int c = k0 < C ? k0 : k0 - C;
-            const float4* src = reinterpret_cast<const float4*>((is_u ? p.U : p.V) + i * C + c);
-            const float4 x = __ldg(src), y = __ldg(src + 1);
-            v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
-            v[4] = y.x, v[5] = y.y, v[6] = y.z, v[7] = y.w;
+            const float* src = (is_u ? p.U : p.V) + i * C + c;
+            if (vec) {
+                const float4 x = __ldg(reinterpret_cast<const float4*>(src));
+                const float4 y = __ldg(reinterpret_cast<const float4*>(src) + 1);
+                v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+                v[4] = y.x, v[5] = y.y, v[6] = y.z, v[7] = y.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = __ldg(src + j);
+            }
             if (is_u) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[j] *= p.alpha[c + j];
@@ -182,6 +189,7 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    const bool vec = ((reinterpret_cast<uintptr_t>(p.U) | reinterpret_cast<uintptr_t>(p.V)) & 15) == 0;
 
     if (warp < K::kXformWarps) {
         // ------------------------------------------------------- transform warps
@@ -218,7 +226,7 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
                     xa[r][2 * k + 1] = make_float2(v.z, v.w);
                 }
                 for (int k8 = slot; k8 < K::KC / 8; k8 += K::kSlots)
-                    split_operand<C>(p, i, 8 * k8, true,
+                    split_operand<C>(p, i, 8 * k8, true, vec,
                                      s_a + r * K::kPlaneA + ((row >> 3) * (K::KC / 8) + k8) * 128 + (row & 7) * 16,
                                      R * K::kPlaneA);
                 if (slot == 0 && first_chunk && i < n) {
@@ -427,11 +435,12 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
             uint8_t* st = s_stage + (size_t)stage * K::kStageBytes;
             const int cnt = (int)min((int64_t)kChunk, n - q * kChunk);
             if (cnt < kChunk)
-                for (int t = cnt * D + ct; t < kChunk * D; t += 32 * kConvWarps) reinterpret_cast<float*>(st)[t] = 0.0f;
+                for (int t = cnt * D + ct; t < kChunk * D; t += 32 * kConvWarps)
+                    reinterpret_cast<float*>(st)[t] = reinterpret_cast<const float*>(st)[(cnt - 1) * D + t % D];
 #pragma unroll 2
             for (int t = ct; t < kChunk * (K::KC / 8); t += 32 * kConvWarps) {
                 const int j = t % kChunk, k8 = t / kChunk;  // (neighbouring lanes fill one core matrix)
-                split_operand<C>(p, q * kChunk + j, 8 * k8, false,
+                split_operand<C>(p, q * kChunk + j, 8 * k8, false, vec,
                                  st + K::kXBytes + ((j >> 3) * (K::KC / 8) + k8) * 128 + (j & 7) * 16, K::kPlaneB);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

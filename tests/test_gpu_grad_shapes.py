@@ -37,3 +37,25 @@ def test_quadforms_over_shapes(n, d, c, kern):
     mag = oracle.grad_quadforms(h, X, np.abs(U), np.abs(V), np.abs(alpha))
     assert np.all(np.abs(first - ref) <= 1e-5 * mag + 1e-12), np.abs(first - ref) / mag
     ap.ap_destroy(ctx)
+
+
+@pytest.mark.parametrize("c", [1, 4, 16, 32])
+def test_static_quadforms_take_arrays_of_any_float_alignment(c):
+    """ap_grad_quadforms_static reads the caller's U and V in place: an array that starts
+    4 bytes past a 16-byte boundary gives the same bits as an aligned one."""
+    n = 300
+    p = wl.random_problem(n, 4, 128, c, wl.MATERN32, 0.1, 42)
+    ctx = ap.ap_create(_t(p.X), ap.Hyper(p.kernel, p.lengthscale, p.outputscale, p.noise), ap.ap_opts_default(block=128))
+    rng = np.random.default_rng(10)
+    U, V = _t(rng.standard_normal((n, c))), _t(rng.standard_normal((n, c)))
+    alpha = rng.uniform(-1, 1, c)
+    want = ap.ap_grad_quadforms_static(ctx, U, V, alpha)
+
+    def shifted(t):
+        flat = torch.empty(n * c + 1, device="cuda:0")[1:]
+        flat.copy_(t.reshape(-1))
+        return flat.view(n, c)
+
+    for a, b in [(shifted(U), V), (U, shifted(V)), (shifted(U), shifted(V))]:
+        assert np.array_equal(ap.ap_grad_quadforms_static(ctx, a, b, alpha), want)
+    ap.ap_destroy(ctx)
