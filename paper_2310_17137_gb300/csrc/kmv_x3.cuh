@@ -23,7 +23,7 @@
 // 1.1e-7 on sums of equal sign (drains every 128 columns: 1.7e-7 for 2 % less time,
 // every 32: 0.8e-7 for 8 % more).
 // Measured time (GB300): n = 131,072, d = 3, c = 16, n^2 entries of Matern-5/2 19.1 ->
-// 12.7 ms; n = 65,536, d = 8, c = 32, 4096 columns of Matern-3/2 665 -> 310 us, at
+// 12.3 ms; n = 65,536, d = 8, c = 32, 4096 columns of Matern-3/2 665 -> 302 us, at
 // 70 % of the issue slots and 59 % of the FMA pipe (tensor pipe 15 %).
 // Infinities and NaNs in V are taken out of the split, noted
 // per column and chunk, and added by the drain.
@@ -57,7 +57,8 @@ constexpr int kStages = 3;    // shared-memory operand stages
 constexpr int kSlots = 4;     // transform warps per lane quarter
 constexpr int kXformWarps = 4 * kSlots;
 constexpr int kConvWarps = 2;
-constexpr int kFlagRing = 8;  // chunks of non-finite flags: more than can be in flight
+constexpr int kFlagRing = 8;  // chunks of non-finite flags, half of them being cleared ahead
+static_assert(kFlagRing >= 2 * (kStages + 1), "a cleared flag is neither in use nor set yet");
 constexpr uint32_t kBufCols = 48;  // tensor-memory columns of one P buffer: 2 units x 3 planes x 8
 
 template <int D, int C, int R>
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
         uint32_t sphase = 0, use = 0;
         if (total > 0) load_rows(g);
         for (int c = 0; c < total && ok; ++c) {
-            // the copy itself, then the tail of a short chunk (zeroed by the splitters)
+            // the copy itself, then the tail of a short chunk (filled by the splitters)
             ok = mbar_wait(&bar_full[stage], sphase, &s_abort, p.err) &&
                  mbar_wait(&bar_ready[stage], sphase, &s_abort, p.err);
             ok = __all_sync(0xffffffffu, ok);
@@ -561,14 +562,13 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
             uint8_t* v3 = st + K::kXBytes + K::kVBytes;
             const int cnt = (int)min((int64_t)kChunk, ncols - (int64_t)q * kChunk);
             if (cnt < kChunk)
-                for (int t = cnt * D + ct; t < kChunk * D; t += 64) sx[t] = 0.0f;
+                for (int t = cnt * D + ct; t < kChunk * D; t += 64) sx[t] = sx[(cnt - 1) * D + t % D];
             int* nf = s_nf[c % kFlagRing];
-            if (s_any[c % kFlagRing]) {  // left by the chunk kFlagRing before this one
-                asm volatile("bar.sync 2, 64;" ::: "memory");
-                if (ct < C) nf[ct] = 0;
-                if (ct == 0) s_any[c % kFlagRing] = 0;
-                asm volatile("bar.sync 2, 64;" ::: "memory");
-            }
+            // The flags of four chunks ahead: their last user, chunk c - 4, is drained (this
+            // stage was free, so the MMAs of chunk c - 3 began, after that drain), and chunk
+            // c + 4 is not split before this chunk is complete.
+            if (ct < C) s_nf[(c + kFlagRing / 2) % kFlagRing][ct] = 0;
+            if (ct == 0) s_any[(c + kFlagRing / 2) % kFlagRing] = 0;
             // item: column k of V and 8 consecutive rows = one 16-byte core row per plane
             for (int t = ct; t < C * (kChunk / 8); t += 64) {
                 const int k = t % C, j8 = t / C;
