@@ -86,6 +86,7 @@ struct ap_ctx {
     // flags and tickets of `state` and the products are known to be zero: set when a call
     // has read clean flags, so that the next one need not clear them
     bool clean = false;
+    bool timed_out = false;  // a wait ran out: its kernel's arrival tickets may be partial
     int64_t gpart_alloc = 0;
     unsigned* ticket = nullptr;
     int* sel = nullptr;
@@ -232,7 +233,7 @@ ap_status clear_flags(ap_ctx* ctx) {
         if (ctx->gtick) AP_CK(cudaMemsetAsync(ctx->gtick, 0, sizeof(unsigned) * ctx->gtick_alloc, ctx->st));
         if (ctx->tc_tick) AP_CK(cudaMemsetAsync(ctx->tc_tick, 0, sizeof(int) * ctx->num_sms, ctx->st));
     }
-    ctx->clean = false;
+    ctx->clean = ctx->timed_out = false;
     return AP_OK;
 }
 
@@ -241,6 +242,7 @@ ap_status read_state(ap_ctx* ctx, SolveState* out) {
     AP_CK(cudaMemcpyAsync(out, ctx->state, sizeof(SolveState), cudaMemcpyDeviceToHost, ctx->st));
     AP_CK(cudaStreamSynchronize(ctx->st));
     ctx->clean = !out->nan_flag && !out->tc_err;
+    ctx->timed_out |= out->tc_err != 0;
     return AP_OK;
 }
 
@@ -1266,7 +1268,7 @@ ap_status ap_residual(ap_ctx* ctx, const float* B_dev, int32_t c, const float* W
     ctx->r_tracked_c = 0;
     AP_TRY(enter(ctx));
     const bool waits = Cp >= kX3MinC && !use_compensated(ctx);  // the tensor-core form runs
-    if (waits) AP_TRY(clear_flags(ctx));
+    if (waits || ctx->timed_out) AP_TRY(clear_flags(ctx));
     AP_CK(launch_pad_copy(B_dev, ctx->n, c, ctx->Bp, Cp, ctx->st));
     AP_CK(launch_pad_copy(W_dev, ctx->n, c, ctx->Tmp, Cp, ctx->st));
     ctx->launches += 2;
