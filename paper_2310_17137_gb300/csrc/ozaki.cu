@@ -65,7 +65,7 @@ constexpr uint32_t kOzSmem = kSlices * (kPlaneA + kPlaneB); // 192 KB
 constexpr int kEpiWarps = 16;                             // four per tensor-memory lane quarter
 constexpr int kOzThreads = (kEpiWarps + 1) * 32;          // and one that issues copies and MMAs
 constexpr uint32_t kRowBytes = T * 2;                       // one slice row (64 BF16)
-constexpr int kBadExp = -(1 << 30);  // row exponent marking a non-finite panel row
+constexpr int kBadExp = -(1 << 28);  // row exponent marking a non-finite panel row (two add up without overflow)
 
 // byte offset of (row, kk) in a slice plane: K-major core matrices of 8 rows x
 // 8 BF16, 8 K-cores (1 KB) per 8-row group
@@ -150,7 +150,7 @@ __device__ __forceinline__ long long level_int(int h1, int h2, int l1, int l2) {
 // 2^e0 v rounded to a double (half away from zero), for results in the normal range:
 // normalised and rounded with integer instructions and no branches, so that a thread's
 // sixteen chains run side by side.  `extreme` is set when the exponent leaves the
-// normal doubles (also for the marked row exponents): the result is then not usable.
+// normal doubles: the result is then not usable.
 __device__ __forceinline__ double level_sum(long long v, int e0, bool& extreme) {
     const long long sign = v >> 63;
     const unsigned long long m0 = (unsigned long long)((v ^ sign) - sign);
@@ -338,6 +338,10 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
                 ec[2 * cb] = e2.x;
                 ec[2 * cb + 1] = e2.y;
             }
+            // (the slices of a non-finite row are zero, so its mark is the only sign)
+            bool marked = false;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) marked |= er[t] == kBadExp || ec[t] == kBadExp;
             double* C0 = A + (int64_t)z * ld * ld + r * ld + (int64_t)j * T + cl;
             auto entry = [&](int rr, int cb) { return reinterpret_cast<double2*>(C0 + (int64_t)(8 * rr) * ld + 8 * cb); };
             // half of the entries to update are on their way before the MMAs are waited for
@@ -391,7 +395,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
 #pragma unroll
             for (int rr = 0; rr < 4; ++rr) {
                 double t[4];
-                bool extreme = false;
+                bool extreme = marked;
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
                     t[c] = level_sum(level_int(q[0][rr][c], q[1][rr][c], q[2][rr][c], q[3][rr][c]),
