@@ -48,7 +48,7 @@ import workloads as wl  # noqa: E402
 
 METRIC = "AP time-to-tol & kernel-entries/s, BF16+refine vs FP32; serve p50/p99"
 T_START = time.perf_counter()
-# forms of the residual update: FP32 SIMT, tensor-core BF16 hi/lo
+# forms of the residual update: FP32 entries (contraction in split precision), BF16 hi/lo
 FORMS = {"fp32": lambda ap: ap.AP_FP32, "bf16": lambda ap: ap.AP_BF16_REFINE}
 DTYPES = {"fp32": "f32", "bf16": "bf16"}
 FP32_LANES_PER_SM = 128
@@ -140,7 +140,7 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-KERNEL_SOURCES = {"kmv_fp32_update": ["kmv_fp32.cuh", "ap_internal.cuh"],
+KERNEL_SOURCES = {"kmv_fp32_update": ["kmv_x3.cuh", "tcgen05.cuh", "kmv_fp32.cuh", "ap_internal.cuh"],
                   "kmv_tc_update": ["kmv_tc.cu", "tcgen05.cuh", "kmv_fp32.cuh", "ap_internal.cuh"]}
 
 
@@ -523,8 +523,9 @@ def roofline(p, args, t_launch: float, units: float, sm_max: float, sfu=(32.0, 1
         return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if achieved else None,
                 "traffic": traffic_from_profiles("kmv_fp32_update", args.workload, "fp32", units),
-                "kernel": "kmv_fp32_kernel (fused residual update, one AP step)",
-                "per_unit": f"{flops_per_entry} FP32 flop per kernel entry (2c contraction + 3d distance)",
+                "kernel": "kmv_x3_kernel (fused residual update, one AP step)",
+                "per_unit": f"{flops_per_entry} FP32 flop per kernel entry (2c contraction, on the tensor cores "
+                            f"as six BF16 split products, + 3d distance)",
                 "peak_note": f"FP32 FMA pipe: {NUM_SMS} SMs x {FP32_LANES_PER_SM} lanes x 2 flop x "
                              f"{sm_max:.0f} MHz (derived from unit counts and max clock)"}
     # SFU operations per entry: exp2 for every kernel, sqrt for the Matern ones.
@@ -714,7 +715,7 @@ def main():
     ap_.add_argument("--workload", default="matern52_ard")
     ap_.add_argument("--precision", choices=sorted(FORMS), default="bf16",
                      help="form of the timed steps: bf16 = tensor-core BF16 hi/lo with FP32 refinement, "
-                          "fp32 = FP32 SIMT")
+                          "fp32 = FP32 entries, FP32-accurate contraction")
     ap_.add_argument("--refine-every", type=int, default=10)
     ap_.add_argument("--no-compare", action="store_true", help="skip the timed runs of the other forms")
     ap_.add_argument("--min-epochs", type=int, default=11)

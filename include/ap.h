@@ -63,7 +63,9 @@ typedef enum {
 typedef enum { AP_RBF = 0, AP_MATERN32 = 1, AP_MATERN52 = 2 } ap_kernel;
 
 /* Arithmetic of the residual update.
- *   AP_FP32:         kernel blocks and contraction in FP32 (SIMT).
+ *   AP_FP32:         kernel blocks in FP32; contraction in FP32 or, with more than 4
+ *                    right-hand sides, in split precision on the tensor cores (three
+ *                    BF16 parts per operand, FP32 sums: FP32 accuracy).
  *   AP_BF16_REFINE:  kernel blocks and K*Delta on tensor cores with BF16
  *                    operands and FP32 accumulation; accuracy recovered by
  *                    recomputing R = B - K_hat W in the FP32 form (iterative
@@ -237,8 +239,9 @@ ap_status ap_predict_mean(ap_ctx* ctx, const float* w_dev, const float* Xs_dev, 
 /* The fused derivative quadratic forms of Eq. loss_grad_unbiased:
  *   out_host[p] = sum_col alpha_host[col] * U[:,col]^T (dK_hat / dtheta_p) V[:,col]
  * for theta = (l_1..l_d, s, sigma^2): d + 2 doubles.  U_dev, V_dev are n x c
- * (device), alpha_host has c entries.  One pass over all n^2 kernel entries;
- * no kernel block is stored. */
+ * (device), alpha_host has c entries.  One pass over the kernel entries (the
+ * derivatives are symmetric: i < j and the diagonal); no kernel block is stored.
+ * AP_ERR_TIMEOUT when a bounded device wait ran out. */
 ap_status ap_grad_quadforms(ap_ctx* ctx, const float* U_dev, const float* V_dev, int32_t c,
                             const double* alpha_host, double* out_host);
 
@@ -262,7 +265,7 @@ ap_status ap_grad_quadforms(ap_ctx* ctx, const float* U_dev, const float* V_dev,
  *   - c must be 1, 4, 16 or 32: U_dev and V_dev (n x c, device) are read in
  *     place, without a padding copy.
  *   - Scratch: one AP_STATIC_SCRATCH_BYTES device array shared by every call
- *     in the process, holding (D + 2) doubles per block of 128 rows (256 rows
+ *     in the process; (D + 2) doubles per block of 128 rows must fit (256 rows
  *     when D + c <= 40), D = d rounded up to 4, 8, 12, 16, 24 or 32: n up to
  *     about 490k at d = 32 with c = 32 and 3.3M at d <= 8.  A larger problem
  *     returns AP_ERR_SCRATCH_LIMIT before anything is launched.
