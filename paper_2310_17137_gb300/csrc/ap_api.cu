@@ -79,6 +79,7 @@ struct ap_ctx {
     float *gscr = nullptr, *pscr = nullptr;
     unsigned *gtick = nullptr, *ptick = nullptr;
     int64_t gscr_alloc = 0, gtick_alloc = 0, pscr_alloc = 0, ptick_alloc = 0;
+    bool groups_released = false;  // the next solve or residual asks for its area again
     int sol_tpc = 1, sol_maxj = 1;
     // always-present device scalars
     double *norms = nullptr, *gout = nullptr, *gpart = nullptr;
@@ -177,6 +178,7 @@ bool release_groups(ap_ctx* ctx) {
     dfree(ctx, ctx->pscr);
     dfree(ctx, ctx->ptick);
     ctx->gscr_alloc = ctx->gtick_alloc = ctx->pscr_alloc = ctx->ptick_alloc = 0;
+    ctx->groups_released = true;
     return true;
 }
 
@@ -364,9 +366,40 @@ bool use_compensated(const ap_ctx* ctx) {
     return ctx->o.tol <= 1e-5 || ctx->comp_auto;
 }
 
+// Blocks factored together: an FP64 workspace of at most 16 GiB (or what the HBM budget
+// leaves), as many blocks per group as fit, the groups of equal size (every group pays
+// the same chain of dependent launches, however few blocks it holds).  The optional
+// column-group sums make room when the budget would otherwise cost a group.  NOMEM when
+// not even one block fits.
+ap_status cache_group(ap_ctx* ctx, int64_t* group) {
+    const int64_t edge = (int64_t)ctx->nt * kTile;
+    size_t per_block = (size_t)(edge * edge + edge * kTile) * sizeof(double);
+    if (ctx->o.cache_gemm == AP_CACHE_TC_EXACT)
+        per_block += oz_slice_bytes(ctx->nt) + oz_expo_ints(ctx->nt) * sizeof(int);
+    // (a context's first factorisation allocates the factors themselves before the workspace)
+    const size_t factors = ctx->Linv ? 0 : (size_t)(ctx->m * ctx->ntri) * kTile * kTile * sizeof(float);
+    auto fitting = [&]() {
+        size_t cap = (size_t)16 << 30;
+        if (ctx->o.hbm_budget) {
+            const size_t held = ctx->bytes + factors;
+            cap = std::min(cap, ctx->o.hbm_budget > held ? ctx->o.hbm_budget - held : 0);
+        }
+        return std::min<int64_t>((int64_t)(cap / per_block), ctx->m);
+    };
+    int64_t g = fitting();
+    if (ctx->o.hbm_budget && g < ctx->m && release_groups(ctx)) g = fitting();
+    if (g < 1) return AP_ERR_NOMEM;
+    g = std::min<int64_t>(g, 65535);
+    const int64_t ngroups = (ctx->m + g - 1) / g;
+    *group = (ctx->m + ngroups - 1) / ngroups;
+    return AP_OK;
+}
+
 ap_status build_cache(ap_ctx* ctx) {
     PhaseRange range("ap: Cholesky cache (prep, K_II, FP64 factor, inverse)");
     drop_graph(ctx);
+    int64_t g = 0;
+    AP_TRY(cache_group(ctx, &g));  // (a refusal comes before the inputs are scaled anew)
     AP_TRY(clear_flags(ctx));
     AP_TRY(prep_inputs(ctx, ctx->X, ctx->n, ctx->Xs, ctx->Xs_lo));
     if (ctx->tc) {
@@ -378,22 +411,6 @@ ap_status build_cache(ap_ctx* ctx) {
     if (!ctx->Linv) AP_TRY(dalloc_t(ctx, &ctx->Linv, (size_t)(ctx->m * ctx->ntri * tile_elems)));
     const int64_t edge = (int64_t)ctx->nt * kTile;
     const bool emulate = ctx->o.cache_gemm == AP_CACHE_TC_EXACT;
-    const size_t per_block = (size_t)(edge * edge + ctx->nt * tile_elems) * sizeof(double) +
-                             (emulate ? oz_slice_bytes(ctx->nt) + oz_expo_ints(ctx->nt) * sizeof(int) : 0);
-    // FP64 workspace of at most 16 GiB (or what the HBM budget leaves): as many
-    // blocks per group as fit, the groups of equal size (every group pays the
-    // same chain of dependent launches, however few blocks it holds)
-    size_t cap = (size_t)16 << 30;
-    if (ctx->o.hbm_budget) {
-        const size_t left = ctx->o.hbm_budget > ctx->bytes ? ctx->o.hbm_budget - ctx->bytes : 0;
-        cap = std::min(cap, left);
-    }
-    int64_t g = (int64_t)(cap / per_block);
-    if (g < 1) return AP_ERR_NOMEM;
-    g = std::min<int64_t>(g, ctx->m);
-    g = std::min<int64_t>(g, 65535);
-    const int64_t ngroups = (ctx->m + g - 1) / g;
-    g = (ctx->m + ngroups - 1) / ngroups;
     double* A = nullptr;
     double* Dinv = nullptr;
     AP_TRY(dalloc_t(ctx, &A, (size_t)(g * edge * edge)));
@@ -510,7 +527,15 @@ ap_status ensure_solve(ap_ctx* ctx, int Cp) {
         ctx->part_alloc = need;
         for (const KmvSplit& sp : {a, b, whole})
             AP_TRY(grow_groups(ctx, sp, &ctx->gscr, &ctx->gscr_alloc, &ctx->gtick, &ctx->gtick_alloc));
+        ctx->groups_released = false;
         ctx->Cp = Cp;
+    } else if (ctx->groups_released) {
+        // (the epoch graph was dropped with the area)
+        ctx->groups_released = false;
+        drop_graph(ctx);
+        for (const KmvSplit& sp : {step_split(ctx, Cp, ctx->b), step_split(ctx, Cp, ctx->n),
+                                   kmv_split(ctx->D, Cp, ctx->n, 1, ctx->n)})
+            AP_TRY(grow_groups(ctx, sp, &ctx->gscr, &ctx->gscr_alloc, &ctx->gtick, &ctx->gtick_alloc));
     }
     return AP_OK;
 }
@@ -1207,6 +1232,8 @@ ap_status ap_set_hyper(ap_ctx* ctx, const ap_hyper* h) {
     AP_DEVICE_GUARD(ctx);
     AP_TRY(check_hyper(h, ctx->d));
     if (h->kernel != ctx->kernel) return AP_ERR_INVALID_ARG;
+    int64_t g = 0;
+    AP_TRY(cache_group(ctx, &g));  // (a refusal leaves the context as it was)
     copy_hyper(ctx, h);
     AP_TRY(enter(ctx));
     return build_cache(ctx);
