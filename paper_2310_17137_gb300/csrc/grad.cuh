@@ -18,18 +18,26 @@
 //   Contraction on the tensor cores: S = [alpha U | V] [V | alpha U]^T, both operands
 //   split into three BF16 parts (exact up to the last rounding), the six products of
 //   weight above 2^-24 into two or three FP32 accumulators per entry: hi x hi in chains
-//   of at most two steps, the small ones on their own; the parts are added in FP32.
+//   of at most two steps, the small ones on their own, those of weight 2^-16 first; the
+//   parts are added in FP32.  The tensor cores cut their sums off towards zero, a mean
+//   error that n^2 entries would not average out: all three parts are rounded to nearest,
+//   so that the small products have no preferred sign (with hi cut off, sums of one sign
+//   came out 2.8e-9 low at c = 32; now 0.3e-9, as with scalar multiply-adds).
 // What is left are 4 d multiply-add lanes (as packed pairs) and about 14 instructions
 // per visited entry.  Measured (GB300, n = 131,072, d = 8, c = 32, Matern-3/2): 47.0 ->
-// 14.2 ms for the n^2 forms, FMA pipe 68 % busy, error against 64 bits unchanged (7.7e-8).
-// (With two stages 16.5 ms: the chunk's copy, split and MMAs follow one another.)
+// 14.3 ms for the n^2 forms, FMA pipe 68 % busy.  (With two stages 16.5 ms: the chunk's
+// copy, split and MMAs follow one another.)  Error of the doubles against 64 bits, relative
+// to the forms of absolute values, n = 8192, root mean square over 40 inputs, scalar form
+// -> this one: RBF d = 8, c = 32 3.25e-9 -> 3.30e-9; Matern-3/2 d = 3, c = 16 6.07e-9 ->
+// 6.08e-9; Matern-5/2 d = 20, c = 32 3.47e-9 -> 3.49e-9: that of exp2, sqrt and the inputs.
 //
 // Work units are (row group, 64-column chunk) pairs of the upper triangle in
 // group-major order, cut into equal ranges over a persistent grid; every CTA keeps
-// one set of sums whatever groups it meets (FP32 over 64 entries per thread, FP64
-// beyond), and the CTA that finishes last adds the CTAs' sums in order.
+// one set of sums whatever groups it meets (FP32 over 128 entries per thread, 64 for
+// D = 16, FP64 beyond; folding every 64 takes 5 to 9 % longer at D = 12 and 20 and leaves
+// the error as it is), and the CTA that finishes last adds the CTAs' sums in order.
 // Warp roles: transform warps (one row, or two rows 128 apart, per thread; 16 columns of
-// every chunk), one MMA issuer, one bulk-copy lane for the columns' coordinates, two
+// every chunk, 32 for D > 16), one MMA issuer, one bulk-copy lane for the columns' coordinates, two
 // warps that split the chunk's [V | alpha U]; the transform warps split the rows' own
 // operand when the group changes.  Every wait is bounded.
 #pragma once
@@ -125,7 +133,7 @@ __device__ __forceinline__ void split_operand(const GradParams& p, int64_t i, in
     }
     uint32_t w[3][4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) split3_rn(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
+    for (int j = 0; j < 4; ++j) split3_nearest(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
 #pragma unroll
     for (int pl = 0; pl < 3; ++pl)
         *reinterpret_cast<uint4*>(dst + pl * plane) = make_uint4(w[pl][0], w[pl][1], w[pl][2], w[pl][3]);
@@ -307,8 +315,8 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
                             const float2 db = __ffma2_rn(make_float2(v.z, v.w), m1, xa[r][2 * k + 1]);
                             sq[r][2 * k] = __fmul2_rn(da, da);
                             sq[r][2 * k + 1] = __fmul2_rn(db, db);
-                            t2[r] = __fadd2_rn(t2[r], sq[r][2 * k]);
-                            t2[r] = __fadd2_rn(t2[r], sq[r][2 * k + 1]);
+                            t2[r] = __ffma2_rn(da, da, t2[r]);
+                            t2[r] = __ffma2_rn(db, db, t2[r]);
                         }
                     }
 #pragma unroll
@@ -374,11 +382,15 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
                     constexpr uint64_t pa = (R * K::kPlaneA) >> 4, pb = K::kPlaneB >> 4;
 #pragma unroll
                     for (int ks = 0; ks < K::kSteps; ++ks) {
+                        // the products of weight 2^-16 of all steps first, while the sum is small
                         const uint64_t ak = a + (uint64_t)(16 * ks), bk = b + (uint64_t)(16 * ks);
-                        // the small products, smallest first, then hi x hi
                         mma_ss(ds, ak + 2 * pa, bk, idesc, ks > 0 ? 1u : 0u);
                         mma_ss(ds, ak + pa, bk + pb, idesc, 1u);
                         mma_ss(ds, ak, bk + 2 * pb, idesc, 1u);
+                    }
+#pragma unroll
+                    for (int ks = 0; ks < K::kSteps; ++ks) {
+                        const uint64_t ak = a + (uint64_t)(16 * ks), bk = b + (uint64_t)(16 * ks);
                         mma_ss(ds, ak + pa, bk, idesc, 1u);
                         mma_ss(ds, ak, bk + pb, idesc, 1u);
                         mma_ss(d + (ks / 2) * kChunk, ak, bk, idesc, (uint32_t)(ks & 1));

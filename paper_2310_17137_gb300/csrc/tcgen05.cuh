@@ -213,6 +213,18 @@ __device__ __forceinline__ void split3_rn(float x0, float x1, uint32_t& hi, uint
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(s1), "f"(s0));
 }
 
+// The same with hi rounded to nearest too: mid then has no preferred sign either, so that
+// what the tensor cores cut off its products' sums does not lean towards zero with the
+// result.  (The largest floats keep a finite hi.)
+__device__ __forceinline__ void split3_nearest(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+    constexpr uint32_t kTop = 0xFFFF0000u;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(x1), "f"(x0));
+    const float r0 = x0 - __uint_as_float(hi << 16), r1 = x1 - __uint_as_float(hi & kTop);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(mid) : "f"(r1), "f"(r0));
+    const float s0 = r0 - __uint_as_float(mid << 16), s1 = r1 - __uint_as_float(mid & kTop);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(s1), "f"(s0));
+}
+
 // Shared-memory matrix descriptor, K-major, no swizzle: core matrices of 8 rows
 // x 16 bytes stored contiguously (128 B); lbo = byte distance between core
 // matrices adjacent along K, sbo = between 8-row groups.
