@@ -115,6 +115,7 @@ __device__ __forceinline__ int64_t packed_tile(int i, int k) { return (int64_t)i
 
 __global__ void __launch_bounds__(256) build_kii_kernel(const CacheParams cp, int64_t blk0, double* A) {
     __shared__ double s_tab[64];
+    __shared__ double s_unit[AP_MAX_DIM];
     __shared__ double s_xi[AP_MAX_DIM * T], s_xj[AP_MAX_DIM * T];  // dimension-major
     const int z = blockIdx.y;
     const int64_t blk = blk0 + z;
@@ -126,15 +127,13 @@ __global__ void __launch_bounds__(256) build_kii_kernel(const CacheParams cp, in
     const int64_t bJ = min(cp.b, cp.n - lo);
     double* Ab = A + (int64_t)z * ld * ld;
     fill_exp2_table(s_tab);
-    // the tile's row and column points relative to the block's first one (differences of
-    // FP32 values, exact in FP64 unless 29 binades apart), in units that make the squared
-    // distance phi's argument: two FP64 operations per entry and dimension are left
+    if (threadIdx.x < d) s_unit[threadIdx.x] = cp.unit[threadIdx.x];
+    // the tile's row and column points (rows past the block are never read)
     for (int t = threadIdx.x; t < T * d; t += blockDim.x) {
         const int r = t / d, k = t % d;
         const int64_t li = (int64_t)ti * T + r, lj = (int64_t)tj * T + r;
-        const double x0 = (double)cp.X[lo * d + k];
-        s_xi[k * T + r] = li < bJ ? ((double)cp.X[(lo + li) * d + k] - x0) * cp.unit[k] : 0.0;
-        s_xj[k * T + r] = lj < bJ ? ((double)cp.X[(lo + lj) * d + k] - x0) * cp.unit[k] : 0.0;
+        s_xi[k * T + r] = li < bJ ? (double)cp.X[(lo + li) * d + k] : 0.0;
+        s_xj[k * T + r] = lj < bJ ? (double)cp.X[(lo + lj) * d + k] : 0.0;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < T * T; t += blockDim.x) {
@@ -142,9 +141,14 @@ __global__ void __launch_bounds__(256) build_kii_kernel(const CacheParams cp, in
         const int64_t li = (int64_t)ti * T + r, lj = (int64_t)tj * T + q;
         double v;
         if (li < bJ && lj < bJ) {
+            // the difference of two FP32 values is exact in FP64 (29 binades apart at most,
+            // otherwise rounded once); its unit makes the squared distance phi's argument.
+            // (Points scaled ahead, relative to the block's first one, would save a
+            // multiplication per entry and dimension but lose near points of a block that
+            // holds a far one.)
             double r2 = 0.0;
             for (int k = 0; k < d; ++k) {
-                const double df = s_xi[k * T + r] - s_xj[k * T + q];
+                const double df = (s_xi[k * T + r] - s_xj[k * T + q]) * s_unit[k];
                 r2 = fma(df, df, r2);
             }
             v = cp.s * phi_of(cp.kernel, r2, s_tab);
