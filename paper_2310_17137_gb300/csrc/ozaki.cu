@@ -15,12 +15,11 @@
 //   2. for every level L = p + q = 2..9 the tensor cores accumulate
 //      acc_L = sum_{p+q=L} sum_kk s_p(r, kk) s_q(c, kk) in FP32.  Every partial
 //      sum is an integer below 2^22, so the accumulation is exact;
-//   3. the levels are combined in integers,
-//      H = sum_{L<=5} acc_L 2^{7(5-L)}, Lo = sum_{L>=6} acc_L 2^{7(9-L)},
-//      T = 2^19 H + round(2^-9 Lo) (below 2^63), and A_rc -= 2^{e_r+e_c-54} T with
-//      two FP64 roundings: T's own to 53 bits, in integer arithmetic, and the sum's.
-// The terms left out (levels above 9, the slice remainders, Lo's last 9 bits) are
-// below about 2^-50 K max_kk|a_r,kk| max_kk|a_c,kk| per entry, the size of FP64
+//   3. the levels are combined in integers, T = sum_L acc_L 2^{7(9-L)} (below 2^68; as a
+//      64-bit integer, or, from 2^62 on, as one without its last 5 bits), and
+//      A_rc -= 2^{e_r+e_c-63} T with two FP64 roundings: T's own to 53 bits, in integer
+//      arithmetic, and the sum's.
+// The terms left out (levels above 9 and the slice remainders) are below about 2^-50 K max_kk|a_r,kk| max_kk|a_c,kk| per entry, the size of FP64
 // rounding when the entries of a panel row have similar magnitudes; the matrix
 // itself stays FP64.  On kernel blocks the factor's backward error ||L L^T - K|| / ||K||
 // matches the all-FP64 factorisation (6e-16 vs 5e-16 on a Matern-5/2 block
@@ -142,9 +141,14 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const double* src0, int64
     if (grp == 0) E[(int64_t)z * rows_pad + r] = nonfinite ? kBadExp : e;
 }
 
-// 2^33 h1 + 2^19 h2 + 2^5 l1 + round(2^-9 l2), h1 .. l2 below 2^29: below 2^63.
-__device__ __forceinline__ long long level_int(int h1, int h2, int l1, int l2) {
-    return (long long)h2 * (1LL << 19) + ((long long)l1 * 32 + ((l2 + 256) >> 9)) + ((long long)h1 << 33);
+// T = 2^42 h1 + 2^28 h2 + 2^14 l1 + l2 for the level pairs h1 .. l2 (h1 below 2^25 + 2^19,
+// the others below 2^29) as v 2^drop: all bits below 2^62, otherwise without the last five
+// (which the rounding to 53 bits drops anyway).
+__device__ __forceinline__ long long level_int(int h1, int h2, int l1, int l2, int& drop) {
+    const long long v = (long long)h2 * (1LL << 23) + ((long long)l1 * (1LL << 9) + (l2 >> 5)) + ((long long)h1 << 37);
+    const bool whole = (unsigned)((int)(v >> 32) + (1 << 25)) < 1u << 26;  // -2^57 <= v < 2^57
+    drop = whole ? 0 : 5;
+    return whole ? (v << 5) | (l2 & 31) : v;
 }
 
 // 2^e0 v rounded to a double (half away from zero), for results in the normal range:
@@ -170,9 +174,28 @@ __device__ __forceinline__ double level_sum(long long v, int e0, bool& extreme) 
 
 // The same for any exponents; a NaN or infinity in the panel (marked row exponents) must
 // reach the next pivot test as NaN.
-__device__ __noinline__ double level_sum_any(long long v, int er, int ec) {
+__device__ __noinline__ double level_sum_any(int h1, int h2, int l1, int l2, int er, int ec) {
     if (er == kBadExp || ec == kBadExp) return __longlong_as_double(0x7ff8000000000000LL);
-    return ldexp((double)v, max(-2000, min(2000, er + ec - 54)));
+    int drop;
+    const long long v = level_int(h1, h2, l1, l2, drop);
+    return ldexp((double)v, max(-2000, min(2000, er + ec - 63 + drop)));
+}
+
+// Four products of a row (exponent er) with four columns from their level pairs; marked:
+// one of the exponents is kBadExp.
+__device__ __forceinline__ void level_row(const int (&h1)[4], const int (&h2)[4], const int (&l1)[4],
+                                          const int (&l2)[4], int er, const int (&ec)[4], bool marked, double (&t)[4]) {
+    bool extreme = marked;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        int drop;
+        const long long v = level_int(h1[c], h2[c], l1[c], l2[c], drop);
+        t[c] = level_sum(v, er + ec[c] - 63 + drop, extreme);
+    }
+    if (extreme) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t[c] = level_sum_any(h1[c], h2[c], l1[c], l2[c], er, ec[c]);
+    }
 }
 
 // kFirst, kRest: A_ij -= A_ik A_jk^T over the trailing lower tiles (SYRK/GEMM);
@@ -345,7 +368,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
             double* C0 = A + (int64_t)z * ld * ld + r * ld + (int64_t)j * T + cl;
             auto entry = [&](int rr, int cb) { return reinterpret_cast<double2*>(C0 + (int64_t)(8 * rr) * ld + 8 * cb); };
             // half of the entries to update are on their way before the MMAs are waited for
-            double2 cv[4][2];
+            double2 cv[2][2];  // two rows at a time
             if (!kTrsm && mine) {
 #pragma unroll
                 for (int rr = 0; rr < 2; ++rr) {
@@ -385,31 +408,21 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(double* A, int n
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_read);
             if (!mine) continue;  // (warp-uniform)
-            if constexpr (!kTrsm) {
-#pragma unroll
-                for (int rr = 2; rr < 4; ++rr) {
-                    cv[rr][0] = *entry(rr, 0);
-                    cv[rr][1] = *entry(rr, 1);
-                }
-            }
 #pragma unroll
             for (int rr = 0; rr < 4; ++rr) {
                 double t[4];
-                bool extreme = marked;
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    t[c] = level_sum(level_int(q[0][rr][c], q[1][rr][c], q[2][rr][c], q[3][rr][c]),
-                                     er[rr] + ec[c] - 54, extreme);
-                if (extreme) {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        t[c] = level_sum_any(level_int(q[0][rr][c], q[1][rr][c], q[2][rr][c], q[3][rr][c]), er[rr], ec[c]);
-                }
+                level_row(q[0][rr], q[1][rr], q[2][rr], q[3][rr], er[rr], ec, marked, t);
 #pragma unroll
                 for (int cb = 0; cb < 2; ++cb) {
                     double2 o = make_double2(t[2 * cb], t[2 * cb + 1]);
-                    if constexpr (!kTrsm) o = make_double2(cv[rr][cb].x - o.x, cv[rr][cb].y - o.y);
+                    if constexpr (!kTrsm) o = make_double2(cv[rr & 1][cb].x - o.x, cv[rr & 1][cb].y - o.y);
                     *entry(rr, cb) = o;
+                }
+                if constexpr (!kTrsm) {
+                    if (rr < 2) {
+                        cv[rr][0] = *entry(rr + 2, 0);
+                        cv[rr][1] = *entry(rr + 2, 1);
+                    }
                 }
             }
         }
