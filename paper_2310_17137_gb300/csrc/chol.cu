@@ -74,8 +74,9 @@ __device__ __forceinline__ double exp_nonpos(double x, const double* tab2) {
 
 __device__ __forceinline__ double sqrt_nonneg(double x) {
     const int hi = __double2hiint(x);
-    if (hi < __double2hiint(1e-36)) return 0.0;  // phi is flat at 0: the error is below the last bit
-    if (hi > __double2hiint(1e12)) return 1e6;   // e^-sqrt(x) underflows either way
+    const bool nan = (hi & 0x7fffffff) > 0x7ff00000;  // (stays one)
+    if (hi < __double2hiint(1e-36)) return nan ? x : 0.0;  // phi is flat at 0: the error is below the last bit
+    if (hi > __double2hiint(1e12)) return nan ? x : 1e6;   // e^-sqrt(x) underflows either way
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     double g = x * y, h = 0.5 * y;
