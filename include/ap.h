@@ -141,9 +141,12 @@ typedef struct ap_opts {
     int32_t profile;      /* 1: time every block solve and residual update with CUDA events */
     int32_t residual_mode; /* ap_residual_mode: arithmetic of the residual recompute */
     int32_t cache_gemm;   /* ap_cache_gemm: arithmetic of the Cholesky trailing updates */
-    int64_t wait_limit_cycles; /* bound of each device-side wait of the tensor-core update, in SM
+    int64_t wait_limit_cycles; /* bound of each device-side wait of the low-precision update, in SM
                                   clock cycles; <= 0: about 2 s.  A wait that runs out ends the
-                                  kernel early and the call returns AP_ERR_TIMEOUT */
+                                  kernel early and the call returns AP_ERR_TIMEOUT.  The FP32
+                                  products with more than 4 right-hand sides and the gradient
+                                  forms keep shorter bounds too (in the waits of their copy
+                                  issuers); longer ones leave them at 2 s */
     const volatile int32_t* cancel; /* optional host flag: when it reads non-zero at the end of an
                                        epoch, ap_solve / ap_mll_grad stop with AP_ERR_CANCELLED
                                        (W holds the last iterate) */
@@ -209,7 +212,7 @@ ap_status ap_set_hyper(ap_ctx* ctx, const ap_hyper* h);
  * Returns OK when the stopping rule held after >= min_epochs epochs,
  * NOT_CONVERGED at max_epochs / max_steps (W still written), NAN (a NaN or Inf
  * in the residual, e.g. from B), CANCELLED (opts.cancel), TIMEOUT (a bounded
- * device wait of the tensor-core update ran out), CUDA. */
+ * device wait of a tensor-core kernel ran out), CUDA. */
 ap_status ap_solve(ap_ctx* ctx, const float* B_dev, int32_t c, const float* W0_dev,
                    float* W_dev, ap_info* info);
 
@@ -225,7 +228,9 @@ ap_status ap_solve_host(const float* X_host, int64_t n, int32_t d, const ap_hype
 
 /* True residual R = B - K_hat W (n x c, device), FP32 form, all n^2 kernel
  * entries evaluated on the fly (the residual lemma of App. B).  Used for
- * refinement and certification. */
+ * refinement and certification.  AP_ERR_TIMEOUT (R_dev not usable) when a
+ * bounded device wait ran out, with more than 4 right-hand sides in the plain
+ * FP32 form. */
 ap_status ap_residual(ap_ctx* ctx, const float* B_dev, int32_t c, const float* W_dev,
                       float* R_dev);
 
@@ -269,6 +274,7 @@ ap_status ap_grad_quadforms(ap_ctx* ctx, const float* U_dev, const float* V_dev,
  *     when D + c <= 40), D = d rounded up to 4, 8, 12, 16, 24 or 32: n up to
  *     about 490k at d = 32 with c = 32 and 3.3M at d <= 8.  A larger problem
  *     returns AP_ERR_SCRATCH_LIMIT before anything is launched.
+ *   - AP_ERR_TIMEOUT when a bounded device wait ran out.
  *   - The first call on each device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current; make that first call
  *     before any stream capture.

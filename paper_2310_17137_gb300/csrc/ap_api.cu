@@ -628,6 +628,7 @@ ap_status launch_step(ap_ctx* ctx, bool colnorms, int64_t j) {
     kp.blk = ctx->b;
     kp.dependent = !prof;
     kp.err = &ctx->state->tc_err;
+    kp.wait_cycles = ctx->o.wait_limit_cycles;
     kp.epi = make_epi(ctx, kEpiBlockNorms | (colnorms ? kEpiColNorms : 0), 1, sh);
     AP_CK(launch_kmv(ctx->kernel, kp, ctx->D, Cp, ctx->st));
     ++ctx->launches;
@@ -678,6 +679,7 @@ ap_status launch_full_residual(ap_ctx* ctx, const float* base, const float* V, f
     kp.Xa_lo = ctx->Xs_lo;
     kp.Xb_lo = ctx->Xs_lo;
     kp.err = &ctx->state->tc_err;
+    kp.wait_cycles = ctx->o.wait_limit_cycles;
     kp.epi = make_epi(ctx, flags, 0, sh);
     if (!blocks) kp.epi.seg = ctx->n;
     if (comp) AP_CK(launch_kmv_comp(ctx->kernel, kp, ctx->D, ctx->Cp, ctx->st));
@@ -1038,6 +1040,7 @@ void ctx_grad_view(const ap_ctx* ctx, GradView* v) {
     v->s = ctx->s;
     v->ell = ctx->ell;
     v->stream = ctx->ust;
+    v->wait_cycles = ctx->o.wait_limit_cycles;
 }
 
 void grad_finish(const GradView& v, const double* raw, double* out_host) {
@@ -1368,6 +1371,7 @@ static ap_status grad_quadforms_impl(ap_ctx* ctx, const float* U, const float* V
     for (int k = 0; k < c; ++k) gp.alpha[k] = (float)alpha[k];
     gp.part = ctx->gpart;
     gp.err = &ctx->state->tc_err;
+    gp.wait_cycles = ctx->o.wait_limit_cycles;
     gp.ticket = ctx->ticket + 1;
     gp.out = ctx->gout;
     AP_CK(launch_grad(ctx->kernel, gp, ctx->D, Cp, ctx->st));

@@ -131,6 +131,7 @@ struct KmvParams {
     float* gscr;           // G > 1: partial sums (KmvSplit::scratch floats)
     unsigned int* gtick;   // G > 1: arrival tickets (KmvSplit::tickets), zero between launches
     int* err;              // wait-timeout flag of the tensor-core form
+    long long wait_cycles; // bound of its copy issuer's waits (<= 0: the default, about 2 s)
     bool dependent;        // launch without waiting for the kernel before (launch_dependent)
     EpiParams epi;
 };
@@ -266,6 +267,7 @@ struct GradParams {
     unsigned int* ticket;  // zero between launches
     double* out;           // D + 2
     int* err;              // wait-timeout flag
+    long long wait_cycles; // bound of the copy issuer's waits (<= 0: the default, about 2 s)
 };
 constexpr int kGradCtas = 152;  // persistent grid: one CTA per SM
 cudaError_t launch_grad(int kernel, const GradParams& p, int D, int C, cudaStream_t st);
@@ -352,6 +354,7 @@ struct GradView {
     float s;
     const float* ell;
     cudaStream_t stream;  // the caller's stream of the context
+    long long wait_cycles;
 };
 void ctx_grad_view(const ap_ctx* ctx, GradView* v);
 // Turn the raw D + 2 sums of the gradient kernel into the d + 2 quadratic forms.

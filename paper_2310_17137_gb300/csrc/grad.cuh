@@ -418,7 +418,8 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
             int stage = 0;
             for (int c = 0; c < total && ok; ++c) {
                 if (c >= kStages)
-                    ok = mbar_wait(&bar_empty[stage], (uint32_t)((c / kStages - 1) & 1), &s_abort, p.err);
+                    ok = mbar_wait_issuer(&bar_empty[stage], (uint32_t)((c / kStages - 1) & 1), &s_abort, p.err,
+                                          p.wait_cycles);
                 if (!ok) break;
                 const int cnt = (int)min((int64_t)kChunk, n - q * kChunk);
                 const bool in = AP_CHK(q >= 0 && cnt > 0 && q * kChunk + cnt <= n);

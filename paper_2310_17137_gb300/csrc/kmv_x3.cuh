@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
             int q = q0, stage = 0;
             for (int c = 0; c < total && ok; ++c) {
                 if (c >= kStages)
-                    ok = mbar_wait(&bar_empty[stage], (uint32_t)((c / kStages - 1) & 1), &s_abort, p.err);
+                    ok = mbar_wait_issuer(&bar_empty[stage], (uint32_t)((c / kStages - 1) & 1), &s_abort, p.err, p.wait_cycles);
                 if (!ok) break;
                 uint8_t* dst = x3_smem + (size_t)stage * K::kStageBytes;
                 const int64_t lc = (int64_t)q * kChunk;

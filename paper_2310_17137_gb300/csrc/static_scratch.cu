@@ -85,6 +85,7 @@ extern "C" ap_status ap_grad_quadforms_static(ap_ctx* ctx, const float* U_dev, c
     gp.ticket = reinterpret_cast<unsigned int*>(scratch + kTicketOff);
     gp.out = scratch + kOutOff;
     gp.err = reinterpret_cast<int*>(scratch + kErrOff);
+    gp.wait_cycles = v.wait_cycles;
     double raw[AP_MAX_DIM + 2] = {};
     double err = 0.0;  // the flag's eight bytes
     if (cudaMemsetAsync(gp.ticket, 0, 2 * sizeof(double), v.stream) != cudaSuccess ||

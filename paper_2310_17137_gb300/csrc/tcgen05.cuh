@@ -97,6 +97,15 @@ static __device__ __noinline__ bool mbar_wait_strict(uint64_t* bar, uint32_t par
     }
 }
 
+// A copy issuer's wait under opts.wait_limit_cycles: bounds shorter than the default are
+// enforced here, with non-blocking probes; the issuer runs ahead of the pipeline, so its
+// waits are the ones that run out, and the other warps leave when they see the abort flag.
+__device__ __forceinline__ bool mbar_wait_issuer(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                                 int* err_flag, long long limit) {
+    return limit > 0 && limit < kWaitCycles ? mbar_wait_strict(bar, parity, abort_flag, err_flag, limit)
+                                            : mbar_wait(bar, parity, abort_flag, err_flag);
+}
+
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
