@@ -183,17 +183,36 @@ __device__ __forceinline__ void flush_row(const SolveParams& p, int row, int slo
     if (*s_last) {
         __threadfence();
         const float* src = p.spart + (int64_t)row * p.maxj * T * C;
-        for (int t = tid; t < T * C; t += kSolveThreads) {
-            float sum = 0.0f;
-            // slots in order, eight at a time with all their loads in flight
-            for (int j0 = 0; j0 < nslots; j0 += 8) {
-                float v[8];
+        // slots in order, several of them and up to four sums per thread at a time, with all
+        // their loads in flight: a row of a short block has a slot per tile, and one sum at
+        // a time made the last CTA wait for memory C / 4 times over
+        constexpr int E = (T * C + kSolveThreads - 1) / kSolveThreads, EB = E < 4 ? E : 4, SB = C == 16 ? 4 : 8;
+#pragma unroll 1
+        for (int e0 = 0; e0 < E; e0 += EB) {
+            float sum[EB];
 #pragma unroll
-                for (int jj = 0; jj < 8; ++jj) v[jj] = j0 + jj < nslots ? __ldcg(src + (int64_t)(j0 + jj) * T * C + t) : 0.0f;
+            for (int x = 0; x < EB; ++x) sum[x] = 0.0f;
+            const int t0 = tid + e0 * kSolveThreads;
+#pragma unroll 1
+            for (int j0 = 0; j0 < nslots; j0 += SB) {
+                float v[SB][EB];
 #pragma unroll
-                for (int jj = 0; jj < 8; ++jj) sum += v[jj];
+                for (int jj = 0; jj < SB; ++jj)
+#pragma unroll
+                    for (int x = 0; x < EB; ++x)
+                        v[jj][x] = j0 + jj < nslots && (T * C % kSolveThreads == 0 || t0 < T * C)
+                                       ? __ldcg(src + (int64_t)(j0 + jj) * T * C + t0 + x * kSolveThreads)
+                                       : 0.0f;
+#pragma unroll
+                for (int jj = 0; jj < SB; ++jj)
+#pragma unroll
+                    for (int x = 0; x < EB; ++x) sum[x] += v[jj][x];
             }
-            emit(t / C, t % C, sum);
+#pragma unroll
+            for (int x = 0; x < EB; ++x) {
+                const int t = t0 + x * kSolveThreads;
+                if (T * C % kSolveThreads == 0 || t < T * C) emit(t / C, t % C, sum[x]);
+            }
         }
         if (tid == 0) p.sticket[row] = 0u;
     }
