@@ -626,7 +626,12 @@ ap_status launch_step(ap_ctx* ctx, bool colnorms, int64_t j) {
     kp.noise_diag = 1;
     kp.sel = ctx->sel;
     kp.blk = ctx->b;
-    kp.dependent = !prof;
+    // A dependent launch spares a microsecond or two where the block solve leaves most SMs
+    // free.  Where it fills them (136 CTAs at b = 1000) the SIMT form's clusters would be
+    // placed on what is left and stay there: n = 8000, d = 8, b = 1000, c = 32 72 against 65
+    // us a step, n = 50,000, b = 4096, c = 1 213 against 190; b = 512 (36 CTAs), c = 4 20.5
+    // against 21.7.  The tensor-core form's CTAs need an SM each and wait: 62 against 63 us.
+    kp.dependent = !prof && (Cp >= kX3MinC || 4 * block_solve_ctas(ctx->nt, ctx->sol_tpc) <= ctx->num_sms);
     kp.err = &ctx->state->tc_err;
     kp.wait_cycles = ctx->o.wait_limit_cycles;
     kp.epi = make_epi(ctx, kEpiBlockNorms | (colnorms ? kEpiColNorms : 0), 1, sh);

@@ -238,6 +238,7 @@ struct SolveParams {
 };
 // Work split of the block solve for nt tiles per block edge and C right-hand sides.
 void block_solve_layout(int nt, int C, int num_sms, int* tpc, int* maxj);
+int64_t block_solve_ctas(int nt, int tpc);
 cudaError_t launch_block_solve(const SolveParams& p, cudaStream_t st, int64_t* launches);
 
 // ---- small helpers ----------------------------------------------------------

@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kSolveThreads, solve_ctas_per_sm(C)) solve_upp
 
 template <int C>
 cudaError_t launch_solve_inst(const SolveParams& p, cudaStream_t st) {
-    const unsigned grid = (unsigned)((solve_ntri(p.nt) + p.tpc - 1) / p.tpc);
+    const unsigned grid = (unsigned)block_solve_ctas(p.nt, p.tpc);
     constexpr size_t smem = solve_smem<C>();
     cudaError_t err;
     if ((err = cudaFuncSetAttribute(solve_lower_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
@@ -387,6 +387,8 @@ void block_solve_layout(int nt, int C, int num_sms, int* tpc, int* maxj) {
     *tpc = (int)std::max<int64_t>(1, (solve_ntri(nt) + target - 1) / target);
     *maxj = (nt + *tpc - 1) / *tpc + 1;
 }
+
+int64_t block_solve_ctas(int nt, int tpc) { return (solve_ntri(nt) + tpc - 1) / tpc; }
 
 cudaError_t launch_block_solve(const SolveParams& p, cudaStream_t st, int64_t* launches) {
     if (launches) *launches += 2;
