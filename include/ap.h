@@ -64,8 +64,9 @@ typedef enum { AP_RBF = 0, AP_MATERN32 = 1, AP_MATERN52 = 2 } ap_kernel;
 
 /* Arithmetic of the residual update.
  *   AP_FP32:         kernel blocks in FP32; contraction in FP32 or, with more than 4
- *                    right-hand sides, in split precision on the tensor cores (three
- *                    BF16 parts per operand, FP32 sums: FP32 accuracy).
+ *                    right-hand sides and enough entries, in split precision on the
+ *                    tensor cores (three BF16 parts per operand, FP32 sums: FP32
+ *                    accuracy).
  *   AP_BF16_REFINE:  kernel blocks and K*Delta on tensor cores with BF16
  *                    operands and FP32 accumulation; accuracy recovered by
  *                    recomputing R = B - K_hat W in the FP32 form (iterative

@@ -297,6 +297,7 @@ ap_status grow_groups(ap_ctx* ctx, const KmvSplit& sp, float** scr, int64_t* scr
 // Fill the split's part of the launch parameters from an area that grow_groups
 // sized (or could not).
 void set_split(KmvParams* kp, const KmvSplit& sp, float* scr, int64_t scr_n, unsigned* tick, int64_t tick_n) {
+    kp->x3 = sp.x3;
     kp->rm = sp.rm;
     kp->G = sp.scratch <= scr_n && sp.tickets <= tick_n ? sp.G : 1;
     kp->ctas = kp->G > 1 ? sp.ctas : (int)std::min<int64_t>(sp.ctas, sp.ntiles);
@@ -631,7 +632,7 @@ ap_status launch_step(ap_ctx* ctx, bool colnorms, int64_t j) {
     // placed on what is left and stay there: n = 8000, d = 8, b = 1000, c = 32 72 against 65
     // us a step, n = 50,000, b = 4096, c = 1 213 against 190; b = 512 (36 CTAs), c = 4 20.5
     // against 21.7.  The tensor-core form's CTAs need an SM each and wait: 62 against 63 us.
-    kp.dependent = !prof && (Cp >= kX3MinC || 4 * block_solve_ctas(ctx->nt, ctx->sol_tpc) <= ctx->num_sms);
+    kp.dependent = !prof && (split.x3 || 4 * block_solve_ctas(ctx->nt, ctx->sol_tpc) <= ctx->num_sms);
     kp.err = &ctx->state->tc_err;
     kp.wait_cycles = ctx->o.wait_limit_cycles;
     kp.epi = make_epi(ctx, kEpiBlockNorms | (colnorms ? kEpiColNorms : 0), 1, sh);
@@ -1302,7 +1303,8 @@ ap_status ap_residual(ap_ctx* ctx, const float* B_dev, int32_t c, const float* W
     AP_TRY(ensure_solve(ctx, Cp));
     ctx->r_tracked_c = 0;
     AP_TRY(enter(ctx));
-    const bool waits = Cp >= kX3MinC && !use_compensated(ctx);  // the tensor-core form runs
+    // (the tensor-core form has bounded waits to look at)
+    const bool waits = !use_compensated(ctx) && kmv_split(ctx->D, Cp, ctx->n, 1, ctx->n).x3;
     if (waits || ctx->timed_out) AP_TRY(clear_flags(ctx));
     AP_CK(launch_pad_copy(B_dev, ctx->n, c, ctx->Bp, Cp, ctx->st));
     AP_CK(launch_pad_copy(W_dev, ctx->n, c, ctx->Tmp, Cp, ctx->st));

@@ -125,6 +125,7 @@ struct KmvParams {
     int64_t blk;
     const float* Xa_lo;    // compensated form only: low parts of the scaled inputs
     const float* Xb_lo;
+    bool x3;               // the tensor-core form (KmvSplit)
     int rm;                // rows per thread (KmvSplit)
     int G;                 // > 1: row tiles are shared between CTAs through gscr (KmvSplit)
     int ctas;              // CTAs of the tensor-core form's persistent grid (KmvSplit)
@@ -142,13 +143,23 @@ struct KmvParams {
 // Tensor-core form: a persistent grid over (tile, column chunk) units; G > 1 lets a
 // range of units end inside a tile.
 struct KmvSplit {
+    bool x3;  // the tensor-core form
     int rm, S, G, ctas;
     int64_t rows, tps, ntiles;
     int64_t scratch;  // floats of partial sums when G > 1
     int64_t tickets;  // arrival tickets when G > 1
 };
 KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols);
-constexpr int kX3MinC = 16;  // right-hand sides (padded) from which the tensor-core form runs
+constexpr int kX3MinC = 16;  // right-hand sides (padded) from which the tensor-core form exists
+// Entries of a product from which the tensor-core form runs, 16 and 32 right-hand sides: it
+// has some 12 us more of start-up (tensor memory, splitting and draining the first chunk,
+// the hand-over of shared row groups), the SIMT form the slope of its FP32 contraction.
+// Measured (GB300, us per call or step, SIMT : tensor cores), 16: ap_residual 2048^2 50 : 55,
+// 3000^2 65 : 68, 4096^2 94 : 74; steps 8000 x 1000 48 : 55, 16,000 x 1000 59 : 66, 8192 x
+// 2048 76 : 77, 20,000 x 2048 108 : 92.  32: 1024^2 46 : 57, 2048^2 67 : 66, 4096^2 95 : 83;
+// steps 2000 x 256 37 : 45, 2000 x 1000 71 : 73, 10,000 x 256 43 : 41, 16,000 x 1000 102 : 81
+// (all at d = 8, Matern-3/2).
+constexpr double kX3MinEntries16 = 1 << 24, kX3MinEntries32 = 2.5e6;
 constexpr int kX3MaxD2 = 16; // largest D whose two rows per thread fit the registers
 constexpr int kX3Chunk = 128;
 

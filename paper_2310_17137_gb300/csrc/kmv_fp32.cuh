@@ -1,7 +1,8 @@
-// FP32 SIMT form (up to 4 right-hand sides; kmv_x3.cuh for more) of the fused kernel-matrix product (the AP residual update,
+// FP32 SIMT form of the fused kernel-matrix product (the AP residual update,
 // Eq. text_update_of_r, the residual recompute of the App. B lemma and the
 // posterior mean of Sec. 2), with the block-norm / Gauss-Southwell epilogue of
-// Eq. approximate_gauss_southwell fused in.
+// Eq. approximate_gauss_southwell fused in.  Up to 4 right-hand sides always, more for
+// products too small for the tensor cores to pay (kX3MinEntries16 / 32; kmv_x3.cuh).
 //
 // Work decomposition
 //   grid.x = row tiles of ROWS = 128 * RM rows; a tile never straddles an AP
@@ -183,9 +184,13 @@ __device__ __forceinline__ bool epi_store(const KmvParams& p, float* s_part, int
     auto cluster_sum = [&](int t) {
         const int lc = (rank * rpr + t / C) * C + t % C;
         if (S == 1) return s_part[lc];
+        // (all remote loads in flight before the first is added)
         cg::cluster_group cluster = cg::this_cluster();
-        float sum = 0.0f;
-        for (int src = 0; src < S; ++src) sum += cluster.map_shared_rank(s_part, src)[lc];
+        float v[kMaxSplit], sum = 0.0f;
+#pragma unroll
+        for (int src = 0; src < kMaxSplit; ++src) v[src] = src < S ? cluster.map_shared_rank(s_part, src)[lc] : 0.0f;
+#pragma unroll
+        for (int src = 0; src < kMaxSplit; ++src) sum += v[src];
         return sum;
     };
     // slot of group g: this rank's rpr x C sums of the tile
@@ -204,17 +209,10 @@ __device__ __forceinline__ bool epi_store(const KmvParams& p, float* s_part, int
         if (!*s_last) return false;
         __threadfence();
     }
-    for (int t = tid; t < rpr * C; t += kKmvThreads) {
+    auto put = [&](int t, float sum) {
         const int lr = rank * rpr + t / C;
         const int c = t % C;  // == tid % C since kKmvThreads % C == 0
         const int64_t i = r0 + lr;
-        float sum = 0.0f;
-        if (G > 1) {
-#pragma unroll 8
-            for (int g = 0; g < G; ++g) sum += __ldcg(slots + (int64_t)g * ROWS * C + t);
-        } else {
-            sum = cluster_sum(t);
-        }
         if (i < r1 && AP_CHK(i < p.na)) {
             const float bv = p.base ? p.base[i * C + c] : p.base_const;
             const float o = fmaf(p.sgn, sum, bv);
@@ -222,6 +220,17 @@ __device__ __forceinline__ bool epi_store(const KmvParams& p, float* s_part, int
             const double od = (double)o;
             sq += od * od;
             colacc += od * od;
+        }
+    };
+    if (G == 1) {
+#pragma unroll 4
+        for (int t = tid; t < rpr * C; t += kKmvThreads) put(t, cluster_sum(t));
+    } else {
+        for (int t = tid; t < rpr * C; t += kKmvThreads) {
+            float sum = 0.0f;
+#pragma unroll 8
+            for (int g = 0; g < G; ++g) sum += __ldcg(slots + (int64_t)g * ROWS * C + t);
+            put(t, sum);
         }
     }
     const EpiParams& e = p.epi;
@@ -483,6 +492,8 @@ cudaError_t dispatch_kmv(const KmvParams& p, int D, int C, cudaStream_t st) {
     switch (C) {                                                          \
         case 1: return launch_kmv_inst<KERN, DD, 1>(p, st);               \
         case 4: return launch_kmv_inst<KERN, DD, 4>(p, st);               \
+        case 16: return launch_kmv_inst<KERN, DD, 16>(p, st);             \
+        case 32: return launch_kmv_inst<KERN, DD, 32>(p, st);             \
         default: return cudaErrorInvalidValue;                            \
     }
     switch (D) {

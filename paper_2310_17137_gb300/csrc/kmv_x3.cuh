@@ -1,5 +1,5 @@
-// FP32 kernel-matrix product for c > 4 right-hand sides: entries in FP32 on the
-// CUDA cores, the contraction with V on the tensor cores in split-precision form.
+// FP32 kernel-matrix product for c > 4 right-hand sides (from kX3MinEntries16 / 32
+// entries on; kmv_fp32.cuh below): entries in FP32 on the CUDA cores, the contraction with V on the tensor cores in split-precision form.
 //
 //   out[i,:] = base[i,:] + sgn * (s * sum_j phi(x_i, x_j) V[j,:] + noise V_i (diagonal))
 //
@@ -25,8 +25,9 @@
 // Measured time (GB300): n = 131,072, d = 3, c = 16, n^2 entries of Matern-5/2 19.1 ->
 // 12.3 ms; n = 65,536, d = 8, c = 32, 4096 columns of Matern-3/2 665 -> 302 us, at
 // 70 % of the issue slots and 59 % of the FMA pipe (tensor pipe 15 %).
-// Infinities and NaNs in V are taken out of the split, noted
-// per column and chunk, and added by the drain.
+// Infinities and NaNs in V are taken out of the split, noted per column and chunk, and
+// added by the drain to every row of the tile: a row whose kernel entry underflows to 0
+// gets the infinity too (the SIMT form: 0 times infinity, NaN).
 //
 // One persistent CTA per SM.  Work units are (row group, 128-column chunk) pairs in
 // group-major order, cut into equal contiguous ranges; a group has 128 R rows (R = 2:

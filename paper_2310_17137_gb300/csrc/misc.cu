@@ -29,10 +29,13 @@ double kernel_input_scale(int kernel) {
 // Measured on GB300: n = 100,003, d = 11, 1024 test points, 16 CTAs (cluster only)
 // 1102 us per ap_predict_mean call, with the groups 135 us; n = 20,600, d = 8, one
 // column, ap_residual 500 -> 377 us.
+// With 16 and 32 right-hand sides a group needs 64 columns per right-hand side: the sums
+// that pass through global memory grow with them (3000 x 3000, c = 32: 91 us with groups of
+// 75 columns, 80 us without).
 // Tensor-core form: one CTA per SM over equal ranges of (tile, 128-column chunk) units.
 KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
     constexpr int64_t kSms = 152, kMaxScratch = (int64_t)8 << 20;
-    const bool x3 = C >= kX3MinC;
+    const bool x3 = C >= kX3MinC && (double)(seg * nseg) * (double)ncols >= (C == 16 ? kX3MinEntries16 : kX3MinEntries32);
     const int64_t chunk = x3 ? kX3Chunk : kKmvTN;
     const double places = x3 ? kSms : 2.0 * kSms;
     const double instr = x3 ? D + 16.0 : D + C + 8.0, lds = x3 ? D / 4.0 : (D + C) / 4.0;
@@ -51,6 +54,7 @@ KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
         if (!best.rm || cost < best_cost) best = sp, best_cost = cost;
     }
     best.S = 1;
+    best.x3 = x3;
     if (x3) {
         best.ctas = (int)std::min<int64_t>(kSms, best.ntiles * ((ncols + chunk - 1) / chunk));
         best.G = 2;
@@ -63,8 +67,9 @@ KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
     auto groups = [&](int64_t want, int64_t min_cols) {
         return std::min<int64_t>((want + ctas - 1) / ctas, ncols / (best.S * min_cols));
     };
-    int64_t G = groups(64 * kSms, 512);
-    if (ctas < 4 * kSms) G = std::max(G, groups(8 * kSms, chunk));
+    const int64_t wide = C >= kX3MinC ? 64 * C : 0;
+    int64_t G = groups(64 * kSms, std::max<int64_t>(512, wide));
+    if (ctas < 4 * kSms) G = std::max(G, groups(8 * kSms, std::max(chunk, wide)));
     G = std::min<int64_t>(G, kMaxScratch / (best.ntiles * best.rows * C));
     best.G = (int)std::max<int64_t>(1, std::min<int64_t>(G, 1024));
     if (best.G > 1) {
@@ -75,7 +80,7 @@ KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
 }
 
 cudaError_t launch_kmv(int kernel, const KmvParams& p, int D, int C, cudaStream_t st) {
-    const bool x3 = C >= kX3MinC;
+    const bool x3 = p.x3;
     switch (kernel) {
         case AP_RBF: return x3 ? launch_x3_rbf(p, D, C, st) : launch_kmv_rbf(p, D, C, st);
         case AP_MATERN32: return x3 ? launch_x3_m32(p, D, C, st) : launch_kmv_m32(p, D, C, st);
