@@ -40,6 +40,7 @@ struct SolveState {
     double colnorm[AP_MAX_RHS];  // ||R_:,c||^2
     int nan_flag;                // a norm (or an input) was not finite
     int tc_err;                  // a bounded device wait ran out
+    double gout[AP_MAX_DIM + 4]; // sums of the gradient kernel
 };
 
 struct ap_ctx {
@@ -82,7 +83,7 @@ struct ap_ctx {
     bool groups_released = false;  // the next solve or residual asks for its area again
     int sol_tpc = 1, sol_maxj = 1;
     // always-present device scalars
-    double *norms = nullptr, *gout = nullptr, *gpart = nullptr;
+    double *norms = nullptr, *gpart = nullptr;
     SolveState* state = nullptr;
     // flags and tickets of `state` and the products are known to be zero: set when a call
     // has read clean flags, so that the next one need not clear them
@@ -1204,7 +1205,6 @@ ap_status ap_create(ap_ctx** out, const float* X_dev, int64_t n, int32_t d, cons
     if ((s = dalloc_t(ctx, &ctx->Xs_lo, (size_t)(n * ctx->D))) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->norms, (size_t)ctx->m)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->state, 1)) != AP_OK) return fail(s);
-    if ((s = dalloc_t(ctx, &ctx->gout, AP_MAX_DIM + 4)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->ticket, 4)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->sel, 1)) != AP_OK) return fail(s);
     if ((s = dalloc_t(ctx, &ctx->step, 1)) != AP_OK) return fail(s);
@@ -1380,14 +1380,13 @@ static ap_status grad_quadforms_impl(ap_ctx* ctx, const float* U, const float* V
     gp.err = &ctx->state->tc_err;
     gp.wait_cycles = ctx->o.wait_limit_cycles;
     gp.ticket = ctx->ticket + 1;
-    gp.out = ctx->gout;
+    gp.out = ctx->state->gout;
     AP_CK(launch_grad(ctx->kernel, gp, ctx->D, Cp, ctx->st));
     ++ctx->launches;
-    double raw[AP_MAX_DIM + 2] = {};
-    AP_CK(cudaMemcpyAsync(raw, ctx->gout, sizeof(double) * NA, cudaMemcpyDeviceToHost, ctx->st));
     SolveState now = {};
     AP_TRY(read_state(ctx, &now));
     if (now.tc_err) return AP_ERR_TIMEOUT;
+    const double* raw = now.gout;
     const double fac = ctx->kernel == AP_RBF ? 2.0 / 1.4426950408889634 : (ctx->kernel == AP_MATERN32 ? 1.0 : 1.0 / 3.0);
     for (int k = 0; k < ctx->d; ++k) out_host[k] = (double)ctx->s * fac * raw[k] / (double)ctx->ell[k];
     out_host[ctx->d] = raw[ctx->D];
@@ -1403,6 +1402,8 @@ ap_status ap_grad_quadforms(ap_ctx* ctx, const float* U_dev, const float* V_dev,
     const int Cp = pad_c(c);
     AP_TRY(ensure_solve(ctx, Cp));
     AP_TRY(enter(ctx));
+    if (c == Cp)  // (the kernel takes arrays of any float alignment)
+        return grad_quadforms_impl(ctx, U_dev, V_dev, Cp, alpha_host, c, out_host);
     AP_CK(launch_pad_copy(U_dev, ctx->n, c, ctx->Tmp, Cp, ctx->st));
     AP_CK(launch_pad_copy(V_dev, ctx->n, c, ctx->Bp, Cp, ctx->st));
     ctx->launches += 2;
@@ -1444,12 +1445,13 @@ ap_status ap_mll_grad(ap_ctx* ctx, const float* y_dev, int32_t n_probes, const f
     for (int k = 1; k < c; ++k) alpha[k] = 0.5 / (double)l;
     double g[AP_MAX_DIM + 2] = {};
     if ((s = grad_quadforms_impl(ctx, ctx->W, ctx->Tmp, Cp, alpha, c, g)) != AP_OK) return done(s);
-    if (launch_dot0(ctx->W, Cp, nullptr, 0, ctx->n, ctx->gpart, ctx->ticket + 2, ctx->gout, ctx->st) != cudaSuccess ||
-        launch_dot0(ctx->W, Cp, Bfull, c, ctx->n, ctx->gpart, ctx->ticket + 2, ctx->gout + 1, ctx->st) != cudaSuccess)
+    double* gout = ctx->state->gout;
+    if (launch_dot0(ctx->W, Cp, nullptr, 0, ctx->n, ctx->gpart, ctx->ticket + 2, gout, ctx->st) != cudaSuccess ||
+        launch_dot0(ctx->W, Cp, Bfull, c, ctx->n, ctx->gpart, ctx->ticket + 2, gout + 1, ctx->st) != cudaSuccess)
         return done(AP_ERR_CUDA);
     ctx->launches += 2;
     double dots[2] = {0.0, 0.0};
-    if (cudaMemcpyAsync(dots, ctx->gout, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->st) != cudaSuccess)
+    if (cudaMemcpyAsync(dots, gout, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->st) != cudaSuccess)
         return done(AP_ERR_CUDA);
     if ((s = leave(ctx)) != AP_OK) return done(s);
     const double usum = dots[0];

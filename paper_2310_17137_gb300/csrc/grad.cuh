@@ -25,8 +25,8 @@
 //   came out 2.8e-9 low at c = 32; now 0.3e-9, as with scalar multiply-adds).
 // What is left are 4 d multiply-add lanes (as packed pairs) and about 14 instructions
 // per visited entry.  Measured (GB300, n = 131,072, d = 8, c = 32, Matern-3/2): 47.0 ->
-// 14.3 ms for the n^2 forms, FMA pipe 68 % busy.  (With two stages 16.5 ms: the chunk's
-// copy, split and MMAs follow one another.)  Error of the doubles against 64 bits, relative
+// 14.35 ms for the n^2 forms, FMA pipe 68 % busy; n = 1024, d = 8, c = 4 a call 62 -> 45 us.
+// (With two stages 16.5 ms: the chunk's copy, split and MMAs follow one another.)  Error of the doubles against 64 bits, relative
 // to the forms of absolute values, n = 8192, root mean square over 40 inputs, scalar form
 // -> this one: RBF d = 8, c = 32 3.25e-9 -> 3.30e-9; Matern-3/2 d = 3, c = 16 6.07e-9 ->
 // 6.08e-9; Matern-5/2 d = 20, c = 32 3.47e-9 -> 3.49e-9: that of exp2, sqrt and the inputs.
@@ -237,15 +237,21 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
                     split_operand<C>(p, i, 8 * k8, true, vec,
                                      s_a + r * K::kPlaneA + ((row >> 3) * (K::KC / 8) + k8) * 128 + (row & 7) * 16,
                                      R * K::kPlaneA);
-                if (slot == 0 && first_chunk && i < n) {
-                    float s = 0.0f;
-                    for (int c = 0; c < C; ++c) s = fmaf(p.alpha[c] * __ldg(p.U + i * C + c), __ldg(p.V + i * C + c), s);
-                    diag += (double)s;
-                }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_a);
+            // (the MMAs need not wait for the diagonal)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int64_t i = g * K::kRows + 128 * r + row;
+                if (slot == 0 && first_chunk && i < n) {
+                    float s = 0.0f;
+#pragma unroll 8
+                    for (int c = 0; c < C; ++c) s = fmaf(p.alpha[c] * __ldg(p.U + i * C + c), __ldg(p.V + i * C + c), s);
+                    diag += (double)s;
+                }
+            }
         };
         const float2 m1 = make_float2(-1.0f, -1.0f);
         bool ok = true;
@@ -345,12 +351,32 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
             }
         }
         fold();
-        // warp sums in FP64
+        // Warp sums in FP64 by halving exchanges: lanes 16, 8, .. apart split the sums
+        // between them, NP - 1 additions a lane instead of five per sum (FP64 runs at 2
+        // results per clock per SM: 9 us of every call at D = 12 otherwise).
+        constexpr int NP = K::NA <= 8 ? 8 : K::NA <= 16 ? 16 : K::NA <= 32 ? 32 : 64;
+        double a[NP];
 #pragma unroll
-        for (int k = 0; k < K::NA; ++k) {
-            double v = k < D ? accd[k] : k == D ? accd[D] + diag : diag;
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) s_part[warp][k] = v;
+        for (int k = 0; k < NP; ++k) a[k] = k < D ? accd[k < D ? k : 0] : k == D ? accd[D] + diag : k == D + 1 ? diag : 0.0;
+#pragma unroll
+        for (int o = 16, w = NP / 2; o > 0; o >>= 1, w /= 2) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int k = 0; k < (w > 0 ? w : 1); ++k) {
+                if (w > 0) {
+                    const double keep = up ? a[k + w] : a[k];
+                    a[k] = keep + __shfl_xor_sync(0xffffffffu, up ? a[k] : a[k + w], o);
+                } else {
+                    a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+                }
+            }
+        }
+        // the lane's bits, 16 first, spell the index of what is left
+        constexpr int kPerLane = NP > 32 ? NP / 32 : 1, kRepeat = NP < 32 ? 32 / NP : 1;
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k) {
+            const int idx = lane / kRepeat * kPerLane + k;
+            if (lane % kRepeat == 0 && idx < K::NA) s_part[warp][idx] = a[k];
         }
     } else if (warp == K::kMmaWarp) {
         // ------------------------------------------------------------ MMA issuer
@@ -437,25 +463,26 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
     } else {
         // --------------------------------------- splitters of the chunk's [V | alpha U]
         const int ct = tid - K::kConvWarp * 32;
-        bool ok = true;
         int64_t g = g0, q = q0;
         int stage = 0;
         uint32_t sphase = 0;
-        for (int c = 0; c < total && ok; ++c) {
-            // the copy into this stage has landed, so the stage's last users are done
-            ok = __all_sync(0xffffffffu, mbar_wait(&bar_full[stage], sphase, &s_abort, p.err));
-            if (!ok) break;
+        for (int c = 0; c < total; ++c) {
+            // when the copy into this stage has landed the stage's last users are done (the
+            // first chunks find their stages unused)
+            auto landed = [&]() { return __all_sync(0xffffffffu, mbar_wait(&bar_full[stage], sphase, &s_abort, p.err)); };
+            if (c >= kStages && !landed()) break;
             uint8_t* st = s_stage + (size_t)stage * K::kStageBytes;
             const int cnt = (int)min((int64_t)kChunk, n - q * kChunk);
-            if (cnt < kChunk)
-                for (int t = cnt * D + ct; t < kChunk * D; t += 32 * kConvWarps)
-                    reinterpret_cast<float*>(st)[t] = reinterpret_cast<const float*>(st)[(cnt - 1) * D + t % D];
 #pragma unroll 2
             for (int t = ct; t < kChunk * (K::KC / 8); t += 32 * kConvWarps) {
                 const int j = t % kChunk, k8 = t / kChunk;  // (neighbouring lanes fill one core matrix)
                 split_operand<C>(p, q * kChunk + j, 8 * k8, false, vec,
                                  st + K::kXBytes + ((j >> 3) * (K::KC / 8) + k8) * 128 + (j & 7) * 16, K::kPlaneB);
             }
+            if (c < kStages && !landed()) break;
+            if (cnt < kChunk)
+                for (int t = cnt * D + ct; t < kChunk * D; t += 32 * kConvWarps)
+                    reinterpret_cast<float*>(st)[t] = reinterpret_cast<const float*>(st)[(cnt - 1) * D + t % D];
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar_ready[stage]);
@@ -495,9 +522,20 @@ __global__ void __launch_bounds__(Cfg<D, C>::kThreads, 1) grad_kernel(const Grad
     __syncthreads();
     if (s_last) {
         __threadfence();
+        // ranges of CTAs side by side, then the ranges in order
+        constexpr int NG = K::kXformWarps;
+        const int per = ((int)gridDim.x + NG - 1) / NG;
+        for (int t = tid; t < NG * K::NA; t += K::kThreads) {
+            const int g = t / K::NA, k = t % K::NA;
+            double acc = 0.0;
+#pragma unroll 10
+            for (int b = g * per; b < min((g + 1) * per, (int)gridDim.x); ++b) acc += __ldcg(p.part + (int64_t)b * K::NA + k);
+            s_part[g][k] = acc;
+        }
+        __syncthreads();
         for (int k = tid; k < K::NA; k += K::kThreads) {
             double acc = 0.0;
-            for (unsigned b = 0; b < gridDim.x; ++b) acc += __ldcg(p.part + (int64_t)b * K::NA + k);
+            for (int g = 0; g < NG; ++g) acc += s_part[g][k];
             p.out[k] = acc;
         }
         if (tid == 0) *p.ticket = 0u;
