@@ -517,17 +517,25 @@ def result_line(ap, p, args, world, ms_max, value, infos, statuses, launches, cl
 def roofline(p, args, t_launch: float, units: float, sm_max: float, sfu=(32.0, 16.0)) -> dict:
     """Roofline of the dominant kernel (the fused residual update of one AP step)."""
     if args.precision == "fp32":
-        flops_per_entry = 2 * p.c + 3 * p.d
+        # What runs on the FMA pipe: the distance, and the contraction (up to 4 right-hand
+        # sides) or the split of the entry into its BF16 parts (two multiply-adds; the
+        # contraction is six split products on the tensor cores then, reported beside it).
+        split = p.c > 4
+        flops_per_entry = 3 * p.d + (4 if split else 2 * p.c)
         achieved = units * flops_per_entry / t_launch / 1e12 if t_launch > 0 else None
         peak = NUM_SMS * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
-        return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+        line = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if achieved else None,
                 "traffic": traffic_from_profiles("kmv_fp32_update", args.workload, "fp32", units),
-                "kernel": "kmv_x3_kernel (fused residual update, one AP step)",
-                "per_unit": f"{flops_per_entry} FP32 flop per kernel entry (2c contraction, on the tensor cores "
-                            f"as six BF16 split products, + 3d distance)",
+                "kernel": f"{'kmv_x3_kernel' if split else 'kmv_fp32_kernel'} (fused residual update, one AP step)",
+                "per_unit": f"{flops_per_entry} FP32 flop per kernel entry on the FMA pipe (3d distance + "
+                            f"{'4 for the split into BF16 parts' if split else '2c contraction'})",
                 "peak_note": f"FP32 FMA pipe: {NUM_SMS} SMs x {FP32_LANES_PER_SM} lanes x 2 flop x "
                              f"{sm_max:.0f} MHz (derived from unit counts and max clock)"}
+        if split:
+            line["tensor_flops_per_entry"] = 6 * 2 * (16 if p.c <= 16 else 32)
+            line["tensor_tflops"] = units * line["tensor_flops_per_entry"] / t_launch / 1e12 if t_launch > 0 else None
+        return line
     # SFU operations per entry: exp2 for every kernel, sqrt for the Matern ones.
     # Peak: the measured per-clock rates of this GPU (ap_sfu_rates) at the
     # maximum SM clock; for the Matern mix (one of each per entry) the pipe
