@@ -44,12 +44,6 @@ __device__ __forceinline__ F2 add_f(F2 a, float b) {
     return fast_two_sum(s.h, s.l + a.l);
 }
 
-__device__ __forceinline__ F2 mul(F2 a, F2 b) {
-    F2 p = two_prod(a.h, b.h);
-    const float e = fmaf(a.h, b.l, fmaf(a.l, b.h, p.l));
-    return fast_two_sum(p.h, e);
-}
-
 __device__ __forceinline__ F2 mul_f(F2 a, float b) {
     F2 p = two_prod(a.h, b);
     return fast_two_sum(p.h, fmaf(a.l, b, p.l));
