@@ -13,18 +13,24 @@
 // Precision: an FP32 value has 24 significant bits, so P = phi is exactly
 // P_hi + P_mid + P_lo with three BF16 parts (8 bits each, cut off by masking); V is
 // split the same way with rounding.  The six products of weight above 2^-24
-// (hh, hm, mh, hl, mm, lh) go to three FP32 accumulators by weight (hh | hm + mh |
+// (hh, hm, mh, hl, mm, lh) go to FP32 accumulators by weight (hh | hm + mh |
 // hl + mm + lh); ml, lm and ll are below 2^-25 of the product.  The accumulators are
-// drained every 64 columns and summed in FP32 registers with rounding to nearest, so
-// the tensor cores' own accumulation (which cuts off) covers 4 steps of 16 only.
-// Measured against 64 bits, root mean square of the error relative to the result,
-// random signs in V: 1.4e-7 .. 2.1e-7 over d = 3 .. 20, n = 4096 .. 16,384 (SIMT form,
-// one chain of n additions: 3.3e-7 .. 8.9e-7); the cut-off leaves a mean error below
-// 1.1e-7 on sums of equal sign (drains every 128 columns: 1.7e-7 for 2 % less time,
-// every 32: 0.8e-7 for 8 % more).
+// drained every 64 columns and summed in FP32 registers with rounding to nearest.
+// The tensor cores cut their sums off towards zero: each step of 16 columns that is added
+// to a running sum takes about half a unit of that sum's last place, always in the same
+// sense.  So hh has an accumulator per step (two for the four steps where tensor memory or
+// the drain's time do not allow more: 32 columns, and D = 4, where the drain is not hidden)
+// and V's parts are rounded to nearest, so that neither the small sums nor the dropped
+// products have a preferred sign.
+// Measured against 64 bits, root mean square of the error relative to the result, random
+// signs in V, SIMT form -> this one: n = 16,384, d = 8, c = 16 Matern-3/2 8.8e-7 -> 2.2e-7;
+// n = 65,536, d = 3, c = 16 Matern-5/2 5.6e-7 here; what the error has in common with the
+// result (a factor on it): +5e-9 -> +3e-9 there, +2.9e-8 -> +2.9e-8 with V >= 0 (that of
+// exp2 and sqrt; -2.9e-8 and -1.9e-8 with one accumulator for hh and V's hi cut off, which
+// doubled the error of a training step's gradient).
 // Measured time (GB300): n = 131,072, d = 3, c = 16, n^2 entries of Matern-5/2 19.1 ->
-// 12.3 ms; n = 65,536, d = 8, c = 32, 4096 columns of Matern-3/2 665 -> 302 us, at
-// 70 % of the issue slots and 59 % of the FMA pipe (tensor pipe 15 %).
+// 12.4 ms; n = 65,536, d = 8, c = 32, 4096 columns of Matern-3/2 665 -> 306 us, at
+// 71 % of the issue slots and 61 % of the FMA pipe (tensor pipe 15 %).
 // Infinities and NaNs in V are taken out of the split, noted per column and chunk, and
 // added by the drain to every row of the tile: a row whose kernel entry underflows to 0
 // gets the infinity too (the SIMT form: 0 times infinity, NaN).
@@ -74,7 +80,10 @@ struct Cfg {
     static constexpr uint32_t kXBytes = kChunk * D * 4, kVBytes = kChunk * C * 4;
     static constexpr uint32_t kV3Bytes = 3u * C * kChunk * 2u;
     static constexpr uint32_t kStageBytes = kXBytes + kVBytes + kV3Bytes;
-    static constexpr uint32_t kAccCols = R * 3 * C;
+    static constexpr int kSteps = kChunk / kDrains / 16;      // steps of 16 columns between drains
+    static constexpr int kHh = C == 16 && D >= 8 ? kSteps : 2;  // accumulators of hi x hi
+    static constexpr uint32_t kTileCols = (kHh + 2) * C;      // hh_{kHh-1} .. hh_0 | hm + mh | hl + mm + lh
+    static constexpr uint32_t kAccCols = R * kTileCols;
     static constexpr int kBufs = (int)((512 - kAccCols) / kBufCols) < 8 ? (int)((512 - kAccCols) / kBufCols) : 8;
     static constexpr int kUnitCols = R == 2 ? 16 : 32;  // columns of a work item
     static constexpr int kItems = kChunk / kUnitCols;   // work items per chunk
@@ -91,7 +100,10 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&r)[4])
                  : "memory");
 }
 
-// x0, x1 >= 0 as three exact BF16 parts each, packed (x0 low half, x1 high half).
+// x0, x1 >= 0 as three exact BF16 parts each, packed (x0 low half, x1 high half): parts cut
+// off by masking.  (For D = 4 rounding them by conversions is faster, split3_nearest: the
+// masks' pipe is the busier one there, n = 40,000, c = 16 1230 : 1187 us; from D = 8 on it
+// takes 1 to 3 % longer.)
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
     constexpr uint32_t kTop = 0xFFFF0000u;
     const uint32_t b0 = __float_as_uint(x0), b1 = __float_as_uint(x1);
@@ -236,7 +248,10 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
                             for (int r = 0; r < R; ++r) kv[r][jj] = phi_fp32<KERN>(tp[r].x + tp[r].y);
                         }
 #pragma unroll
-                        for (int r = 0; r < R; ++r) split3(kv[r][0], kv[r][1], hi[r][w], mid[r][w], lo[r][w]);
+                        for (int r = 0; r < R; ++r) {
+                            if constexpr (D == 4) split3_nearest(kv[r][0], kv[r][1], hi[r][w], mid[r][w], lo[r][w]);
+                            else split3(kv[r][0], kv[r][1], hi[r][w], mid[r][w], lo[r][w]);
+                        }
                     }
                     if (sub == 0 && use > 0) {
                         ok = __all_sync(0xffffffffu, mbar_wait(&bar_free[buf], (use - 1) & 1u, &s_abort, p.err));
@@ -297,17 +312,24 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
                 tc_fence_after();
 #pragma unroll
                 for (int tt = 0; tt < K::kTpd; ++tt) {
-                    const uint32_t a = tmem + lane_base + (uint32_t)((tile0 + tt) * 3 * C);
+                    const uint32_t a = tmem + lane_base + (uint32_t)(tile0 + tt) * K::kTileCols;
 #pragma unroll
                     for (int k0 = 0; k0 < C; k0 += 8) {
-                        uint32_t w0[8], w1[8], w2[8];
-                        tmem_ld8(a + k0, w0);
-                        tmem_ld8(a + C + k0, w1);
-                        tmem_ld8(a + 2 * C + k0, w2);
-                        tmem_wait_ld();
+                        float t[8];
 #pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            acc[tt][k0 + k] += __uint_as_float(w0[k]) + (__uint_as_float(w1[k]) + __uint_as_float(w2[k]));
+                        for (int h = K::kHh; h >= 0; h -= 2) {  // the small sums, then hi x hi in pairs
+                            uint32_t w0[8], w1[8];
+                            tmem_ld8(a + h * C + k0, w0);
+                            tmem_ld8(a + (h + 1) * C + k0, w1);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) {
+                                const float v = __uint_as_float(w0[k]) + __uint_as_float(w1[k]);
+                                t[k] = h == K::kHh ? v : t[k] + v;
+                            }
+                        }
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) acc[tt][k0 + k] += t[k];
                     }
                 }
                 tc_fence_before();
@@ -505,11 +527,18 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
                         const uint32_t pa = tmem_p + kBufCols * (uint32_t)buf + 24u * (uint32_t)u;
-                        const uint32_t acc = tmem + (R == 2 ? (uint32_t)(u * 3 * C) : 0u);
+                        const uint32_t acc = tmem + (R == 2 ? (uint32_t)u * K::kTileCols : 0u) + (K::kHh - 1) * C;  // hh_0
                         const uint64_t b = dv + (uint64_t)((R == 2 ? it : 2 * it + u) * 16);
-                        mma_ts(acc, pa, b, i3, (!first || (R == 1 && u > 0)) ? 1u : 0u);  // hi x [hi; mid; lo]
-                        mma_ts(acc + C, pa + 8, b, i2, 1u);                               // mid x [hi; mid]
-                        mma_ts(acc + 2 * C, pa + 16, b, i1, 1u);                          // lo x hi
+                        const int step = R == 2 ? it % kPerDrain : 2 * (it % kPerDrain) + u, j = step % K::kHh;
+                        const uint32_t add = step > 0 ? 1u : 0u, add_hh = step >= K::kHh ? 1u : 0u;
+                        if (j == 0) {
+                            mma_ts(acc, pa, b, i3, add);  // hi x [hi; mid; lo]
+                        } else {
+                            mma_ts(acc - (uint32_t)(j * C), pa, b, i1, add_hh);                               // hi x hi
+                            mma_ts(acc + C, pa, b + (uint64_t)(C / 8 * (kChunk / 8) * 8), i2, add);  // hi x [mid; lo]
+                        }
+                        mma_ts(acc + C, pa + 8, b, i2, 1u);       // mid x [hi; mid]
+                        mma_ts(acc + 2 * C, pa + 16, b, i1, 1u);  // lo x hi
                     }
                     tc_commit(&bar_free[buf]);
                     if ((it + 1) % kPerDrain == 0) tc_commit(&bar_acc);
@@ -592,10 +621,9 @@ __global__ void __launch_bounds__(Cfg<D, C, R>::kThreads, 1) kmv_x3_kernel(const
                     atomicOr(&nf[k], flags);
                     s_any[c % kFlagRing] = 1;
                 }
-                // hi rounds towards zero (v may be the largest float), mid and lo to nearest
                 uint32_t w[3][4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) split3_rn(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
+                for (int j = 0; j < 4; ++j) split3_nearest(v[2 * j], v[2 * j + 1], w[0][j], w[1][j], w[2][j]);
 #pragma unroll
                 for (int pl = 0; pl < 3; ++pl) {
                     const int vr = pl * C + k;

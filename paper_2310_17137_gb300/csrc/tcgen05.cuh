@@ -210,28 +210,18 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// x0, x1 as BF16 parts: hi cut off, mid and lo rounded to nearest (what is dropped of
-// the products then has no preferred sign).
-__device__ __forceinline__ void split3_rn(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-    constexpr uint32_t kTop = 0xFFFF0000u;
-    const uint32_t b0 = __float_as_uint(x0), b1 = __float_as_uint(x1);
-    hi = __byte_perm(b0, b1, 0x7632);
-    const float r0 = x0 - __uint_as_float(b0 & kTop), r1 = x1 - __uint_as_float(b1 & kTop);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(mid) : "f"(r1), "f"(r0));
-    const float s0 = r0 - __uint_as_float(mid << 16), s1 = r1 - __uint_as_float(mid & kTop);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(s1), "f"(s0));
-}
-
-// The same with hi rounded to nearest too: mid then has no preferred sign either, so that
-// what the tensor cores cut off its products' sums does not lean towards zero with the
-// result.  (The largest floats keep a finite hi.)
+// x0, x1 as three BF16 parts, each rounded to nearest: no part has a preferred sign, so
+// neither what is dropped of the products nor what the tensor cores cut off the small
+// products' sums leans towards zero with the result.  (The largest floats keep a finite
+// hi.)
 __device__ __forceinline__ void split3_nearest(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
     constexpr uint32_t kTop = 0xFFFF0000u;
     asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(x1), "f"(x0));
-    const float r0 = x0 - __uint_as_float(hi << 16), r1 = x1 - __uint_as_float(hi & kTop);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(mid) : "f"(r1), "f"(r0));
-    const float s0 = r0 - __uint_as_float(mid << 16), s1 = r1 - __uint_as_float(mid & kTop);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(s1), "f"(s0));
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    const float2 r = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & kTop)), m1, make_float2(x0, x1));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(mid) : "f"(r.y), "f"(r.x));
+    const float2 s = __ffma2_rn(make_float2(__uint_as_float(mid << 16), __uint_as_float(mid & kTop)), m1, r);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(s.y), "f"(s.x));
 }
 
 // Shared-memory matrix descriptor, K-major, no swizzle: core matrices of 8 rows
