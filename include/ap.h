@@ -366,7 +366,9 @@ ap_status ap_phi_fp64_eval(int32_t kernel, const double* r2_host, int64_t count,
  * device footprint fits in the HBM budget; each admitted request runs its own
  * context (cache, Alg. 1 with one CUDA graph per epoch, posterior mean) on its
  * worker's stream, so requests overlap on the device.  Results are
- * deterministic: the same alone and in a mix. */
+ * deterministic, the same alone and in a mix, while the device can supply the
+ * reserved memory (a product whose optional work area the allocator refuses
+ * adds its sums in another order). */
 typedef struct ap_server ap_server;
 
 /* One request.  All host buffers are owned by the caller and must stay valid

@@ -160,7 +160,11 @@ constexpr int kX3MinC = 16;  // right-hand sides (padded) from which the tensor-
 // steps 2000 x 256 37 : 45, 2000 x 1000 71 : 73, 10,000 x 256 43 : 41, 16,000 x 1000 102 : 81
 // (all at d = 8, Matern-3/2).
 constexpr double kX3MinEntries16 = 1 << 24, kX3MinEntries32 = 2.5e6;
-constexpr int kX3MaxD2 = 16; // largest D whose two rows per thread fit the registers
+// Largest D with two rows per thread (beyond, their coordinates do not fit the registers).
+// One row : two, n = 32,768, Matern-3/2, c = 16, us: D = 4 890 : 808, 8 1143 : 1033, 12 1434 :
+// 1315, 16 1687 : 1518, although the two-row instances spill some registers; one row against
+// the SIMT form: D = 24 2305 : 2968, 32 3004 : 3517 (c = 32 2430 : 3937, 3130 : 4500).
+constexpr int kX3MaxD2 = 16;
 constexpr int kX3Chunk = 128;
 
 // FP32 SIMT kernel-matrix product with the AP epilogue (one per kernel family TU).

@@ -33,7 +33,7 @@ constexpr int kSms = 152;
 // FMAs instead of the library exp and sqrt.  FP64 arithmetic (2 results per clock per
 // SM) is all that bounds the K_II build, and comparisons, conversions and rounding count
 // as much as a multiply-add, so ranges are tested and integers taken on the bits
-// (GB300, 5 blocks of 4096, d = 8: 4.28 -> 3.23 ms).
+// (GB300, 5 blocks of 4096, d = 8: 4.28 -> 3.79 ms).
 //
 // exp(x), x <= 0: Tang's table-driven method (P. T. P. Tang, "Table-driven
 // implementation of the exponential function in IEEE floating-point
@@ -580,8 +580,10 @@ cudaError_t cache_factor_group(const CacheParams& cp, int64_t blk0, int g, doubl
     // column is updated in a launch of its own, and the diagonal tiles run on a second
     // stream beside the rest, which leaves them g SMs.  The rest takes about 10.5 us per
     // super-tile and SM; a share g / 152 of that is lost, which must stay below the chain.
-    // Measured (GB300, b = 4096): training step on 5 blocks 34.3 -> 31.2 ms, host solve on
-    // 13 blocks 59.8 -> 57.3 ms.
+    // Measured (GB300): training step on 5 blocks of 4096 34.3 -> 31.2 ms, host solve on 13
+    // blocks 59.8 -> 57.3 ms; ap_set_hyper, never ahead : by this rule : always, ms: 64 blocks
+    // of 256 1.11 : 1.07 : 1.09, 16 of 2048 12.5 : 10.9 : 10.9, 64 of 2048 34.3 : 33.8 : 37.0,
+    // 1 of 4096 12.8 : 11.3 : 11.3, 32 of 4096 90.1 : 88.8 : 92.3, 8 of 8192 144 : 137 : 137.
     auto ahead_of = [&](int k) {
         const int64_t rem = nt - k - 1, tiles = rem * rem / 4;
         return oz && oz->side && g <= kSms / 2 && tiles * g * g < 170000;

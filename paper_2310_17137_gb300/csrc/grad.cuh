@@ -74,6 +74,11 @@ constexpr int kStages = 4;
 constexpr int kConvWarps = 2;
 constexpr int kFold = 4;  // chunks between folds of the FP32 sums into FP64
 
+// Rows per thread, one : two (n = 32,768, Matern-3/2, us): D = 8 c = 16 1145 : 925, c = 32 1619 :
+// 1030, D = 12 1522 : 1343 and 1740 : 1461; the two-row instances spill 150 to 470 bytes all the
+// same.  Transform warps, 8 : 16: D = 12 c = 16 1421 : 1343, D = 16 1922 : 1828.  All of them
+// against the scalar form of one pass over n^2: D = 4 1702 : 640, 16 3752 : 1828, 24 5706 : 2591,
+// 32 8576 : 3326 (c = 16).
 template <int D, int C>
 struct Cfg {
     static constexpr int R = D <= 12 ? 2 : 1;                // rows per thread

@@ -17,7 +17,9 @@
 // squares of unnormalised differences (s + e)^2 = s^2 + e (2 s + e) and one
 // renormalisation of the sum spare a quarter of the distance.  Measured (GB300,
 // n = 16,384, d = 8, one column, RBF): 3.42 -> 2.61 ms for the n^2 entries,
-// the same results.
+// the same results.  A coordinate is kept twice, which takes up to 50 registers more (D = 32,
+// C = 32: one CTA per SM fewer); n = 8192, RBF, us: D = 24 c = 1 2162 -> 1499, c = 32 3903 ->
+// 3168; D = 32 c = 1 2519 -> 1961, c = 16 3072 -> 2999, c = 32 4569 -> 3913.
 #pragma once
 
 #include "dfloat.cuh"

@@ -10,8 +10,10 @@
 // low-precision form), posterior mean (Sec. 2), copy out -- so the work of
 // different requests overlaps on the device.  Every per-request computation is
 // deterministic (fixed-order reductions), so a result is the same alone and in
-// a mix.  The paper has no serving component; this is the deployment shape of
-// its solver.
+// a mix, as long as the device supplies what is reserved (a product whose
+// optional work area the allocator refuses adds its sums in another order).
+// The paper has no serving component; this is the deployment shape of its
+// solver.
 #include <math.h>
 #include <string.h>
 
