@@ -154,12 +154,12 @@ constexpr int kX3MinC = 16;  // right-hand sides (padded) from which the tensor-
 // Entries of a product from which the tensor-core form runs, 16 and 32 right-hand sides: it
 // has some 12 us more of start-up (tensor memory, splitting and draining the first chunk,
 // the hand-over of shared row groups), the SIMT form the slope of its FP32 contraction.
-// Measured (GB300, us per call or step, SIMT : tensor cores), 16: ap_residual 2048^2 50 : 55,
-// 3000^2 65 : 68, 4096^2 94 : 74; steps 8000 x 1000 48 : 55, 16,000 x 1000 59 : 66, 8192 x
-// 2048 76 : 77, 20,000 x 2048 108 : 92.  32: 1024^2 46 : 57, 2048^2 67 : 66, 4096^2 95 : 83;
-// steps 2000 x 256 37 : 45, 2000 x 1000 71 : 73, 10,000 x 256 43 : 41, 16,000 x 1000 102 : 81
-// (all at d = 8, Matern-3/2).
-constexpr double kX3MinEntries16 = 1 << 24, kX3MinEntries32 = 2.5e6;
+// Measured at d = 8, Matern-3/2 (GB300, us per ap_residual call R or step, SIMT : tensor
+// cores; rows x columns).  16: R 3000^2 60 : 69, 4096^2 68 : 75, 4500^2 73 : 80; 8000 x 1000
+// 46 : 52, 8000 x 2000 66 : 68, 6000 x 3000 82 : 81, 24,000 x 1000 75 : 67, 12,000 x 2000 79 :
+// 75.  32: R 2048^2 65 : 68, 2500^2 72 : 80, 3300^2 82 : 82, 3600^2 88 : 81; 6000 x 1000 58 : 64,
+// 8000 x 1000 67 : 65, 12,000 x 512 66 : 69, 16,000 x 512 73 : 57, 12,000 x 1000 83 : 67.
+constexpr double kX3MinEntries16 = 2.2e7, kX3MinEntries32 = 8e6;
 // Largest D with two rows per thread (beyond, their coordinates do not fit the registers).
 // One row : two, n = 32,768, Matern-3/2, c = 16, us: D = 4 890 : 808, 8 1143 : 1033, 12 1434 :
 // 1315, 16 1687 : 1518, although the two-row instances spill some registers; one row against

@@ -20,7 +20,8 @@ double kernel_input_scale(int kernel) {
 // entry fall as 1 / rm), but a tile of 128 rm rows may be mostly padding (a segment of
 // 600 rows is 60 % of two 512-row tiles) and leaves fewer tiles.  The modelled issue
 // slots per useful entry, times the shortfall of work when the whole product cannot
-// fill the chip, decide.
+// fill the chip, decide (2894 x 2894, d = 6, 16 columns: 96 CTAs of two rows a thread 67 us
+// a call, 184 of one 59).
 //
 // Columns, SIMT form: S splits inside a cluster until 4 CTAs per SM exist, then G groups
 // through global memory: enough of them for about 8 waves of CTAs while every CTA keeps
@@ -39,6 +40,7 @@ KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
     const int64_t chunk = x3 ? kX3Chunk : kKmvTN;
     const double places = x3 ? kSms : 2.0 * kSms;
     const double instr = x3 ? D + 16.0 : D + C + 8.0, lds = x3 ? D / 4.0 : (D + C) / 4.0;
+    const int64_t wide = C >= kX3MinC ? 64 * C : 0;  // columns of a group
     KmvSplit best = {};
     double best_cost = 0.0;
     for (int rm = x3 ? (D <= kX3MaxD2 ? 2 : 1) : rows_per_thread(D, C); rm >= 1; rm /= 2) {
@@ -48,7 +50,10 @@ KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
         sp.tps = (seg + sp.rows - 1) / sp.rows;
         sp.ntiles = nseg * sp.tps;
         const double pad = (double)(sp.tps * sp.rows) / (double)seg;
-        const double units = (double)sp.ntiles * (double)((ncols + chunk - 1) / chunk);
+        // (many right-hand sides in the SIMT form: only as many column ranges as it is cut into)
+        int64_t ranges = (ncols + chunk - 1) / chunk;
+        if (!x3 && C >= kX3MinC) ranges = std::min(ranges, kMaxSplit * std::max<int64_t>(1, ncols / (kMaxSplit * wide)));
+        const double units = (double)sp.ntiles * (double)ranges;
         const double idle = units < places ? places / units : 1.0;
         const double cost = pad * idle * (instr + lds / rm);
         if (!best.rm || cost < best_cost) best = sp, best_cost = cost;
@@ -67,7 +72,6 @@ KmvSplit kmv_split(int D, int C, int64_t seg, int64_t nseg, int64_t ncols) {
     auto groups = [&](int64_t want, int64_t min_cols) {
         return std::min<int64_t>((want + ctas - 1) / ctas, ncols / (best.S * min_cols));
     };
-    const int64_t wide = C >= kX3MinC ? 64 * C : 0;
     int64_t G = groups(64 * kSms, std::max<int64_t>(512, wide));
     if (ctas < 4 * kSms) G = std::max(G, groups(8 * kSms, std::max(chunk, wide)));
     G = std::min<int64_t>(G, kMaxScratch / (best.ntiles * best.rows * C));
